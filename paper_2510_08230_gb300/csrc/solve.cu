@@ -2,7 +2,7 @@
 // SpMV layout, FP64 iterative refinement around FP32 / BF16-stored inner
 // solves) and the host-side helpers of the multi-kernel engine
 // (solve_engine.cuh).
-#include "solve_engine.cuh"
+#include "gridcg.cuh"
 
 namespace gk {
 
@@ -236,6 +236,11 @@ gk_status read_hdr(SolverCache* C, cudaStream_t s) {
     return GK_OK;
 }
 
+std::mutex& grid_cg_mutex() {
+    static std::mutex mu;
+    return mu;
+}
+
 gk_status clear_halt(SolverCache* C, cudaStream_t s) {
     KState* st = (KState*)C->state.ptr;
     GK_CUDA(cudaMemcpyAsync(&st->halt, C->hzero, sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -287,8 +292,14 @@ static gk_status solve_plain(gk_matrix A, const void* b, void* x, const gk_solve
     gk_matrix M = nullptr;
     GK_TRY(solve_matrix(A, s, &M));
     M->wait_ns = A->wait_ns;
-    GK_TRY((solve_mk<V, T>(M, (const T*)b, (T*)x, o->method, (int)o->precond, o->block_size,
-                           o->tol, o->max_iters, m, s, out, false)));
+    gk_status st = GK_ERR_UNSUPPORTED;
+    if (o->engine == 0 && grid_cg_admits(M, o->method, (int)o->precond))
+        st = solve_grid_cg<V, T>(M, (const T*)b, (T*)x, (int)o->precond, o->tol, o->max_iters, s,
+                                 out, false);
+    if (st == GK_ERR_UNSUPPORTED)
+        st = solve_mk<V, T>(M, (const T*)b, (T*)x, o->method, (int)o->precond, o->block_size,
+                            o->tol, o->max_iters, m, s, out, false);
+    GK_TRY(st);
     out->layout = M->fmt;
     out->slice = M->fmt == GK_SELLP ? M->S : 0;
     return GK_OK;
@@ -406,15 +417,19 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         const int pk = (int)o->precond;
         const int32_t bsz = o->block_size;
         const int32_t left = o->max_iters - total_inner;
-        if (L->dtype == GK_F32)
-            GK_TRY((solve_mk<float, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left, m, s,
-                                           &io, true)));
-        else if (L->dtype == GK_F16)
-            GK_TRY((solve_mk<__half, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left, m, s,
-                                            &io, true)));
-        else
-            GK_TRY((solve_mk<__nv_bfloat16, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left,
-                                                   m, s, &io, true)));
+        auto inner_solve = [&](auto vt) -> gk_status {
+            using V = decltype(vt);
+            if (o->engine == 0 && grid_cg_admits(L, o->method, pk)) {
+                const gk_status g = solve_grid_cg<V, float>(L, r32, d32, pk, inner_tol, left, s,
+                                                            &io, true);
+                if (g != GK_ERR_UNSUPPORTED) return g;
+            }
+            return solve_mk<V, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left, m, s, &io,
+                                      true);
+        };
+        GK_TRY(L->dtype == GK_F32   ? inner_solve(float())
+               : L->dtype == GK_F16 ? inner_solve(__half())
+                                    : inner_solve(__nv_bfloat16()));
         total_inner += io.iters;
         restarts += io.restarts;
         last_rec = io.rec;
