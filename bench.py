@@ -101,7 +101,7 @@ def build_items(gk, W, dtypes=("f64", "f32")):
     return items, lap, pl
 
 
-KERNEL_NAMES = {0: "k_csr_vector", 1: "k_csr_rowtile", 2: "k_csr_merge_reg", 3: "k_ell",
+KERNEL_NAMES = {0: "k_csr_vector", 1: "k_csr_rowtile", 2: "k_csr_seg", 3: "k_ell",
                 4: "k_sellp", 5: "k_coo_warp", 6: "k_csr_warptile"}
 
 
@@ -662,7 +662,7 @@ def profile_case(name, dtype):
     """One small case per kernel family for `ncu` captures: inputs larger
     than L2 (129 MB) but a few hundred MB on the device, three launches of
     the kernel after the matrix is built.
-      merge    CSR merge path, Zipf(1.8) power-law n=2^21 (~33M nnz)
+      merge    CSR segmented kernel, Zipf(1.8) power-law n=2^21 (~33M nnz)
       coo      COO of the same power-law matrix
       rowtile  CSR row tiles, 3D 7-point Laplacian 128^3 (14.6M nnz)
       warptile CSR warp tiles, the same Laplacian

@@ -122,7 +122,7 @@ typedef struct {
     int64_t stored;        /* entries held in col/values incl. padding */
     int64_t device_bytes;  /* bytes of the format arrays on the device */
     int32_t spmv_kernel;   /* SpMV kernel apply uses: 0 CSR vector, 1 CSR row-tile,
-                              2 CSR merge-path, 3 ELL, 4 SELL-P, 5 COO,
+                              2 CSR segmented, 3 ELL, 4 SELL-P, 5 COO,
                               6 CSR warp-tile */
     int32_t spmv_launches; /* kernel launches per apply */
     int32_t device_error;  /* nonzero if a kernel on this matrix gave up a
@@ -422,8 +422,8 @@ gk_status gk_triangular_solve(gk_matrix A, int upper, int unit_diagonal, const v
  * not see foreign allocations, or code in a loop where an allocation,
  * which can synchronise the device, is not allowed.
  *
- * It runs the merge-path kernels that gk_apply uses for skewed CSR
- * matrices, with the per-block carry scratch held in a fixed file-scope
+ * It runs a merge-path kernel that needs no plan of the matrix, with the
+ * per-block carry scratch held in a fixed file-scope
  * device array of 768 KB that every GPU loading this library keeps until
  * the process exits.  No cudaMalloc, cudaFree or allocating library call
  * is made.  The first call on each device looks up the array's device

@@ -146,18 +146,24 @@ struct DevBuf {
     gk_status ensure(size_t want);
     void release();
 };
+// Scratch freed at the end of its scope.
+struct TmpBuf : DevBuf {
+    ~TmpBuf() { release(); }
+};
 
 // ------------------------------------------------------------------ matrix
 // CSR launch plan.  Row tiles: tile c covers the rows starting in nonzero
 // chunk c; tile_desc[c] = {first row, end row, aligned first nonzero,
-// staged entries}, staged entries <= tile_cap.  Merge path: block_row[b] =
-// first row of merge block b (n_blocks + 1 entries).
+// staged entries}, staged entries <= tile_cap.  Segmented kernel: units of
+// 256 nonzeros; unit_row[u] = the first nonempty row that ends after 256 u
+// (units + 1 entries).  When rows are empty, row_end / row_id list the
+// others' ends and indices and empty_rows the empty ones.
 constexpr int WT_WARPS = 8;  // warps per block of the warp-tile kernel (CSR kind 3)
 constexpr int WT_SMEM_CAP = 208 * 1024;  // largest ring of one warp-tile block (the
                                          // epilogues' static shared memory fits beside it)
 
 struct CsrPlan {
-    int kind = 0;            // 0 vector (G lanes / row), 1 row-tile, 2 merge, 3 warp-tile
+    int kind = 0;            // 0 vector (G lanes / row), 1 row-tile, 2 segmented, 3 warp-tile
     int lanes = 1;           // vector kernel lanes per row
     int32_t ntiles = 0;
     int32_t chunk = 0;       // nnz per chunk used to cut tiles
@@ -167,12 +173,12 @@ struct CsrPlan {
                              // warp-tile: stages per warp
     int4* tile_desc = nullptr;
     int32_t wt_rpl = 2;      // warp-tile: rows per lane (tiles of 32 * wt_rpl rows)
-    int32_t merge_blocks = 0;
-    int32_t merge_e = 8;     // merge-path items per lane (4, 6 or 8)
-    int32_t merge_warp = 2;  // merge units: 1 one warp (32*E items, operands staged in
-                             // shared memory), 2 one warp (operands in registers),
-                             // 0 one block (256*E items)
-    int32_t* block_row = nullptr;
+    int32_t units = 0;
+    int32_t* unit_row = nullptr;
+    int32_t* row_end = nullptr;
+    int32_t* row_id = nullptr;
+    int32_t* empty_rows = nullptr;
+    int32_t n_empty = 0;
     int32_t* err = nullptr;  // device word set by a kernel whose bounded wait ran out
 };
 
@@ -249,6 +255,7 @@ struct gk_matrix_s {
     gk_dtype dtype = GK_F64;
     int32_t max_row = 0;
     double mean_row = 0.0;
+    int32_t empty_rows_known = -1;  // number of empty rows, -1: not counted
     // CSR
     int32_t* row_ptr = nullptr;
     int32_t* col = nullptr;

@@ -14,7 +14,7 @@
 
 #include <shared_mutex>
 
-#include "prims.cuh"
+#include "spmv.cuh"
 
 namespace gk {
 
@@ -113,15 +113,17 @@ __global__ void k_scan_blocksums(int64_t* __restrict__ bsum, int64_t nb) {
 // ---------------------------------------------------------------- kernels
 
 // Validation of a CSR copy.  err bits: 1 row_ptr[0] != 0, 2 decreasing,
-// 4 row_ptr[n] != nnz, 8 column out of range.  Also max row length.
+// 4 row_ptr[n] != nnz, 8 column out of range.  Also the longest row and the
+// number of empty rows.
 __global__ void k_validate_rowptr(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
-                                  unsigned int* err, int32_t* max_row) {
-    int32_t local_max = 0;
+                                  unsigned int* err, int32_t* max_row, int32_t* n_empty) {
+    int32_t local_max = 0, local_empty = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t a = rp[i], b = rp[i + 1];
         if (b < a) atomicOr(err, 2u);
         else local_max = max(local_max, b - a);
+        local_empty += b == a;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (rp[0] != 0) atomicOr(err, 1u);
@@ -130,6 +132,8 @@ __global__ void k_validate_rowptr(int32_t n, int64_t nnz, const int32_t* __restr
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
     if ((threadIdx.x & 31) == 0 && local_max > 0) atomicMax(max_row, local_max);
+    local_empty = __reduce_add_sync(0xffffffffu, local_empty);
+    if ((threadIdx.x & 31) == 0 && local_empty > 0) atomicAdd(n_empty, local_empty);
 }
 
 __global__ void k_validate_cols(int64_t nnz, int32_t ncols, const int32_t* __restrict__ ci,
@@ -468,21 +472,43 @@ __global__ void k_tile_desc(int32_t n, const int32_t* __restrict__ rp, int32_t c
     }
 }
 
-// Merge plan: block b starts at path item b * items; its first row is the
-// number of rows whose end item lies before that point.
-__global__ void k_merge_rows(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
-                             int32_t items, int32_t nblocks, int32_t* __restrict__ mrow) {
-    const int64_t N = (int64_t)n + nnz;
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b <= nblocks;
-         b += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t d = min(b * (int64_t)items, N);
-        int32_t lo = 0, hi = n;
+// Segmented plan: unit u holds the nonzeros from 256 u on; its first row is
+// the first of the m listed rows that ends after that point.
+__global__ void k_unit_rows(int32_t m, const int32_t* __restrict__ row_end, int32_t nunits,
+                            int32_t* __restrict__ unit_row) {
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u <= nunits;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = u * SEG_UNIT;
+        int32_t lo = 0, hi = m;
         while (lo < hi) {
             const int32_t mid = lo + ((hi - lo) >> 1);
-            if ((int64_t)rp[mid + 1] + mid + 1 > d) hi = mid;
+            if ((int64_t)row_end[mid] > k) hi = mid;
             else lo = mid + 1;
         }
-        mrow[b] = lo;
+        unit_row[u] = lo;
+    }
+}
+
+__global__ void k_nonempty_flags(int32_t n, const int32_t* __restrict__ rp,
+                                 int32_t* __restrict__ flag) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        flag[i] = rp[i + 1] > rp[i];
+}
+
+// rank[i]: nonempty rows before row i
+__global__ void k_split_rows(int32_t n, const int32_t* __restrict__ rp,
+                             const int32_t* __restrict__ rank, int32_t* __restrict__ row_end,
+                             int32_t* __restrict__ row_id, int32_t* __restrict__ empty) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = rp[i + 1], q = rank[i];
+        if (e > rp[i]) {
+            row_end[q] = e;
+            row_id[q] = (int32_t)i;
+        } else {
+            empty[i - q] = (int32_t)i;
+        }
     }
 }
 
@@ -526,7 +552,8 @@ static void free_arrays(gk_matrix A) {
     dfree(A->slice_len);
     dfree(A->slice_set);
     dfree(A->plan.tile_desc);
-    dfree(A->plan.block_row);
+    for (int32_t* q : {A->plan.unit_row, A->plan.row_end, A->plan.row_id, A->plan.empty_rows})
+        dfree(q);
     dfree(A->plan.err);
     dfree(A->dinv);
     dfree(A->binv);
@@ -542,8 +569,7 @@ static void free_arrays(gk_matrix A) {
     A->val = nullptr;
     A->slice_len = nullptr;
     A->slice_set = nullptr;
-    A->plan.tile_desc = nullptr;
-    A->plan.block_row = A->plan.err = nullptr;
+    A->plan = CsrPlan();
     A->dinv = nullptr;
 }
 
@@ -604,11 +630,11 @@ static gk_status build_coo_view(gk_matrix A, cudaStream_t s) {
     return GK_OK;
 }
 
-// CSR launch plan: row tiles when rows are short, merge path otherwise.
+// CSR launch plan: row tiles when rows are short, the segmented kernel otherwise.
 gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
     CsrPlan& P = A->plan;
     dfree(P.tile_desc);
-    dfree(P.block_row);
+    for (int32_t* q : {P.unit_row, P.row_end, P.row_id, P.empty_rows}) dfree(q);
     dfree(P.err);
     P = CsrPlan();
     GK_CUDA(dmalloc_t(&P.err, 4));
@@ -671,25 +697,32 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
                                                        P.tile_desc);
         GK_CUDA(cudaGetLastError());
     } else if (kind == 2) {
-        // Merge-path units: 32*E items per warp.  Default: operands in
-        // registers (k_csr_merge_reg), E = 8 -- measured fastest on the 4M-row
-        // Zipf(1.8) matrix (FP64 424 us; E = 4, 6, 12, 16 and the kernel that
-        // stages operands in shared memory were slower).  GK_MERGE_E and
-        // GK_MERGE_UNIT (reg | warp | block) select the other instances.
-        int E = 8;
-        if (const char* e = getenv("GK_MERGE_E")) E = atoi(e);
-        if (E != 4 && E != 6 && E != 8) E = 8;
-        P.merge_warp = 2;
-        if (const char* w = getenv("GK_MERGE_UNIT"))
-            P.merge_warp = !strcmp(w, "block") ? 0 : !strcmp(w, "warp") ? 1 : 2;
-        P.merge_e = E;
-        const int64_t items = (P.merge_warp ? 32 : 256) * (int64_t)E;  // path items per unit
-        const int64_t N = (int64_t)A->n + A->nnz;
-        P.merge_blocks = (int32_t)std::max<int64_t>(1, (N + items - 1) / items);
-        GK_CUDA(dmalloc_t(&P.block_row, (size_t)P.merge_blocks + 1));
-        k_merge_rows<<<grid_for(P.merge_blocks + 1), 256, 0, s>>>(A->n, A->nnz, A->row_ptr,
-                                                                  (int32_t)items, P.merge_blocks,
-                                                                  P.block_row);
+        // units of SEG_UNIT nonzeros over the nonempty rows
+        P.units = (int32_t)((A->nnz + SEG_UNIT - 1) / SEG_UNIT);
+        TmpBuf flag, rank, tmp;
+        int32_t m = A->n;  // nonempty rows
+        if (A->empty_rows_known != 0) {
+            GK_TRY(flag.ensure(4 * (size_t)A->n));
+            GK_TRY(rank.ensure(4 * ((size_t)A->n + 1)));
+            int32_t* dflag = static_cast<int32_t*>(flag.ptr);
+            int32_t* drank = static_cast<int32_t*>(rank.ptr);
+            k_nonempty_flags<<<grid_for(A->n), 256, 0, s>>>(A->n, A->row_ptr, dflag);
+            GK_TRY(scan_exclusive<int32_t, int32_t>(dflag, drank, A->n, tmp, s));
+            GK_CUDA(cudaMemcpyAsync(&m, drank + A->n, 4, cudaMemcpyDeviceToHost, s));
+            GK_CUDA(cudaStreamSynchronize(s));
+            P.n_empty = A->n - m;
+            if (P.n_empty) {
+                GK_CUDA(dmalloc_t(&P.row_end, (size_t)std::max(m, 1)));
+                GK_CUDA(dmalloc_t(&P.row_id, (size_t)std::max(m, 1)));
+                GK_CUDA(dmalloc_t(&P.empty_rows, (size_t)P.n_empty));
+                k_split_rows<<<grid_for(A->n), 256, 0, s>>>(A->n, A->row_ptr, drank, P.row_end,
+                                                            P.row_id, P.empty_rows);
+                GK_CUDA(cudaStreamSynchronize(s));  // the scratch goes
+            }
+        }
+        GK_CUDA(dmalloc_t(&P.unit_row, (size_t)P.units + 1));
+        k_unit_rows<<<grid_for(P.units + 1), 256, 0, s>>>(
+            m, P.row_end ? P.row_end : A->row_ptr + 1, P.units, P.unit_row);
         GK_CUDA(cudaGetLastError());
     }
     return GK_OK;
@@ -703,16 +736,18 @@ static gk_status finish_csr(gk_matrix A, cudaStream_t s) {
     int32_t* dmax = reinterpret_cast<int32_t*>(derr + 1);
     GK_CUDA(cudaMemsetAsync(flags.ptr, 0, 16, s));
     if (A->n > 0)
-        k_validate_rowptr<<<grid_for(A->n), 256, 0, s>>>(A->n, A->nnz, A->row_ptr, derr, dmax);
+        k_validate_rowptr<<<grid_for(A->n), 256, 0, s>>>(A->n, A->nnz, A->row_ptr, derr, dmax,
+                                                         dmax + 1);
     if (A->nnz > 0)
         k_validate_cols<<<grid_for(A->nnz), 256, 0, s>>>(A->nnz, A->ncols, A->col, derr);
     GK_CUDA(cudaGetLastError());
-    unsigned int h[2] = {0, 0};
-    GK_CUDA(cudaMemcpyAsync(h, flags.ptr, 8, cudaMemcpyDeviceToHost, s));
+    unsigned int h[3] = {0, 0, 0};
+    GK_CUDA(cudaMemcpyAsync(h, flags.ptr, 12, cudaMemcpyDeviceToHost, s));
     GK_CUDA(cudaStreamSynchronize(s));
     flags.release();
     if (h[0]) return GK_ERR_INVALID;
     A->max_row = (int32_t)h[1];
+    A->empty_rows_known = (int32_t)h[2];
     A->mean_row = A->n ? (double)A->nnz / A->n : 0.0;
     GK_TRY(build_csr_plan(A, s));
     GK_CUDA(cudaStreamSynchronize(s));
@@ -973,6 +1008,7 @@ gk_status gk_matrix_convert(gk_matrix A, gk_format fmt, gk_dtype dtype, int32_t 
     B->fmt = fmt;
     B->dtype = dtype;
     B->max_row = A->max_row;
+    B->empty_rows_known = A->empty_rows_known;
     B->mean_row = A->n ? (double)A->nnz / A->n : 0.0;
     const int64_t n = A->n;
     gk_status st = GK_OK;
@@ -1071,7 +1107,7 @@ gk_status gk_matrix_describe(gk_matrix A, gk_matrix_desc* d) {
             d->device_error |= 2 << k;
     }
     d->spmv_launches = A->coo ? (A->n_empty ? 3 : 2)
-                       : (A->fmt == GK_CSR && A->plan.kind == 2) ? 2 : 1;
+                       : (A->fmt == GK_CSR && A->plan.kind == 2) ? (A->plan.n_empty ? 3 : 2) : 1;
     d->solve_format = A->fmt != GK_CSR ? (int32_t)A->fmt
                       : !A->solve_fmt_tuned ? -1
                       : A->solve_fmt ? (int32_t)A->solve_fmt->fmt : (int32_t)GK_CSR;

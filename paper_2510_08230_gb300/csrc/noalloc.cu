@@ -5,8 +5,8 @@
 // Some callers cannot call cudaMalloc: their device memory belongs to a
 // framework's pool allocator that must not see foreign allocations, or
 // they run in a loop where an allocation (which can synchronise the
-// device) is not allowed.  gk_spmv_csr_f64_noalloc serves them: it runs the
-// same merge-path kernels as gk_apply, with the per-block carry scratch
+// device) is not allowed.  gk_spmv_csr_f64_noalloc serves them: it runs
+// a merge-path kernel that needs no plan, with the per-block carry scratch
 // held in the file-scope device array below instead of a cudaMalloc'd
 // buffer.  Every GPU that loads this library holds the array (768 KB)
 // until the process exits.
@@ -70,9 +70,9 @@ extern "C" gk_status gk_spmv_csr_f64_noalloc(int32_t n, int32_t ncols, int64_t n
     double* cval = reinterpret_cast<double*>(static_cast<char*>(scratch) + NA_MAX_BLOCKS * 4);
     constexpr size_t smem = merge_smem_bytes<E, double, double>();
     k_csr_merge<E, double, double><<<(unsigned)nb, 256, smem, s>>>(
-        n, nnz, row_ptr, col_idx, values, b, epi, nullptr, crow, cval);
+        n, nnz, row_ptr, col_idx, values, b, epi, crow, cval);
     const unsigned fg = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nb + 255) / 256, 4096));
-    k_csr_merge_fixup<double><<<fg, 256, 0, s>>>((int32_t)nb, crow, cval, x, alpha, mode);
+    k_carry_fixup<double><<<fg, 256, 0, s>>>((int32_t)nb, crow, cval, x, alpha, mode);
     GK_CUDA(cudaGetLastError());
     return GK_OK;
 }

@@ -1,4 +1,4 @@
-// spmv.cuh - SpMV kernels (CSR row-tile, CSR merge-path, CSR vector, ELL,
+// spmv.cuh - SpMV kernels (CSR row-tile, CSR segmented, CSR vector, ELL,
 // SELL-P) with fused epilogues.
 //
 // A matrix LinOp's apply is an SpMV (Section 4.2); the advanced form adds
@@ -15,7 +15,7 @@
 // close to the rate at which HBM delivers FP64 nonzeros (12 B each).  The
 // kernels therefore spend one FMA per stored nonzero, keep warps converged
 // in the FMA loops, and reduce a row within one thread (row-tile, ELL,
-// SELL-P) or with carries between threads (merge-path); no FP64 shuffle
+// SELL-P) or with carries between threads (segmented); no FP64 shuffle
 // trees on the per-row path.  Loads that feed the FMAs are issued in
 // batches of 8 before the first FMA so that their latencies overlap.
 #pragma once
@@ -389,15 +389,15 @@ constexpr size_t merge_smem_bytes() {
 // FMA per nonzero).  A row whose end lies in a thread's piece is finished
 // there, adding the carries of earlier threads of the block whose pieces
 // ended inside the same row.  The row open at the end of a block is handed
-// to k_csr_merge_fixup as (carry_row, carry_val).  block_row (n_blocks + 1
-// entries) gives each block's first row; when null the block finds it by
-// binary search.
+// to k_carry_fixup as (carry_row, carry_val).  A block finds its first row
+// by binary search (this kernel serves the entry point that may not
+// allocate, which keeps no plan).
 template <int E, typename V, typename T>
 __global__ void __launch_bounds__(256)
 k_csr_merge(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
             const int32_t* __restrict__ ci, const V* __restrict__ va,
-            const T* __restrict__ x, EpiStore<T> epi, const int32_t* __restrict__ block_row,
-            int32_t* __restrict__ carry_row, T* __restrict__ carry_val) {
+            const T* __restrict__ x, EpiStore<T> epi, int32_t* __restrict__ carry_row,
+            T* __restrict__ carry_val) {
     using Sh = MergeShape<E, V, T>;
     constexpr int TI = Sh::TI;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -411,18 +411,14 @@ k_csr_merge(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
     const int64_t d0 = (int64_t)blockIdx.x * TI;
     const int64_t d1 = min(d0 + TI, N);
     if (threadIdx.x < 2) {
-        if (block_row) {
-            s_bounds[threadIdx.x] = __ldg(block_row + blockIdx.x + threadIdx.x);
-        } else {
-            const int64_t d = threadIdx.x == 0 ? d0 : d1;
-            int32_t lo = 0, hi = n;  // rows whose end item lies before d
-            while (lo < hi) {
-                const int32_t mid = lo + ((hi - lo) >> 1);
-                if ((int64_t)__ldg(rp + mid + 1) + mid + 1 > d) hi = mid;
-                else lo = mid + 1;
-            }
-            s_bounds[threadIdx.x] = lo;
+        const int64_t d = threadIdx.x == 0 ? d0 : d1;
+        int32_t lo = 0, hi = n;  // rows whose end item lies before d
+        while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo) >> 1);
+            if ((int64_t)__ldg(rp + mid + 1) + mid + 1 > d) hi = mid;
+            else lo = mid + 1;
         }
+        s_bounds[threadIdx.x] = lo;
     }
     __syncthreads();
     const int32_t i0 = s_bounds[0], i1 = s_bounds[1];
@@ -520,262 +516,148 @@ k_csr_merge(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
     }
 }
 
-// Merge path with register operands (apply only): the same 32*E-item warp
-// units and lane pieces as k_csr_merge_warp, but a lane loads the values and
-// columns of its (at most E, contiguous) nonzeros straight from global
-// memory and gathers their x into registers; only the unit's row ends are
-// staged in shared memory (for the lane's binary search and the row ends it
-// meets).  The walk visits the lane's nonzero slots k = 0..E-1 in order and
-// closes every row that ends before slot k first, so each nonzero costs one
-// FMA on registers indexed at compile time.
-template <int E>
-struct MergeRegShape {
-    static constexpr int WI = 32 * E;
-    static constexpr size_t WARP_BYTES = align16((size_t)(WI + 1) * 4);
-    static constexpr size_t BYTES = 8 * WARP_BYTES;
-};
+// CSR kernel for skewed row lengths (apply only).  The nonzeros are cut into
+// units of 256 per warp, 8 consecutive ones per lane, whatever rows they
+// belong to, so long rows cost no more than short ones.  A lane loads its 8
+// columns and values with 32-byte accesses, gathers their x (8 in flight),
+// and walks them in order, one FMA each.  Where rows end is looked up, not
+// carried with every entry as in COO: the warp marks the last position of
+// each row that ends in its unit with the row's rank in the unit, and every
+// lane reads its 8 marks with one 16-byte access.  Sums of ended rows go to
+// shared memory and leave together, so that y is written (and for beta != 0
+// read) in row order.  A row begun in earlier lanes gets their part from a
+// segmented shuffle scan; the row open at the end of a unit goes to
+// k_carry_fixup.
+// Rows are the matrix's nonempty ones: row_end[i] is the end of the i-th
+// (row_ptr + 1 when no row is empty), row_id[i] its index (null: i);
+// k_empty_rows writes the others.  unit_row[u]: the first of them that ends
+// after 256 u.
+//
+// Bound: every x gather of a warp touches up to 32 different 128-byte lines,
+// one L1 wavefront each (a probe of nothing but 67M uniformly random 8-byte
+// gathers took 231 us).  The merge-path kernel this replaced read columns and
+// values lane by lane (0.75 wavefronts a nonzero more) and y inside the
+// divergent row ends.  4M-row Zipf(1.8) matrix, 67M nonzeros, us, before and
+// after: y = A x 422 / 316 in FP64, 335 / 265 in FP32; r = b - A x 554 / 355 and
+// 405 / 275.  Warps in flight decide: FP64 at 4 blocks per SM took 355 (64
+// registers), at 5 316 (51), at 6 333 with the values loaded after the gathers
+// are issued, which FP32 gains from (6 blocks: 265, 5: 277).
+constexpr int SEG_E = 8;             // nonzeros per lane
+constexpr int SEG_UNIT = 32 * SEG_E;
 
-template <int E, typename V, typename T>
-__global__ void __launch_bounds__(256)
-k_csr_merge_reg(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
-                const int32_t* __restrict__ ci, const V* __restrict__ va,
-                const T* __restrict__ x, EpiStore<T> epi, const int32_t* __restrict__ unit_row,
-                int64_t nunits, int32_t* __restrict__ carry_row, T* __restrict__ carry_val) {
-    constexpr int WI = MergeRegShape<E>::WI;
-    constexpr unsigned FULL = 0xffffffffu;
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t u = (int64_t)blockIdx.x * 8 + warp;
-    if (u >= nunits) return;  // the whole warp; no block barrier follows
-    int32_t* s_rowend = reinterpret_cast<int32_t*>(smem + (size_t)warp * MergeRegShape<E>::WARP_BYTES);
-    const int64_t N = (int64_t)n + nnz;
-    const int64_t d0 = u * WI;
-    const int64_t d1 = min(d0 + WI, N);
-    int32_t bnd = 0;
-    if (lane < 2) bnd = __ldg(unit_row + u + lane);
-    const int32_t i0 = __shfl_sync(FULL, bnd, 0), i1 = __shfl_sync(FULL, bnd, 1);
-    const int32_t nloc = min(i1 - i0 + 1, n - i0);  // staged row ends
-    for (int k = lane; k < nloc; k += 32) s_rowend[k] = __ldg(rp + i0 + k + 1);
-    __syncwarp();
-    // this lane's start on the path: row i, nonzero j
-    const int64_t dt = min(d0 + (int64_t)lane * E, d1);
-    const int64_t dend = min(dt + E, d1);
-    int32_t lo = 0, hi = max(0, nloc);
-    while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if ((int64_t)s_rowend[mid] + i0 + mid + 1 > dt) hi = mid;
-        else lo = mid + 1;
-    }
-    int32_t i = i0 + lo;
-    const int64_t j0 = dt - i;
-    // the lane's end on the path: row iend, nonzero jend (its nonzeros are [j0, jend))
-    lo = 0;
-    hi = max(0, nloc);
-    while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if ((int64_t)s_rowend[mid] + i0 + mid + 1 > dend) hi = mid;
-        else lo = mid + 1;
-    }
-    const int32_t iend = i0 + lo;
-    const int64_t jend = dend - iend;
-    const int cnt = (int)(jend - j0);  // nonzeros of this lane, 0..E
-    V v[E];
-    T xv[E];
-    {
-        int32_t c[E];
+// 8 consecutive entries, 32-byte accesses (not kept in L1)
+__device__ __forceinline__ void load8(const int32_t* p, int32_t (&v)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                   "=r"(v[6]), "=r"(v[7])
+                 : "l"(p));
+}
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                   "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+__device__ __forceinline__ void load8(const double* p, double (&v)[8]) {
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p));
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(v[4]), "=d"(v[5]), "=d"(v[6]), "=d"(v[7])
+                 : "l"(p + 4));
+}
+template <typename H>  // 16-bit types
+__device__ __forceinline__ void load8(const H* p, H (&v)[8]) {
+    struct alignas(16) Q { H e[8]; };
+    const Q q = *reinterpret_cast<const Q*>(p);
 #pragma unroll
-        for (int k = 0; k < E; ++k)
-            if (k < cnt) {
-                c[k] = __ldcs(ci + j0 + k);
-                v[k] = va[j0 + k];
-            }
-#pragma unroll
-        for (int k = 0; k < E; ++k)
-            if (k < cnt) xv[k] = __ldg(x + c[k]);
-    }
-    T acc = T(0);
-    int32_t head_row = -1;
-    T head_val = T(0);
-    int64_t rend = (i < n) ? (int64_t)s_rowend[i - i0] : 0;
-    // close the rows that end at nonzero position p (before its slot)
-    auto close_until = [&](int64_t p) {
-        while (i < iend && rend <= p) {
-            if (head_row < 0) {
-                head_row = i;
-                head_val = acc;
-            } else {
-                epi.row(i, acc, nullptr);
-            }
-            acc = T(0);
-            ++i;
-            rend = (i < n && i - i0 < nloc) ? (int64_t)s_rowend[i - i0] : 0;
-        }
-    };
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        if (k < cnt) {
-            close_until(j0 + k);
-            acc = fmadd(cvt<T>(v[k]), xv[k], acc);
-        }
-    }
-    close_until(jend);  // row ends after the last nonzero of the piece
-    // carries: as in k_csr_merge_warp
-    const bool valid = dt < d1;
-    const int32_t myrow = valid ? i : INT32_MAX;
-    const T sc = warp_seg_scan(myrow, acc);
-    const int32_t prow = __shfl_up_sync(FULL, myrow, 1);
-    const T psc = __shfl_up_sync(FULL, sc, 1);
-    const int32_t nrow = __shfl_down_sync(FULL, myrow, 1);
-    if (head_row >= 0) {
-        T vv = head_val;
-        if (lane > 0 && prow == head_row) vv = psc + vv;
-        epi.row(head_row, vv, nullptr);
-    }
-    if (valid && (lane == 31 || nrow == INT32_MAX)) {
-        carry_row[u] = (i < n) ? i : -1;
-        carry_val[u] = sc;
-    }
+    for (int k = 0; k < 8; ++k) v[k] = q.e[k];
 }
 
-// Shared-memory layout of the warp-level merge kernel, per warp (8 warps a
-// block): values, gathered x, row ends; every array on a 16-byte boundary.
-template <int E, typename V, typename T>
-struct MergeWarpShape {
-    static constexpr int WI = 32 * E;             // path items per warp
-    static constexpr int PADN = WI + WI / 8 + 8;  // padded entries
-    static constexpr size_t OFF_XV = align16((size_t)PADN * sizeof(V));
-    static constexpr size_t OFF_RE = align16(OFF_XV + (size_t)PADN * sizeof(T));
-    static constexpr size_t WARP_BYTES = align16(OFF_RE + (size_t)(WI + 1) * 4);
-    static constexpr size_t BYTES = 8 * WARP_BYTES;
-};
-
-// CSR merge-path kernel at warp granularity (apply only).  The path of n
-// row ends and nnz nonzeros is cut into units of 32*E items, one unit per
-// warp and E items per lane; the 8 warps of a block share nothing but the
-// block's shared memory, so the kernel has no block barrier and a warp
-// never waits for another.  A warp stages its row ends, values and the
-// gathered x values (E independent gathers per lane in flight), each lane
-// walks its piece (one FMA per nonzero), and the carries of lanes whose
-// pieces end inside a row are combined with a 5-level segmented shuffle
-// scan (a level's add runs only in warps where some run is that long).  The
-// row open at the end of a unit goes to k_csr_merge_fixup as (carry_row,
-// carry_val).  unit_row (nunits + 1 entries) gives each unit's first row;
-// when null the warp finds it by binary search.
-template <int E, typename V, typename T>
-__global__ void __launch_bounds__(256)
-k_csr_merge_warp(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
-                 const int32_t* __restrict__ ci, const V* __restrict__ va,
-                 const T* __restrict__ x, EpiStore<T> epi, const int32_t* __restrict__ unit_row,
-                 int64_t nunits, int32_t* __restrict__ carry_row, T* __restrict__ carry_val) {
-    using Sh = MergeWarpShape<E, V, T>;
-    constexpr int WI = Sh::WI;
+template <typename V, typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 5 : 6)
+k_csr_seg(int64_t nnz, int64_t nunits, const int32_t* __restrict__ row_end,
+          const int32_t* __restrict__ row_id, const int32_t* __restrict__ unit_row,
+          const int32_t* __restrict__ ci, const V* __restrict__ va, const T* __restrict__ x,
+          EpiStore<T> epi, int32_t* __restrict__ carry_row, T* __restrict__ carry_val) {
     constexpr unsigned FULL = 0xffffffffu;
-    extern __shared__ __align__(128) unsigned char smem[];
+    constexpr int E = SEG_E;
+    __shared__ __align__(16) int16_t s_mark[8][SEG_UNIT];  // row ending here, or -1
+    __shared__ T s_sum[8][SEG_UNIT];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t u = (int64_t)blockIdx.x * 8 + warp;
     if (u >= nunits) return;  // the whole warp; no block barrier follows
-    unsigned char* base = smem + (size_t)warp * Sh::WARP_BYTES;
-    V* s_val = reinterpret_cast<V*>(base);
-    T* s_xv = reinterpret_cast<T*>(base + Sh::OFF_XV);
-    int32_t* s_rowend = reinterpret_cast<int32_t*>(base + Sh::OFF_RE);
-    const int64_t N = (int64_t)n + nnz;
-    const int64_t d0 = u * WI;
-    const int64_t d1 = min(d0 + WI, N);
-    int32_t bnd = 0;
-    if (unit_row) {
-        if (lane < 2) bnd = __ldg(unit_row + u + lane);
-    } else if (lane < 2) {
-        const int64_t d = lane == 0 ? d0 : d1;
-        int32_t lo = 0, hi = n;  // rows whose end item lies before d
-        while (lo < hi) {
-            const int32_t mid = lo + ((hi - lo) >> 1);
-            if ((int64_t)__ldg(rp + mid + 1) + mid + 1 > d) hi = mid;
-            else lo = mid + 1;
+    int16_t* mark = s_mark[warp];
+    T* sum = s_sum[warp];
+    const int64_t k0 = u * SEG_UNIT;
+    const int64_t kl = k0 + lane * E;  // this lane's first nonzero
+    int32_t c[E];
+    V v[E];
+    T xv[E];
+    if (k0 + SEG_UNIT <= nnz) {
+        load8(ci + kl, c);
+        if constexpr (sizeof(T) == 8) load8(va + kl, v);
+    } else {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            c[k] = kl + k < nnz ? ci[kl + k] : 0;
+            v[k] = kl + k < nnz ? va[kl + k] : V{};
         }
-        bnd = lo;
     }
-    const int32_t i0 = __shfl_sync(FULL, bnd, 0), i1 = __shfl_sync(FULL, bnd, 1);
-    const int64_t j0 = d0 - i0, j1 = d1 - i1;
-    const int32_t nloc = min(i1 - i0 + 1, n - i0);  // staged row ends
-    const int32_t cnt = (int32_t)(j1 - j0);
-    for (int k = lane; k < nloc; k += 32) s_rowend[k] = __ldg(rp + i0 + k + 1);
-    {
-        int32_t c[E];
-        V v[E];
-        T xv[E];
+    int32_t bnd = 0;
+    if (lane < 2) bnd = __ldg(unit_row + u + lane);
+    const int32_t i0 = __shfl_sync(FULL, bnd, 0);
+    const int32_t nrow = __shfl_sync(FULL, bnd, 1) - i0;  // rows that end in the unit
+    reinterpret_cast<int4*>(mark)[lane] = make_int4(-1, -1, -1, -1);
+    __syncwarp();
+    for (int q = lane; q < nrow; q += 32)
+        mark[(int64_t)__ldg(row_end + i0 + q) - 1 - k0] = (int16_t)q;
+    // x at skewed matrices' columns reuses little in L1: through L2 only
+    if (k0 + SEG_UNIT <= nnz) {
 #pragma unroll
-        for (int q = 0; q < E; ++q) {
-            const int k = lane + 32 * q;
-            if (k < cnt) {
-                c[q] = __ldcs(ci + j0 + k);
-                v[q] = va[j0 + k];
-            }
-        }
+        for (int k = 0; k < E; ++k) xv[k] = __ldcg(x + c[k]);
+        if constexpr (sizeof(T) != 8) load8(va + kl, v);
+    } else {
 #pragma unroll
-        for (int q = 0; q < E; ++q) {
-            const int k = lane + 32 * q;
-            if (k < cnt) xv[q] = __ldg(x + c[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-            const int k = lane + 32 * q;
-            if (k < cnt) {
-                s_val[mpad(k)] = v[q];
-                s_xv[mpad(k)] = xv[q];
-            }
-        }
+        for (int k = 0; k < E; ++k) xv[k] = kl + k < nnz ? __ldcg(x + c[k]) : T(0);
     }
     __syncwarp();
-    // this lane's start on the path
-    const int64_t dt = min(d0 + (int64_t)lane * E, d1);
-    int32_t lo = 0, hi = max(0, nloc);
-    while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if ((int64_t)s_rowend[mid] + i0 + mid + 1 > dt) hi = mid;
-        else lo = mid + 1;
-    }
-    int32_t i = i0 + lo;
-    int64_t j = dt - i;
-    const int64_t dend = min(dt + E, d1);
+    const int4 mq = reinterpret_cast<const int4*>(mark)[lane];
+    const int32_t mw[4] = {mq.x, mq.y, mq.z, mq.w};
     T acc = T(0);
-    int32_t head_row = -1;
-    T head_val = T(0);
-    int64_t rend = (i < n) ? (int64_t)s_rowend[i - i0] : 0;
-    for (int64_t d = dt; d < dend; ++d) {
-        if (i < n && j < rend) {
-            const int k = mpad((int)(j - j0));
-            acc = fmadd(cvt<T>(s_val[k]), s_xv[k], acc);
-            ++j;
-        } else {
-            if (head_row < 0) {
-                head_row = i;
-                head_val = acc;
-            } else {
-                epi.row(i, acc, nullptr);
-            }
+    int head = -1;  // first row that ends in this lane
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        acc = fmadd(cvt<T>(v[k]), xv[k], acc);
+        const int m = (k & 1) ? mw[k >> 1] >> 16 : (int)(int16_t)(mw[k >> 1] & 0xffff);
+        if (m >= 0) {
+            sum[m] = acc;
+            if (head < 0) head = m;
             acc = T(0);
-            ++i;
-            rend = (i < n && i - i0 < nloc) ? (int64_t)s_rowend[i - i0] : 0;
         }
     }
-    // Carries: lane l ends its piece inside row myrow with partial sum acc;
-    // rows are non-decreasing over the valid lanes, so a segmented inclusive
-    // scan (fixed order) gives each lane the sum over its run of lanes.
-    const bool valid = dt < d1;
-    const int32_t myrow = valid ? i : INT32_MAX;
-    const T sc = warp_seg_scan(myrow, acc);
-    const int32_t prow = __shfl_up_sync(FULL, myrow, 1);
-    const T psc = __shfl_up_sync(FULL, sc, 1);
-    const int32_t nrow = __shfl_down_sync(FULL, myrow, 1);
-    if (head_row >= 0) {
-        T vv = head_val;
-        if (lane > 0 && prow == head_row) vv = psc + vv;
-        epi.row(head_row, vv, nullptr);
+    // inclusive scan of the open parts over the lanes since the last one in
+    // which a row ended; only as many levels as the longest such run
+    const unsigned ends = __ballot_sync(FULL, head >= 0);
+    const unsigned upto = ends & (FULL >> (31 - lane));
+    const int start = upto ? 31 - __clz(upto) : 0;
+    const int run = (int)__reduce_max_sync(FULL, (unsigned)(lane - start));
+    for (int o = 1; o <= run; o <<= 1) {
+        const T ov = __shfl_up_sync(FULL, acc, o);
+        if (lane - o >= start) acc = ov + acc;
     }
-    // the row open at the end of the unit: carried by the last valid lane
-    if (valid && (lane == 31 || nrow == INT32_MAX)) {
-        carry_row[u] = (i < n) ? i : -1;
-        carry_val[u] = sc;
+    const T before = __shfl_up_sync(FULL, acc, 1);
+    if (head >= 0 && lane > 0) sum[head] = before + sum[head];
+    if (lane == 31) {
+        // the unit's last nonzero ends a row (also when the matrix ends here): no carry
+        const bool open = k0 + SEG_UNIT < nnz && (mw[3] >> 16) < 0;
+        carry_row[u] = open ? (row_id ? __ldg(row_id + i0 + nrow) : i0 + nrow) : -1;
+        carry_val[u] = acc;
+    }
+    __syncwarp();
+    for (int q = lane; q < nrow; q += 32) {
+        const int32_t i = i0 + q;
+        epi.row(row_id ? __ldg(row_id + i) : i, sum[q], nullptr);
     }
 }
 
@@ -787,7 +669,7 @@ k_csr_merge_warp(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
 // row.  The first row a lane ends may have begun in earlier lanes: it adds
 // their carries, combined with the 5-level segmented shuffle scan used by
 // the merge kernel; the run open at the end of a unit goes to
-// k_csr_merge_fixup.  Rows without entries are written by k_coo_empty.
+// k_carry_fixup.  Rows without entries are written by k_empty_rows.
 
 // E consecutive entries starting at k (k % E == 0): 16-byte loads when the
 // group is whole (the arrays start on 256-byte boundaries), else one by one.
@@ -889,7 +771,7 @@ k_coo_warp(int32_t n, int64_t nnz, const int32_t* __restrict__ rows,
 
 // Rows without entries: x_i = 0 (modes 0, 1) or beta x_i (mode 2).
 template <typename T>
-__global__ void k_coo_empty(int32_t count, const int32_t* __restrict__ idx, EpiStore<T> epi) {
+__global__ void k_empty_rows(int32_t count, const int32_t* __restrict__ idx, EpiStore<T> epi) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < count;
          k += (int64_t)gridDim.x * blockDim.x)
         epi.row(idx[k], T(0), nullptr);
@@ -898,7 +780,7 @@ __global__ void k_coo_empty(int32_t count, const int32_t* __restrict__ idx, EpiS
 // Adds the block carries to the rows they belong to: the first block of
 // every run of blocks sharing a carry row sums the run in block order.
 template <typename T>
-__global__ void k_csr_merge_fixup(int32_t nblocks, const int32_t* __restrict__ carry_row,
+__global__ void k_carry_fixup(int32_t nblocks, const int32_t* __restrict__ carry_row,
                                   const T* __restrict__ carry_val, T* __restrict__ y, T alpha,
                                   int mode) {
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblocks;
@@ -1292,11 +1174,5 @@ gk_status launch_spmv_rows(gk_matrix A, const T* x, const Epi& epi, cudaStream_t
 
 // Upper bound of the grid launch_spmv_rows uses for A (sizes partials).
 inline unsigned max_grid_rows(gk_matrix A) { return (unsigned)num_sms() * 8; }
-
-// merge-path items per thread for a value type
-template <typename V>
-struct MergeE {
-    static constexpr int value = 8;
-};
 
 }  // namespace gk

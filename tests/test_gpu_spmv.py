@@ -256,3 +256,52 @@ def test_f16_values_round_once_to_nearest_even(fmt):
                               np.sort(want.view(np.uint16)))
         assert np.all(got[e["col"] < 0].view(np.uint16) == 0)
     A.close()
+
+
+def _rows_of(lengths, ncols, seed):
+    """CSR with the given row lengths, random columns."""
+    rng = np.random.default_rng(seed)
+    rp = np.zeros(len(lengths) + 1, dtype=np.int32)
+    np.cumsum(lengths, out=rp[1:])
+    col = np.concatenate([np.sort(rng.choice(ncols, size=k, replace=False)) if k else
+                          np.zeros(0, np.int64) for k in lengths] + [np.zeros(0, np.int64)])
+    return W.CSR(len(lengths), ncols, rp, col, rng.standard_normal(int(rp[-1])))
+
+
+# row lengths around the segmented kernel's units (256 nonzeros, 8 per lane)
+SEGMENTS = {
+    "unit_ends_a_row": [256, 256, 8, 248, 1],
+    "one_short_of_a_unit": [255],
+    "one_past_a_unit": [200, 56, 1],
+    "every_entry_a_row": [1] * 700,
+    "row_over_many_units": [3, 4000, 2, 1500, 250],
+    "lane_edges": [8] * 40 + [7, 9] * 30 + [16, 24, 33],
+    "empty_rows_between": [0, 0, 5, 0, 256, 0, 0, 1, 0, 300, 0],
+    "long_empty_runs": [0] * 900 + [600] + [0] * 900 + [1] + [0] * 3,
+    "single_entry": [0, 1, 0],
+}
+
+
+@pytest.mark.parametrize("name", list(SEGMENTS))
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16", "f16"])
+def test_segmented_units(name, dtype):
+    """Rows that end at, before and after the units' and lanes' edges, rows
+    over many units, empty rows; infinities and NaN stay in their rows."""
+    m = _rows_of(SEGMENTS[name], 4096, 17)
+    A = _make(m, "csr", dtype, 2)
+    assert A.desc["spmv_kernel"] == 2
+    rng = np.random.default_rng(5)
+    x = rng.uniform(-1, 1, m.ncols)
+    y0 = rng.uniform(-1, 1, m.n)
+    for alpha, beta, use_y0 in ((1.0, 0.0, False), (2.5, 0.0, False), (-1.0, 1.0, True)):
+        y = _run(A, x, alpha, beta, y0 if use_y0 else None, dtype)
+        ref, scale = oracle_apply(m, x, alpha, beta, y0 if use_y0 else None, dtype)
+        assert_rows_close(y, ref, scale, TOL[dtype], f"{name} {dtype} a={alpha} b={beta}")
+    rows = np.repeat(np.arange(m.n), m.row_lengths())
+    for bad in (np.inf, np.nan):
+        xb = x.copy()
+        xb[m.col_idx[0]] = bad
+        hit = np.zeros(m.n, dtype=bool)
+        hit[rows[m.col_idx == m.col_idx[0]]] = True
+        assert np.array_equal(~np.isfinite(_run(A, xb, 1.0, 0.0, None, dtype)), hit)
+    A.close()
