@@ -336,14 +336,14 @@ gk_status gk_solve_async(gk_matrix A, const void* b, void* x,
  * whole batch): its CSR arrays, an ELL copy (where ELL stores at most 1.2 x
  * its nonzeros) or a SELL-P copy with slices of S rows; every layout sums a
  * row in CSR order, so the layout never changes a result.  The layout
- * policy (CSR, ELL, SELL-P with S = 8, 16 or 32) and the block size
- * (128/256/512 threads) are autotuned per batch shape on the first call for
- * that shape (value type, method, preconditioner, log2 of the largest n and
+ * policy (CSR, ELL, SELL-P with S = 8, 16 or 32) and, when no system has more
+ * than 1024 rows, the block size (256 or 512 threads; else 512) are autotuned
+ * per batch shape on the first call for that shape (value type, method, preconditioner, log2 of the largest n and
  * of the count): each candidate runs the batch capped at 30 iterations from
  * the callers' initial guesses, which are restored afterwards; the choice
  * is cached for the process and reported per system in infos (spmv_format,
  * slice_size, block_threads).  Batches of fewer than 64 systems, or with
- * GK_AUTOTUNE=0, use CSR and 256 threads;
+ * GK_AUTOTUNE=0, use CSR and 256 threads (512 above 1024 rows);
  * GK_BATCH_LAYOUT (csr | ell | sellp8 | sellp16 | sellp32 | sellp64) and
  * GK_BATCH_THREADS force either choice.  All
  * matrices must be CSR, square, of the same dtype, with n <= 16384; CG

@@ -42,7 +42,21 @@ struct SysDesc {
     int32_t* sset;
     int64_t pstride;
     int32_t K, S;
+    int32_t id;  // its place in the caller's arrays
 };
+
+// The next system of the batch for this block, -1: none left.  The systems
+// are ordered by work, the largest first, and the blocks of the one wave take
+// them as they come free: the last ones to run are small.  (Dealt out by
+// block index, 2048 systems of 64 to 4096 rows took 20.3 ms and 700 of them
+// kept the SMs busy 32 % of the time.)
+__device__ __forceinline__ int32_t next_system(int32_t* next, int32_t count) {
+    __shared__ int32_t s_next;
+    __syncthreads();  // the block is done with the previous system
+    if (threadIdx.x == 0) s_next = atomicAdd(next, 1);
+    __syncthreads();
+    return s_next < count ? s_next : -1;
+}
 
 struct SysOut {
     int32_t status, iters, restarts, pad;
@@ -61,111 +75,145 @@ struct BlockOpts {
 // block, so the block size (autotuned) never changes a system's result.
 constexpr int VL = 512;
 
-template <int NA>
+// per-thread partial sums: NS = VL / threads virtual lanes of NA sums
+template <int NA, int NS>
 struct VAcc {
-    double v[NA][4];
+    double v[NA][NS] = {};
 };
 
-template <int NA>
-__device__ __forceinline__ VAcc<NA> vacc() {
-    VAcc<NA> a;
-#pragma unroll
-    for (int k = 0; k < NA; ++k)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) a.v[k][s] = 0.0;
-    return a;
-}
-
-// f(i, s) for every row i of this thread; s = (i mod VL) / blockDim.x
-template <class F>
+// f(i, s) for every row i of this thread; s = (i mod VL) / NT
+template <int NT, class F>
 __device__ __forceinline__ void for_rows_vl(int32_t n, F&& f) {
-    const int ns = VL / (int)blockDim.x;
     for (int32_t i0 = threadIdx.x; i0 < n; i0 += VL) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            if (s < ns) {
-                const int32_t i = i0 + s * (int32_t)blockDim.x;
-                if (i < n) f(i, s);
-            }
+        for (int s = 0; s < VL / NT; ++s) {
+            const int32_t i = i0 + s * NT;
+            if (i < n) f(i, s);
         }
     }
 }
 
-// Sum of the virtual-lane partials, returned to every thread.
-template <int NA>
-__device__ __forceinline__ void vl_allsum(const VAcc<NA>& acc, double (&out)[NA]) {
-    __shared__ double sh[NA][VL];
-    __shared__ double tot[NA];
-    const int ns = VL / (int)blockDim.x;
+// The reductions' shared memory, one for all of a kernel's sums.
+struct SumScratch {
+    double sh[2][VL];
+    double tot[2];
+    int code;
+};
+__device__ __forceinline__ SumScratch& sum_scratch() {
+    __shared__ SumScratch z;
+    return z;
+}
+
+// Sums the virtual-lane partials over the block; thread 0 runs fin(totals),
+// which leaves what follows from them in shared memory, and every thread gets
+// its code.  Only thread 0: an FP64 instruction costs the SM 16 cycles per
+// warp that issues it, and the divisions and square roots of an iteration
+// done by all 16 warps took as long as the rows of a 2,000-row system.
+template <int NT, int NA, class Fin>
+__device__ __forceinline__ int vl_sum(const VAcc<NA, VL / NT>& acc, Fin&& fin) {
+    static_assert(NA <= 2, "the scratch holds two values");
+    SumScratch& z = sum_scratch();
 #pragma unroll
     for (int a = 0; a < NA; ++a)
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
-            if (s < ns) sh[a][threadIdx.x + s * blockDim.x] = acc.v[a][s];
+        for (int s = 0; s < VL / NT; ++s) z.sh[a][threadIdx.x + s * NT] = acc.v[a][s];
     __syncthreads();
-    if (threadIdx.x < 32) {
+    // warp a sums value a (each on its own sub-partition's FP64 pipe), lane
+    // l lanes l, l + 32, ... as a pairwise tree
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < NA) {
+        double t[VL / 32];
 #pragma unroll
-        for (int a = 0; a < NA; ++a) {
-            double t[VL / 32];  // lane l: lanes l, l+32, ... as a pairwise tree
+        for (int k = 0; k < VL / 32; ++k) t[k] = z.sh[warp][lane + 32 * k];
 #pragma unroll
-            for (int k = 0; k < VL / 32; ++k) t[k] = sh[a][threadIdx.x + 32 * k];
+        for (int w = VL / 64; w > 0; w >>= 1)
 #pragma unroll
-            for (int w = VL / 64; w > 0; w >>= 1)
-#pragma unroll
-                for (int k = 0; k < w; ++k) t[k] += t[k + w];
-            const double tt = warp_sum(t[0]);
-            if (threadIdx.x == 0) tot[a] = tt;
-        }
+            for (int k = 0; k < w; ++k) t[k] += t[k + w];
+        const double tt = warp_sum(t[0]);
+        if (lane == 0) z.tot[warp] = tt;
     }
     __syncthreads();
-#pragma unroll
-    for (int a = 0; a < NA; ++a) out[a] = tot[a];
+    if (threadIdx.x == 0) z.code = fin(z.tot);
     __syncthreads();
+    return z.code;
 }
 
-template <typename V, typename T, typename G>
-__device__ __forceinline__ T row_dot(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                     const V* __restrict__ va, const G* __restrict__ g, int32_t i) {
+// sqrt(t) <= thr (thr >= 0); the square root, ~1,300 cycles, is taken only
+// where thr^2 does not already decide
+__device__ __forceinline__ bool root_passes(double t, double thr, double thr2) {
+    return t <= 1.000001 * thr2 && sqrt(t) <= thr;
+}
+
+// What thread 0 keeps of a running solve.
+struct BlockScalars {
+    double bn, thr, thr2;
+    double rho, rho_new, alpha, omega, beta;
+    double rec2;  // last squared recurrence residual
+    double tru;
+};
+
+// A row's len entries at positions p, p + step, ... times the gathered
+// vector: four at a time, their columns and values loaded before the gathers
+// and those before the first FMA, so a row is one chain of dependent loads
+// per four entries.  The one to three left over branch: an FMA that every
+// lane skips must not reach the FP64 pipe.  PAD: entries with column -1 (after
+// the row's last one) have value 0 and add nothing.
+template <bool PAD, typename V, typename T, typename G>
+__device__ __forceinline__ T row_chunks(const int32_t* __restrict__ col, const V* __restrict__ val,
+                                        const G* __restrict__ g, int64_t p, int64_t step,
+                                        int32_t len) {
     T s = T(0);
-    const int32_t e = rp[i + 1];
-    for (int32_t k = rp[i]; k < e; ++k) s = fmadd(cvt<T>(va[k]), (T)g[ci[k]], s);
+    auto gather = [&](int32_t c) -> T { return PAD && c < 0 ? T(0) : (T)g[c]; };
+    for (; len >= 4; len -= 4, p += 4 * step) {
+        int32_t c[4];
+        T v[4], x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            c[u] = col[p + u * step];
+            v[u] = cvt<T>(val[p + u * step]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = gather(c[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s = fmadd(v[u], x[u], s);
+    }
+    if (len > 0) {
+        const int32_t c0 = col[p], c1 = len > 1 ? col[p + step] : c0,
+                      c2 = len > 2 ? col[p + 2 * step] : c0;
+        const T v0 = cvt<T>(val[p]), v1 = len > 1 ? cvt<T>(val[p + step]) : T(0),
+                v2 = len > 2 ? cvt<T>(val[p + 2 * step]) : T(0);
+        const T x0 = gather(c0);
+        if (len > 1) {
+            const T x1 = gather(c1);
+            if (len > 2) {
+                const T x2 = gather(c2);
+                s = fmadd(v2, x2, fmadd(v1, x1, fmadd(v0, x0, s)));
+            } else {
+                s = fmadd(v1, x1, fmadd(v0, x0, s));
+            }
+        } else {
+            s = fmadd(v0, x0, s);
+        }
+    }
     return s;
 }
 
 // Row i of a system in its layout (see BatchLayout): entries in CSR order,
 // padding (column -1) only after a row's last entry.
-// L >= 0: every system of the batch has layout L (the branch is resolved at
-// compile time); L = -1: the layout is read per system.
+// L = BL_CSR: every system of the batch (the branch is resolved at compile
+// time); L = -1: the layout is read per system.
 template <typename V, typename T, int L, typename G>
 __device__ __forceinline__ T sys_row_dot(const SysDesc& d, const G* __restrict__ g, int32_t i) {
     const int fmt = L >= 0 ? L : d.fmt;
-    if (fmt == BL_ELL) {
-        const int32_t* __restrict__ col = d.pcol;
-        const V* __restrict__ val = (const V*)d.pval;
-        T s = T(0);
-        int64_t p = i;
-        for (int32_t k = 0; k < d.K; ++k, p += d.pstride) {
-            const int32_t c = col[p];
-            if (c < 0) break;
-            s = fmadd(cvt<T>(val[p]), (T)g[c], s);
-        }
-        return s;
-    }
+    if (fmt == BL_ELL)
+        return row_chunks<true, V, T>(d.pcol, (const V*)d.pval, g, i, d.pstride, d.K);
     if (fmt == BL_SELLP) {
         const int32_t sl = i / d.S, t = i - sl * d.S;
-        const int32_t* __restrict__ col = d.pcol;
-        const V* __restrict__ val = (const V*)d.pval;
-        const int32_t len = d.slen[sl];
-        int64_t p = (int64_t)d.sset[sl] * d.S + t;
-        T s = T(0);
-        for (int32_t k = 0; k < len; ++k, p += d.S) {
-            const int32_t c = col[p];
-            if (c < 0) break;
-            s = fmadd(cvt<T>(val[p]), (T)g[c], s);
-        }
-        return s;
+        return row_chunks<true, V, T>(d.pcol, (const V*)d.pval, g, (int64_t)d.sset[sl] * d.S + t,
+                                      (int64_t)d.S, d.slen[sl]);
     }
-    return row_dot<V, T>(d.rp, d.ci, (const V*)d.va, g, i);
+    const int32_t a = d.rp[i];
+    return row_chunks<false, V, T>(d.ci, (const V*)d.va, g, a, 1, d.rp[i + 1] - a);
 }
 
 // Writes the padded copy of every system whose layout is ELL or SELL-P
@@ -235,17 +283,37 @@ __device__ __forceinline__ T row_dinv(const int32_t* __restrict__ rp, const int3
     return d == T(0) ? T(0) : T(1) / d;
 }
 
+// why a block's solve ends (0: it goes on)
+enum : int { BE_OK = 1, BE_PASSED, BE_NAN, BE_BREAKDOWN, BE_ZERO_DIAG, BE_ZERO_RHS };
+
+// r = b - A x in place; BE_OK when ||r|| <= thr, BE_NAN when not finite
+template <typename V, typename T, int L, int NT>
+__device__ int block_true_resid(const SysDesc& d, T* r, BlockScalars& S) {
+    const T* b = (const T*)d.b;
+    const T* x = (const T*)d.x;
+    VAcc<1, VL / NT> tt;
+    for_rows_vl<NT>(d.n, [&](int32_t i, int s) {
+        const T ri = b[i] - sys_row_dot<V, T, L>(d, x, i);
+        r[i] = ri;
+        tt.v[0][s] = fma((double)ri, (double)ri, tt.v[0][s]);
+    });
+    return vl_sum<NT>(tt, [&](const double* t) -> int {
+        const double tn = sqrt(t[0]);
+        S.tru = tn / S.bn;
+        return !isfinite(tn) ? BE_NAN : tn <= S.thr ? BE_OK : 0;
+    });
+}
+
 // Prepares a system: Jacobi diagonal (in work slot 0), ||b||, true residual.
-// Returns false (and fills o) when the solve is already decided.
-template <typename V, typename T, int L>
-__device__ bool block_setup(const SysDesc& d, const BlockOpts& opt, T* dinv, T* r, double& bn,
-                            double& thr, SysOut& o) {
+template <typename V, typename T, int L, int NT>
+__device__ int block_setup(const SysDesc& d, const BlockOpts& opt, T* dinv, T* r,
+                           BlockScalars& S) {
     const int32_t n = d.n;
     const V* va = (const V*)d.va;
     const T* b = (const T*)d.b;
     T* x = (T*)d.x;
-    VAcc<2> acc = vacc<2>();
-    for_rows_vl(n, [&](int32_t i, int s) {
+    VAcc<2, VL / NT> acc;
+    for_rows_vl<NT>(n, [&](int32_t i, int s) {
         const T bi = b[i];
         acc.v[0][s] = fma((double)bi, (double)bi, acc.v[0][s]);
         if (opt.prec) {
@@ -254,281 +322,265 @@ __device__ bool block_setup(const SysDesc& d, const BlockOpts& opt, T* dinv, T* 
             if (di == T(0)) acc.v[1][s] = 1.0;
         }
     });
-    double tot[2];
-    vl_allsum<2>(acc, tot);
-    o.iters = 0;
-    o.restarts = 0;
-    o.rec = o.tru = 0.0;
-    if (tot[1] != 0.0) {
-        o.status = GK_ERR_ZERO_DIAG;
-        return false;
-    }
-    bn = sqrt(tot[0]);
-    thr = d.tol * bn;
-    if (bn == 0.0) {
-        for (int32_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = T(0);
-        o.status = GK_OK;
-        return false;
-    }
-    if (!isfinite(bn)) {
-        o.status = GK_ERR_NAN;
-        return false;
-    }
-    VAcc<1> rr = vacc<1>();
-    for_rows_vl(n, [&](int32_t i, int s) {
-        const T ri = b[i] - sys_row_dot<V, T, L>(d, x, i);
-        r[i] = ri;
-        rr.v[0][s] = fma((double)ri, (double)ri, rr.v[0][s]);
+    const int code = vl_sum<NT>(acc, [&](const double* t) -> int {
+        S.tru = S.rec2 = 0.0;
+        S.bn = sqrt(t[0]);
+        S.thr = d.tol * S.bn;
+        S.thr2 = S.thr * S.thr;
+        return t[1] != 0.0 ? BE_ZERO_DIAG : S.bn == 0.0 ? BE_ZERO_RHS : !isfinite(S.bn) ? BE_NAN : 0;
     });
-    double t1[1];
-    vl_allsum<1>(rr, t1);
-    const double rn = sqrt(t1[0]);
-    o.rec = o.tru = rn / bn;
-    if (!isfinite(rn)) {
-        o.status = GK_ERR_NAN;
-        return false;
-    }
-    if (rn <= thr) {
-        o.status = GK_OK;
-        return false;
-    }
-    o.status = GK_NOT_CONVERGED;
-    return true;
+    if (code == BE_ZERO_RHS)
+        for (int32_t i = threadIdx.x; i < n; i += NT) x[i] = T(0);
+    if (code != 0) return code;
+    const int res = block_true_resid<V, T, L, NT>(d, r, S);
+    if (threadIdx.x == 0) S.rec2 = -1.0;  // no recurrence yet: its residual is the true one
+    return res;
 }
 
-// r = b - A x in place; returns ||r||
-template <typename V, typename T, int L>
-__device__ double block_true_resid(const SysDesc& d, T* r) {
-    const V* va = (const V*)d.va;
-    const T* b = (const T*)d.b;
-    const T* x = (const T*)d.x;
-    VAcc<1> tt = vacc<1>();
-    for_rows_vl(d.n, [&](int32_t i, int s) {
-        const T ri = b[i] - sys_row_dot<V, T, L>(d, x, i);
-        r[i] = ri;
-        tt.v[0][s] = fma((double)ri, (double)ri, tt.v[0][s]);
-    });
-    double t[1];
-    vl_allsum<1>(tt, t);
-    return sqrt(t[0]);
+// The outcome of a solve that ended with `end` (0: at the iteration cap).
+__device__ __forceinline__ SysOut block_outcome(int end, int32_t iters, int32_t restarts,
+                                                double first_true, const BlockScalars& S) {
+    SysOut o;
+    o.status = end == BE_OK || end == BE_ZERO_RHS ? GK_OK
+               : end == BE_NAN                    ? GK_ERR_NAN
+               : end == BE_BREAKDOWN              ? GK_BREAKDOWN
+               : end == BE_ZERO_DIAG              ? GK_ERR_ZERO_DIAG
+                                                  : GK_NOT_CONVERGED;
+    o.iters = iters;
+    o.restarts = restarts;
+    o.pad = 0;
+    o.tru = S.tru;
+    o.rec = S.rec2 < 0.0 ? first_true : S.rec2 > 0.0 || S.rec2 != S.rec2 ? sqrt(S.rec2) / S.bn : 0.0;
+    return o;
 }
 
 // ---------------------------------------------------------------- CG
 // work slots: 0 dinv, 1 r, 2 q, 3 scratch (final residual)
 constexpr int BLOCK_MAX_THREADS = 512;
 
-template <typename V, typename T, int L>
-__global__ void __launch_bounds__(BLOCK_MAX_THREADS, 1) k_block_cg(const SysDesc* __restrict__ sys, SysOut* __restrict__ outs,
-                           int32_t count, BlockOpts opt) {
+template <typename V, typename T, int L, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_block_cg(const SysDesc* __restrict__ sys, SysOut* __restrict__ outs,
+                           int32_t count, int32_t* next, BlockOpts opt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ BlockScalars S;
     T* ps = reinterpret_cast<T*>(smem_raw);
-    for (int32_t sidx = blockIdx.x; sidx < count; sidx += gridDim.x) {
+    for (int32_t sidx; (sidx = next_system(next, count)) >= 0;) {
         const SysDesc d = sys[sidx];
         const int32_t n = d.n;
-        const V* va = (const V*)d.va;
         T* x = (T*)d.x;
         T* dinv = (T*)d.work;
         T* r = dinv + d.ld;
         T* q = r + d.ld;
         T* scratch = q + d.ld;
-        SysOut o;
-        double bn = 0.0, thr = 0.0;
-        if (block_setup<V, T, L>(d, opt, dinv, r, bn, thr, o)) {
-            double rho = 0.0;
-            auto init_dir = [&]() {
-                VAcc<1> rz = vacc<1>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T ri = r[i];
-                    const T zi = opt.prec ? dinv[i] * ri : ri;
-                    ps[i] = zi;
-                    rz.v[0][s] = fma((double)ri, (double)zi, rz.v[0][s]);
-                });
-                double t[1];
-                vl_allsum<1>(rz, t);
-                rho = t[0];
-            };
-            init_dir();
-            int32_t k = 0;
-            while (k < opt.max_iters) {
-                VAcc<1> pq = vacc<1>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T sv = sys_row_dot<V, T, L>(d, ps, i);
-                    q[i] = sv;
-                    pq.v[0][s] = fma((double)ps[i], (double)sv, pq.v[0][s]);
-                });
-                double tp[1];
-                vl_allsum<1>(pq, tp);
-                if (!isfinite(tp[0])) { o.status = GK_ERR_NAN; break; }
-                if (tp[0] <= 0.0) { o.status = GK_BREAKDOWN; break; }
-                const double alpha = rho / tp[0];
-                const T ta = (T)alpha;
-                VAcc<2> a2 = vacc<2>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    x[i] = fmadd(ta, ps[i], x[i]);
-                    const T ri = fmadd(-ta, q[i], r[i]);
-                    r[i] = ri;
-                    const T zi = opt.prec ? dinv[i] * ri : ri;
-                    a2.v[0][s] = fma((double)ri, (double)zi, a2.v[0][s]);
-                    a2.v[1][s] = fma((double)ri, (double)ri, a2.v[1][s]);
-                });
-                double t2[2];
-                vl_allsum<2>(a2, t2);
-                ++k;
-                const double rn = sqrt(t2[1]);
-                o.rec = rn / bn;
-                if (!isfinite(rn) || !isfinite(t2[0])) { o.status = GK_ERR_NAN; break; }
-                if (rn <= thr) {
-                    const double tn = block_true_resid<V, T, L>(d, r);
-                    if (tn <= thr) { o.status = GK_OK; break; }
-                    o.restarts += 1;  // residual replacement, restart from x
-                    init_dir();
-                    continue;
-                }
-                const double beta = t2[0] / rho;
-                rho = t2[0];
-                const T tb = (T)beta;
-                for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
-                    const T zi = opt.prec ? dinv[i] * r[i] : r[i];
-                    ps[i] = fmadd(tb, ps[i], zi);
-                }
-                __syncthreads();
+        int32_t k = 0, restarts = 0;
+        int end = block_setup<V, T, L, NT>(d, opt, dinv, r, S);
+        const double first_true = S.tru;
+        const bool run = end == 0;
+        auto init_dir = [&]() {
+            VAcc<1, VL / NT> rz;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T ri = r[i];
+                const T zi = opt.prec ? dinv[i] * ri : ri;
+                ps[i] = zi;
+                rz.v[0][s] = fma((double)ri, (double)zi, rz.v[0][s]);
+            });
+            vl_sum<NT>(rz, [&](const double* t) {
+                S.rho = t[0];
+                return 0;
+            });
+        };
+        if (run) init_dir();
+        while (end == 0 && k < opt.max_iters) {
+            VAcc<1, VL / NT> pq;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T sv = sys_row_dot<V, T, L>(d, ps, i);
+                q[i] = sv;
+                pq.v[0][s] = fma((double)ps[i], (double)sv, pq.v[0][s]);
+            });
+            end = vl_sum<NT>(pq, [&](const double* t) -> int {
+                S.alpha = S.rho / t[0];
+                return !isfinite(t[0]) ? BE_NAN : t[0] <= 0.0 ? BE_BREAKDOWN : 0;
+            });
+            if (end != 0) break;
+            const T ta = (T)S.alpha;
+            VAcc<2, VL / NT> a2;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                x[i] = fmadd(ta, ps[i], x[i]);
+                const T ri = fmadd(-ta, q[i], r[i]);
+                r[i] = ri;
+                const T zi = opt.prec ? dinv[i] * ri : ri;
+                if (opt.prec) q[i] = zi;  // q has been used: z waits there for beta
+                a2.v[0][s] = fma((double)ri, (double)zi, a2.v[0][s]);
+                a2.v[1][s] = fma((double)ri, (double)ri, a2.v[1][s]);
+            });
+            end = vl_sum<NT>(a2, [&](const double* t) -> int {
+                S.rec2 = t[1];
+                if (!isfinite(t[1]) || !isfinite(t[0])) return BE_NAN;
+                if (root_passes(t[1], S.thr, S.thr2)) return BE_PASSED;
+                S.beta = t[0] / S.rho;
+                S.rho = t[0];
+                return 0;
+            });
+            ++k;
+            if (end == BE_PASSED) {
+                // the true residual decides; a NaN there ends no solve here
+                end = block_true_resid<V, T, L, NT>(d, r, S) == BE_OK ? BE_OK : 0;
+                if (end != 0) break;
+                restarts += 1;  // residual replacement, restart from x
+                init_dir();
+                continue;
             }
-            o.iters = k;
-            o.tru = block_true_resid<V, T, L>(d, scratch) / bn;
+            if (end != 0) break;
+            const T tb = (T)S.beta;
+            for (int32_t i = threadIdx.x; i < n; i += NT)
+                ps[i] = fmadd(tb, ps[i], opt.prec ? q[i] : r[i]);
+            __syncthreads();
         }
-        if (threadIdx.x == 0) outs[sidx] = o;
-        __syncthreads();
+        if (run) block_true_resid<V, T, L, NT>(d, scratch, S);
+        if (threadIdx.x == 0) outs[d.id] = block_outcome(end, k, restarts, first_true, S);
     }
 }
 
 // ---------------------------------------------------------------- BiCGSTAB
 // work slots: 0 dinv, 1 r, 2 rhat, 3 p, 4 phat, 5 v, 6 s, 7 shat, 8 t
-template <typename V, typename T, int L>
-__global__ void __launch_bounds__(BLOCK_MAX_THREADS, 1) k_block_bicgstab(const SysDesc* __restrict__ sys, SysOut* __restrict__ outs,
-                                 int32_t count, BlockOpts opt) {
+template <typename V, typename T, int L, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_block_bicgstab(const SysDesc* __restrict__ sys, SysOut* __restrict__ outs,
+                                 int32_t count, int32_t* next, BlockOpts opt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ BlockScalars S;
     T* gs = reinterpret_cast<T*>(smem_raw);  // gathered vector
-    for (int32_t sidx = blockIdx.x; sidx < count; sidx += gridDim.x) {
+    for (int32_t sidx; (sidx = next_system(next, count)) >= 0;) {
         const SysDesc d = sys[sidx];
         const int32_t n = d.n;
-        const V* va = (const V*)d.va;
         T* x = (T*)d.x;
         T* dinv = (T*)d.work;
         T *r = dinv + d.ld, *rh = r + d.ld, *p = rh + d.ld, *ph = p + d.ld, *v = ph + d.ld;
         T *sv = v + d.ld, *sh = sv + d.ld, *t = sh + d.ld;
-        SysOut o;
-        double bn = 0.0, thr = 0.0;
-        if (block_setup<V, T, L>(d, opt, dinv, r, bn, thr, o)) {
-            double rho = 1.0, alpha = 1.0, omega = 1.0, rho_new = 0.0;
-            auto restart = [&]() {
-                VAcc<1> a = vacc<1>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T ri = r[i];
-                    rh[i] = ri;
-                    p[i] = T(0);
-                    v[i] = T(0);
-                    a.v[0][s] = fma((double)ri, (double)ri, a.v[0][s]);
-                });
-                double tt[1];
-                vl_allsum<1>(a, tt);
-                rho = alpha = omega = 1.0;
-                rho_new = tt[0];
-            };
-            restart();
-            int32_t k = 0;
-            while (k < opt.max_iters) {
-                if (!isfinite(rho_new)) { o.status = GK_ERR_NAN; break; }
-                if (rho_new == 0.0) { o.status = GK_BREAKDOWN; break; }
-                const T beta = (T)((rho_new / rho) * (alpha / omega));
-                const T tw = (T)omega;
-                for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        int32_t k = 0, restarts = 0;
+        int end = block_setup<V, T, L, NT>(d, opt, dinv, r, S);
+        const double first_true = S.tru;
+        const bool run = end == 0;
+        // beta of the next step from rho', or why there is none
+        auto next_beta = [&]() -> int {
+            if (!isfinite(S.rho_new)) return BE_NAN;
+            if (S.rho_new == 0.0) return BE_BREAKDOWN;
+            S.beta = (S.rho_new / S.rho) * (S.alpha / S.omega);
+            return 0;
+        };
+        auto restart = [&]() -> int {
+            VAcc<1, VL / NT> a;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T ri = r[i];
+                rh[i] = ri;
+                p[i] = T(0);
+                v[i] = T(0);
+                a.v[0][s] = fma((double)ri, (double)ri, a.v[0][s]);
+            });
+            return vl_sum<NT>(a, [&](const double* tt) -> int {
+                S.rho = S.alpha = S.omega = 1.0;
+                S.rho_new = tt[0];
+                return next_beta();
+            });
+        };
+        // the true residual decides a passed recurrence residual: 0 and a
+        // restart from it when it fails
+        auto confirm = [&]() -> int {
+            if (block_true_resid<V, T, L, NT>(d, r, S) == BE_OK) return BE_OK;
+            restarts += 1;
+            return restart();
+        };
+        if (run) end = restart();
+        // what stops a step (NaN, breakdown) counts only while steps are left
+        if (run && opt.max_iters <= 0) end = 0;
+        while (end == 0 && k < opt.max_iters) {
+            {
+                const T beta = (T)S.beta, tw = (T)S.omega;
+                for (int32_t i = threadIdx.x; i < n; i += NT) {
                     const T pi = fmadd(beta, fmadd(-tw, v[i], p[i]), r[i]);
                     p[i] = pi;
                     const T hi = opt.prec ? dinv[i] * pi : pi;
                     ph[i] = hi;
                     gs[i] = hi;
                 }
-                __syncthreads();
-                VAcc<1> rv = vacc<1>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T vi = sys_row_dot<V, T, L>(d, gs, i);
-                    v[i] = vi;
-                    rv.v[0][s] = fma((double)rh[i], (double)vi, rv.v[0][s]);
-                });
-                double trv[1];
-                vl_allsum<1>(rv, trv);
-                if (!isfinite(trv[0])) { o.status = GK_ERR_NAN; break; }
-                if (trv[0] == 0.0) { o.status = GK_BREAKDOWN; break; }
-                alpha = rho_new / trv[0];
-                const T ta = (T)alpha;
-                VAcc<1> ss = vacc<1>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T si = fmadd(-ta, v[i], r[i]);
-                    sv[i] = si;
-                    ss.v[0][s] = fma((double)si, (double)si, ss.v[0][s]);
-                });
-                double tss[1];
-                vl_allsum<1>(ss, tss);
-                ++k;
-                const double sn = sqrt(tss[0]);
-                if (!isfinite(sn)) { o.status = GK_ERR_NAN; break; }
-                if (sn <= thr) {  // half-step exit
-                    for (int32_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = fmadd(ta, ph[i], x[i]);
-                    o.rec = sn / bn;
-                    __syncthreads();
-                    const double tn = block_true_resid<V, T, L>(d, r);
-                    if (tn <= thr) { o.status = GK_OK; break; }
-                    o.restarts += 1;
-                    restart();
-                    continue;
-                }
-                for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
-                    const T hi = opt.prec ? dinv[i] * sv[i] : sv[i];
-                    sh[i] = hi;
-                    gs[i] = hi;
-                }
-                __syncthreads();
-                VAcc<2> a2 = vacc<2>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    const T ti = sys_row_dot<V, T, L>(d, gs, i);
-                    t[i] = ti;
-                    a2.v[0][s] = fma((double)ti, (double)sv[i], a2.v[0][s]);
-                    a2.v[1][s] = fma((double)ti, (double)ti, a2.v[1][s]);
-                });
-                double t2[2];
-                vl_allsum<2>(a2, t2);
-                if (!isfinite(t2[0]) || !isfinite(t2[1])) { o.status = GK_ERR_NAN; break; }
-                if (t2[1] == 0.0) { o.status = GK_BREAKDOWN; break; }
-                omega = t2[0] / t2[1];
-                if (omega == 0.0) { o.status = GK_BREAKDOWN; break; }
-                const T to = (T)omega;
-                VAcc<2> a3 = vacc<2>();
-                for_rows_vl(n, [&](int32_t i, int s) {
-                    x[i] = fmadd(to, sh[i], fmadd(ta, ph[i], x[i]));
-                    const T ri = fmadd(-to, t[i], sv[i]);
-                    r[i] = ri;
-                    a3.v[0][s] = fma((double)rh[i], (double)ri, a3.v[0][s]);
-                    a3.v[1][s] = fma((double)ri, (double)ri, a3.v[1][s]);
-                });
-                double t3[2];
-                vl_allsum<2>(a3, t3);
-                rho = rho_new;
-                rho_new = t3[0];
-                const double rn = sqrt(t3[1]);
-                o.rec = rn / bn;
-                if (!isfinite(rn)) { o.status = GK_ERR_NAN; break; }
-                if (rn <= thr) {
-                    const double tn = block_true_resid<V, T, L>(d, r);
-                    if (tn <= thr) { o.status = GK_OK; break; }
-                    o.restarts += 1;
-                    restart();
-                }
             }
-            o.iters = k;
-            o.tru = block_true_resid<V, T, L>(d, t) / bn;
+            __syncthreads();
+            VAcc<1, VL / NT> rv;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T vi = sys_row_dot<V, T, L>(d, gs, i);
+                v[i] = vi;
+                rv.v[0][s] = fma((double)rh[i], (double)vi, rv.v[0][s]);
+            });
+            end = vl_sum<NT>(rv, [&](const double* tt) -> int {
+                S.alpha = S.rho_new / tt[0];
+                return !isfinite(tt[0]) ? BE_NAN : tt[0] == 0.0 ? BE_BREAKDOWN : 0;
+            });
+            if (end != 0) break;
+            const T ta = (T)S.alpha;
+            VAcc<1, VL / NT> ss;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T si = fmadd(-ta, v[i], r[i]);
+                sv[i] = si;
+                ss.v[0][s] = fma((double)si, (double)si, ss.v[0][s]);
+            });
+            ++k;
+            end = vl_sum<NT>(ss, [&](const double* tt) -> int {
+                if (!isfinite(tt[0])) return BE_NAN;
+                if (!root_passes(tt[0], S.thr, S.thr2)) return 0;
+                S.rec2 = tt[0];
+                return BE_PASSED;
+            });
+            if (end == BE_PASSED) {  // half-step exit
+                for (int32_t i = threadIdx.x; i < n; i += NT) x[i] = fmadd(ta, ph[i], x[i]);
+                __syncthreads();
+                end = confirm();
+                if (end > 0 && end != BE_OK && k >= opt.max_iters) end = 0;
+                continue;
+            }
+            if (end != 0) break;
+            for (int32_t i = threadIdx.x; i < n; i += NT) {
+                const T hi = opt.prec ? dinv[i] * sv[i] : sv[i];
+                sh[i] = hi;
+                gs[i] = hi;
+            }
+            __syncthreads();
+            VAcc<2, VL / NT> a2;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                const T ti = sys_row_dot<V, T, L>(d, gs, i);
+                t[i] = ti;
+                a2.v[0][s] = fma((double)ti, (double)sv[i], a2.v[0][s]);
+                a2.v[1][s] = fma((double)ti, (double)ti, a2.v[1][s]);
+            });
+            end = vl_sum<NT>(a2, [&](const double* tt) -> int {
+                if (!isfinite(tt[0]) || !isfinite(tt[1])) return BE_NAN;
+                if (tt[1] == 0.0) return BE_BREAKDOWN;
+                S.omega = tt[0] / tt[1];
+                return S.omega == 0.0 ? BE_BREAKDOWN : 0;
+            });
+            if (end != 0) break;
+            const T to = (T)S.omega;
+            VAcc<2, VL / NT> a3;
+            for_rows_vl<NT>(n, [&](int32_t i, int s) {
+                x[i] = fmadd(to, sh[i], fmadd(ta, ph[i], x[i]));
+                const T ri = fmadd(-to, t[i], sv[i]);
+                r[i] = ri;
+                a3.v[0][s] = fma((double)rh[i], (double)ri, a3.v[0][s]);
+                a3.v[1][s] = fma((double)ri, (double)ri, a3.v[1][s]);
+            });
+            end = vl_sum<NT>(a3, [&](const double* tt) -> int {
+                S.rho = S.rho_new;
+                S.rho_new = tt[0];
+                S.rec2 = tt[1];
+                if (!isfinite(tt[1])) return BE_NAN;
+                if (root_passes(tt[1], S.thr, S.thr2)) return BE_PASSED;
+                return k < opt.max_iters ? next_beta() : 0;
+            });
+            if (end == BE_PASSED) {
+                end = confirm();
+                if (end > 0 && end != BE_OK && k >= opt.max_iters) end = 0;
+            }
         }
-        if (threadIdx.x == 0) outs[sidx] = o;
-        __syncthreads();
+        if (run) block_true_resid<V, T, L, NT>(d, t, S);
+        if (threadIdx.x == 0) outs[d.id] = block_outcome(end, k, restarts, first_true, S);
     }
 }
 
@@ -541,11 +593,20 @@ static int nslots(int method) { return method == GK_CG ? 4 : 9; }
 // an ELL copy when ELL stores at most 1.2 x its nonzeros, else keeps its
 // CSR; BL_SELLP gives each system a SELL-P copy with slices of S rows.
 // nt: threads per block.  The untuned default (batches of fewer than
-// TUNE_MIN_COUNT systems) is CSR with 256 threads: on lone serving-size systems (n 1,575 to
-// 13,689; stencils and banded SPD) CSR took 0.31-0.65x the time of ELL or
-// SELL-P(32) in the one-block kernel (e.g. 2D Laplacian n = 13,456: 33.8 ms
-// against 56.8 ms with ELL).
+// TUNE_MIN_COUNT systems) is CSR: on lone serving-size systems (n 1,575 to
+// 13,689; stencils and banded SPD) it took 0.31-0.65x the time of ELL or
+// SELL-P(32) in the one-block kernel.
 constexpr int32_t TUNE_MIN_COUNT = 64;  // smallest batch the autotuner times
+
+// Threads per block where the largest system decides: 512 above this many
+// rows, below it 256, or what the autotuner times of the two.  A batch ends
+// with its slowest systems alone on their SMs, where twice the threads hide
+// twice the latency; the tuner's short trials do not see that end.  ms with
+// 256 / 512 threads, FP64: 2048 systems of up to 4096 rows 10.1 / 7.1, 700
+// 6.2 / 4.0, 20 2.7 / 1.9, one of 1881 rows 1.5 / 1.0; 1500 of up to 1024
+// rows 1.7 / 1.8; FP32: 4.2 / 2.9, 2.6 / 1.7, 1.1 / 0.75, 0.42 / 0.37; 0.77 /
+// 0.82.  (128 threads: 1.4 to 2.4 times as long as 256.)
+constexpr int32_t WIDE_BLOCK_ROWS = 1024;
 
 struct BatchCfg {
     int nt = 256;
@@ -589,30 +650,31 @@ struct BatchLease {
     }
 };
 
-// The block kernel for a method, value type and batch layout (lay: the one
-// layout of every system, or -1 for a mix).
-template <typename V, typename T, int L>
+// The block kernel for a method, value type, batch layout (every system
+// CSR, or -1: read per system) and block size.
+template <typename V, typename T, int L, int NT>
 static auto block_kernel(int method) {
-    return method == GK_CG ? k_block_cg<V, T, L> : k_block_bicgstab<V, T, L>;
+    return method == GK_CG ? k_block_cg<V, T, L, NT> : k_block_bicgstab<V, T, L, NT>;
 }
 
 template <typename V, typename T>
-static auto block_kernel(int method, int lay) {
-    switch (lay) {
-        case BL_CSR: return block_kernel<V, T, BL_CSR>(method);
-        case BL_ELL: return block_kernel<V, T, BL_ELL>(method);
-        case BL_SELLP: return block_kernel<V, T, BL_SELLP>(method);
-        default: return block_kernel<V, T, -1>(method);
-    }
+static auto block_kernel(int method, int lay, int nt) {
+    if (lay == BL_CSR)
+        return nt == 128   ? block_kernel<V, T, BL_CSR, 128>(method)
+               : nt == 256 ? block_kernel<V, T, BL_CSR, 256>(method)
+                           : block_kernel<V, T, BL_CSR, 512>(method);
+    return nt == 128   ? block_kernel<V, T, -1, 128>(method)
+           : nt == 256 ? block_kernel<V, T, -1, 256>(method)
+                       : block_kernel<V, T, -1, 512>(method);
 }
 
 template <typename V, typename T>
 static gk_status launch_block(int method, int lay, const SysDesc* ddesc, SysOut* dout,
-                              int32_t count, const BlockOpts& bo, int nt, size_t smem,
-                              unsigned grid, cudaStream_t s) {
-    auto k = block_kernel<V, T>(method, lay);
+                              int32_t count, int32_t* next, const BlockOpts& bo, int nt,
+                              size_t smem, unsigned grid, cudaStream_t s) {
+    auto k = block_kernel<V, T>(method, lay, nt);
     GK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k<<<grid, nt, smem, s>>>(ddesc, dout, count, bo);
+    k<<<grid, nt, smem, s>>>(ddesc, dout, count, next, bo);
     GK_CUDA(cudaGetLastError());
     return GK_OK;
 }
@@ -670,16 +732,24 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
         B.hcap = (size_t)count;
     }
     GK_TRY(B.desc.ensure(sizeof(SysDesc) * (size_t)count));
-    GK_TRY(B.outs.ensure(sizeof(SysOut) * (size_t)count));
+    GK_TRY(B.outs.ensure(sizeof(SysOut) * (size_t)count + 16));
     GK_TRY(B.work.ensure(wbytes + 256));
     if (pbytes) GK_TRY(B.pad.ensure(pbytes + 256));
     char* w = (char*)B.work.ptr;
     char* pw = (char*)B.pad.ptr;
     bool any_pad = false;
-    for (int32_t i = 0; i < count; ++i) {
+    std::vector<int32_t> order((size_t)count);  // the largest system first
+    for (int32_t i = 0; i < count; ++i) order[i] = i;
+    auto work = [&](int32_t i) { return As[i]->nnz + 8 * (int64_t)As[i]->n; };
+    std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
+        return work(a) != work(b) ? work(a) > work(b) : a < b;
+    });
+    for (int32_t k = 0; k < count; ++k) {
+        const int32_t i = order[k];
         gk_matrix A = As[i];
-        SysDesc& d = B.hdesc[i];
+        SysDesc& d = B.hdesc[k];
         std::memset(&d, 0, sizeof(d));
+        d.id = i;
         d.n = A->n;
         size_t pb = 0;
         d.fmt = sys_layout(A, cfg, &pb);
@@ -710,6 +780,8 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
         d.tol = o->batch_tols ? o->batch_tols[i] : o->tol;
         w += (size_t)d.ld * vb * ns;
     }
+    int32_t* next = (int32_t*)((SysOut*)B.outs.ptr + count);
+    GK_CUDA(cudaMemsetAsync(next, 0, sizeof(int32_t), s));
     GK_CUDA(cudaMemcpyAsync(B.desc.ptr, B.hdesc, sizeof(SysDesc) * (size_t)count,
                             cudaMemcpyHostToDevice, s));
     BlockOpts bo{o->tol, o->max_iters, o->precond == GK_PRECOND_JACOBI};
@@ -738,19 +810,19 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
     int lay = count > 0 ? B.hdesc[0].fmt : BL_CSR;
     for (int32_t i = 1; i < count && lay >= 0; ++i)
         if (B.hdesc[i].fmt != lay) lay = -1;
-    if (dt == GK_F64) occ = occ_of(block_kernel<double, double>(o->method, lay));
-    else if (dt == GK_F32) occ = occ_of(block_kernel<float, float>(o->method, lay));
-    else occ = occ_of(block_kernel<__nv_bfloat16, float>(o->method, lay));
+    if (dt == GK_F64) occ = occ_of(block_kernel<double, double>(o->method, lay, nt));
+    else if (dt == GK_F32) occ = occ_of(block_kernel<float, float>(o->method, lay, nt));
+    else occ = occ_of(block_kernel<__nv_bfloat16, float>(o->method, lay, nt));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(count, (int64_t)sms * occ));
     const SysDesc* dd = (const SysDesc*)B.desc.ptr;
     SysOut* dout = (SysOut*)B.outs.ptr;
     if (dt == GK_F64)
-        st = launch_block<double, double>(o->method, lay, dd, dout, count, bo, nt, smem, grid, s);
+        st = launch_block<double, double>(o->method, lay, dd, dout, count, next, bo, nt, smem, grid, s);
     else if (dt == GK_F32)
-        st = launch_block<float, float>(o->method, lay, dd, dout, count, bo, nt, smem, grid, s);
+        st = launch_block<float, float>(o->method, lay, dd, dout, count, next, bo, nt, smem, grid, s);
     else
-        st = launch_block<__nv_bfloat16, float>(o->method, lay, dd, dout, count, bo, nt, smem,
-                                                grid, s);
+        st = launch_block<__nv_bfloat16, float>(o->method, lay, dd, dout, count, next, bo, nt,
+                                                smem, grid, s);
     GK_CUDA(cudaEventRecord(e1, s));
     if (st == GK_OK) {
         GK_CUDA(cudaMemcpyAsync(B.hout, B.outs.ptr, sizeof(SysOut) * (size_t)count,
@@ -760,7 +832,8 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
         cudaEventElapsedTime(&ms, e0, e1);
         if (ms_out) *ms_out = ms;
         if (infos)
-            for (int32_t i = 0; i < count; ++i) {
+            for (int32_t k = 0; k < count; ++k) {
+                const int32_t i = B.hdesc[k].id;
                 const SysOut& so = B.hout[i];
                 infos[i].status = (gk_status)so.status;
                 infos[i].iters = so.iters;
@@ -769,11 +842,11 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
                 infos[i].rel_res_recurrence = so.rec;
                 infos[i].rel_res_true = so.tru;
                 infos[i].device_ms = ms;
-                infos[i].spmv_format = B.hdesc[i].fmt == BL_ELL     ? GK_ELL
-                                       : B.hdesc[i].fmt == BL_SELLP ? GK_SELLP
+                infos[i].spmv_format = B.hdesc[k].fmt == BL_ELL     ? GK_ELL
+                                       : B.hdesc[k].fmt == BL_SELLP ? GK_SELLP
                                                                     : GK_CSR;
                 infos[i].block_threads = nt;
-                infos[i].slice_size = B.hdesc[i].fmt == BL_SELLP ? cfg.S : 0;
+                infos[i].slice_size = B.hdesc[k].fmt == BL_SELLP ? cfg.S : 0;
             }
     }
     cudaEventDestroy(e0);
@@ -809,8 +882,8 @@ gk_status solve_small(gk_matrix A, const void* b, void* x, const gk_solve_opts* 
 // ------------------------------------------------------------ autotuner
 // The configuration of a batch shape -- each system's SpMV layout (policy
 // CSR, ELL where its padding is at most 20 %, or SELL-P with slices of
-// S = 8, 16 or 32 rows) and the threads per block (128, 256, 512, which set
-// how many rows a warp and a thread take per sweep) -- is picked by timing
+// S = 8, 16 or 32 rows) and, for small systems (see WIDE_BLOCK_ROWS), the
+// threads per block (256 or 512) -- is picked by timing
 // every candidate on a run of the batch itself capped at 30 iterations (the
 // callers' initial guesses are saved before and restored after the trials)
 // and cached per key: value type, method, preconditioner, log2 of the
@@ -855,8 +928,11 @@ static gk_status autotune(int32_t count, const gk_matrix* As, const void* const*
     float best_ms = 1e30f;
     *best = BatchCfg();
     const int layouts[5][2] = {{BL_CSR, 0}, {BL_ELL, 0}, {BL_SELLP, 8}, {BL_SELLP, 16}, {BL_SELLP, 32}};
+    int32_t nmax = 0;
+    for (int32_t i = 0; i < count; ++i) nmax = std::max(nmax, As[i]->n);
     for (const auto& L : layouts)
-        for (int nt : {128, 256, 512}) {
+        for (int nt : {256, 512}) {
+            if (nt == 256 && nmax > WIDE_BLOCK_ROWS) continue;
             BatchCfg c;
             c.layout = L[0];
             c.S = L[0] == BL_SELLP ? L[1] : 32;
@@ -922,7 +998,10 @@ extern "C" gk_status gk_solve_batched(int32_t count, const gk_matrix* As, const 
         if (A->device != dev) return GK_ERR_UNSUPPORTED;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    BatchCfg cfg;  // untuned default: CSR, 256 threads
+    int32_t nmax = 0;
+    for (int32_t i = 0; i < count; ++i) nmax = std::max(nmax, As[i]->n);
+    BatchCfg cfg;  // untuned default: CSR
+    cfg.nt = nmax > WIDE_BLOCK_ROWS ? 512 : 256;
     int nt = 0;
     if (const char* e = getenv("GK_BATCH_THREADS")) nt = atoi(e);
     const bool fnt = nt == 128 || nt == 256 || nt == 512;
@@ -933,8 +1012,6 @@ extern "C" gk_status gk_solve_batched(int32_t count, const gk_matrix* As, const 
     // loop's varying small batches, each a new shape, lost ~20 % of their
     // throughput to them: 81 against 100 solves/s at saturation)
     if (!(fnt && flay) && !(at && at[0] == '0') && count >= TUNE_MIN_COUNT) {
-        int32_t nmax = 0;
-        for (int32_t i = 0; i < count; ++i) nmax = std::max(nmax, As[i]->n);
         const uint64_t key = tune_key(As[0]->dtype, o, nmax, count);
         bool found = false;
         BatchCfg tuned;
