@@ -121,7 +121,8 @@ typedef struct {
     int32_t num_slices;    /* SELL-P: ceil(n / S) */
     int64_t stored;        /* entries held in col/values incl. padding */
     int64_t device_bytes;  /* bytes of the format arrays on the device */
-    int32_t spmv_kernel;   /* SpMV kernel apply uses: 0 CSR vector, 1 CSR row-tile,
+    int32_t spmv_kernel;   /* SpMV kernel apply uses: 0 CSR vector (or one row per
+                              thread), 1 CSR row-tile,
                               2 CSR segmented, 3 ELL, 4 SELL-P, 5 COO,
                               6 CSR warp-tile */
     int32_t spmv_launches; /* kernel launches per apply */

@@ -50,7 +50,7 @@ static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double bet
         GK_CUDA(cudaGetLastError());
         return GK_OK;
     }
-    if (A->fmt == GK_CSR && A->plan.kind == 2) {
+    if (A->fmt == GK_CSR && A->plan.seg) {
         const int64_t units = A->plan.units;
         if (units > 0) {
             GK_TRY(A->carry.ensure((size_t)units * (sizeof(int32_t) + sizeof(T)) + 16));
@@ -58,9 +58,13 @@ static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double bet
             T* cval = reinterpret_cast<T*>(static_cast<char*>(A->carry.ptr) +
                                            (((size_t)units * sizeof(int32_t) + 15) & ~(size_t)15));
             const int32_t* row_end = A->plan.row_end ? A->plan.row_end : A->row_ptr + 1;
-            k_csr_seg<V, T><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(
-                A->nnz, units, row_end, A->plan.row_id, A->plan.unit_row, A->col,
-                (const V*)A->val, static_cast<const T*>(b), epi, crow, cval);
+            auto seg = [&](auto kern) {
+                kern<<<(unsigned)((units + 7) / 8), 256, 0, s>>>(
+                    A->nnz, units, row_end, A->plan.row_id, A->plan.unit_row, A->col,
+                    (const V*)A->val, static_cast<const T*>(b), epi, crow, cval);
+            };
+            if (A->plan.local_cols) seg(k_csr_seg<true, V, T>);
+            else seg(k_csr_seg<false, V, T>);
             const unsigned fg =
                 (unsigned)std::max<int64_t>(1, std::min<int64_t>((units + 255) / 256, 4096));
             k_carry_fixup<T><<<fg, 256, 0, s>>>((int32_t)units, crow, cval, static_cast<T*>(x),

@@ -163,7 +163,9 @@ constexpr int WT_SMEM_CAP = 208 * 1024;  // largest ring of one warp-tile block 
                                          // epilogues' static shared memory fits beside it)
 
 struct CsrPlan {
-    int kind = 0;            // 0 vector (G lanes / row), 1 row-tile, 2 segmented, 3 warp-tile
+    int kind = 0;            // fused row epilogues: 0, 2 vector (G lanes / row), 1 row-tile,
+                             // 3 warp-tile
+    int seg = 0;             // gk_apply runs the segmented kernel instead
     int lanes = 1;           // vector kernel lanes per row
     int32_t ntiles = 0;
     int32_t chunk = 0;       // nnz per chunk used to cut tiles
@@ -179,6 +181,7 @@ struct CsrPlan {
     int32_t* row_id = nullptr;
     int32_t* empty_rows = nullptr;
     int32_t n_empty = 0;
+    int32_t local_cols = 0;  // the units' columns lie close together
     int32_t* err = nullptr;  // device word set by a kernel whose bounded wait ran out
 };
 

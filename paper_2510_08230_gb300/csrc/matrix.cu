@@ -489,6 +489,24 @@ __global__ void k_unit_rows(int32_t m, const int32_t* __restrict__ row_end, int3
     }
 }
 
+// Counts the sampled units (every step-th) whose columns span at most
+// `span`.  One warp per unit.
+__global__ void k_unit_span(int64_t nnz, int32_t nunits, int32_t step, int32_t span,
+                            const int32_t* __restrict__ ci, int32_t* __restrict__ count) {
+    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t u = w * step;
+    if (u >= nunits) return;
+    int32_t lo = INT32_MAX, hi = 0;
+    for (int64_t k = u * SEG_UNIT + lane; k < min((u + 1) * (int64_t)SEG_UNIT, nnz); k += 32) {
+        lo = min(lo, ci[k]);
+        hi = max(hi, ci[k]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0 && hi - lo <= span) atomicAdd(count, 1);
+}
+
 __global__ void k_nonempty_flags(int32_t n, const int32_t* __restrict__ rp,
                                  int32_t* __restrict__ flag) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -630,6 +648,10 @@ static gk_status build_coo_view(gk_matrix A, cudaStream_t s) {
     return GK_OK;
 }
 
+// A segmented unit whose columns span at most this much of x counts as local
+// (the L1 that the kernel's shared memory leaves is about 100 KB).
+constexpr int64_t LOCAL_COLS_BYTES = 64 * 1024;
+
 // CSR launch plan: row tiles when rows are short, the segmented kernel otherwise.
 gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
     CsrPlan& P = A->plan;
@@ -674,13 +696,47 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
         return (int64_t)WT_WARPS * (((int64_t)nst * wt_cap * (4 + vb) + 8 * nst + 127) & ~(int64_t)127);
     };
     const bool wt_fits = wt_block_bytes(wt_nst) <= WT_SMEM_CAP;
+    // The kernel of the fused row epilogues (solver) and, unless P.seg, of
+    // gk_apply: 3 warp tiles for short rows of near-uniform length, else 1 row
+    // tiles, else (kind 2: longer than 1024) the vector kernel.
     int kind = (A->max_row <= 1024) ? 1 : 2;
     if (wt_fits && wt_block_bytes(wt_nst) <= 112 * 1024 && A->max_row <= 2.0 * mean + 1.0)
         kind = 3;
-    if (const char* force = getenv("GK_CSR_KERNEL")) kind = atoi(force);
+    // gk_apply runs the segmented kernel wherever warp tiles do not apply.
+    // Against row tiles (us, FP64 / FP32; n x mean length, exponential
+    // lengths, columns within 2000 of the diagonal): 200,000 x 4: 17.6 / 7.0
+    // row tiles, 10.1 / 7.9 segmented; x 16: 70.6 / 26.7, 17.9 / 12.6; 2M x 8:
+    // 190 / 75, 71 / 47; 4,000 rows of Zipf lengths: 151 / 39, 6.2 / 5.6.
+    P.seg = kind != 3;
+    // Small matrices, where a launch is latency: kernels that neither stage
+    // nor carry.  Rows of at most 16 entries: one row per thread while one
+    // wave of its blocks holds them all (us, FP64 / FP32, against warp tiles:
+    // 4,096 rows 2.1 / 1.9 and 3.3 / 2.4, 62,500 2.9 / 2.3 and 3.5 / 2.6; past
+    // the wave 90,000 4.3 / 3.1 and 4.6 / 2.7).  Longer rows: the vector
+    // kernel up to where the other kernel catches up (n x lanes): against warp
+    // tiles FP64 10,000 x 32: 5.7 / 6.1 but 30,000 x 16: 7.0 / 4.1, FP32
+    // 3,000 x 32: 1.9 / 3.4 but 30,000 x 16: 2.9 / 2.7; against the segmented
+    // kernel FP64 30,000 x 8: 5.8 / 7.4, x 16: 9.3 / 8.8, FP32 30,000 x 32:
+    // 6.4 / 8.5, 200,000 x 8: 10.4 / 8.8.  A longest row of more than 24
+    // steps waits too long (4,000 Zipf rows: 16.5 / 6.2).
+    const int64_t threads = (int64_t)A->n * lanes;
+    const int64_t line = vb == 8 ? (P.seg ? 320 : 160) : (P.seg ? 1024 : 256);
+    if (A->max_row <= 16 ? A->n <= (int64_t)ROW_THREADS * 8 * num_sms()
+                         : threads <= line * 1024 && A->max_row <= 24 * lanes) {
+        kind = 0;
+        P.seg = 0;
+        if (A->max_row <= 16) P.lanes = 1;
+    }
+    if (const char* force = getenv("GK_CSR_KERNEL")) {
+        kind = atoi(force);
+        P.seg = kind == 2;
+    }
     if (kind == 3 && !wt_fits) kind = 1;
     // a single staged tile must fit in shared memory
-    if (kind == 1 && ((cap + 7) & ~7) * (int64_t)(4 + value_bytes(A->dtype)) > 200 * 1024) kind = 2;
+    if (kind == 1 && ((cap + 7) & ~7) * (int64_t)(4 + value_bytes(A->dtype)) > 200 * 1024) {
+        kind = 2;
+        P.seg = 1;
+    }
     P.kind = kind;
     P.stages = 1;
     if (const char* e = getenv("GK_ROWTILE_STAGES")) P.stages = std::max(1, std::min(3, atoi(e)));
@@ -696,7 +752,8 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
         k_tile_desc<<<grid_for(P.ntiles), 256, 0, s>>>(A->n, A->row_ptr, chunk, P.ntiles,
                                                        P.tile_desc);
         GK_CUDA(cudaGetLastError());
-    } else if (kind == 2) {
+    }
+    if (P.seg) {
         // units of SEG_UNIT nonzeros over the nonempty rows
         P.units = (int32_t)((A->nnz + SEG_UNIT - 1) / SEG_UNIT);
         TmpBuf flag, rank, tmp;
@@ -720,6 +777,22 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
                 GK_CUDA(cudaStreamSynchronize(s));  // the scratch goes
             }
         }
+        // gathers through L1 when most units' columns fit a part of it
+        if (P.units > 0) {
+            const int32_t step = std::max(1, P.units / 4096);
+            const int32_t sampled = (P.units + step - 1) / step;
+            TmpBuf cnt;
+            GK_TRY(cnt.ensure(4));
+            GK_CUDA(cudaMemsetAsync(cnt.ptr, 0, 4, s));
+            k_unit_span<<<(unsigned)((sampled + 7) / 8), 256, 0, s>>>(
+                A->nnz, P.units, step, (int32_t)(LOCAL_COLS_BYTES / vector_bytes(A->dtype)), A->col,
+                (int32_t*)cnt.ptr);
+            int32_t close = 0;
+            GK_CUDA(cudaMemcpyAsync(&close, cnt.ptr, 4, cudaMemcpyDeviceToHost, s));
+            GK_CUDA(cudaStreamSynchronize(s));
+            P.local_cols = 2 * close > sampled;
+        }
+        GK_TRY(A->carry.ensure((size_t)P.units * (4 + vector_bytes(A->dtype)) + 16));
         GK_CUDA(dmalloc_t(&P.unit_row, (size_t)P.units + 1));
         k_unit_rows<<<grid_for(P.units + 1), 256, 0, s>>>(
             m, P.row_end ? P.row_end : A->row_ptr + 1, P.units, P.unit_row);
@@ -1089,7 +1162,7 @@ gk_status gk_matrix_describe(gk_matrix A, gk_matrix_desc* d) {
     d->stride_factor = A->f;
     d->num_slices = A->nslices;
     d->spmv_kernel = A->coo ? 5
-                     : A->fmt == GK_CSR ? (A->plan.kind == 3 ? 6 : A->plan.kind)
+                     : A->fmt == GK_CSR ? (A->plan.seg ? 2 : A->plan.kind == 3 ? 6 : A->plan.kind)
                      : A->fmt == GK_ELL ? 3 : 4;
     if (A->plan.err) {
         int32_t e = 0;
@@ -1107,7 +1180,7 @@ gk_status gk_matrix_describe(gk_matrix A, gk_matrix_desc* d) {
             d->device_error |= 2 << k;
     }
     d->spmv_launches = A->coo ? (A->n_empty ? 3 : 2)
-                       : (A->fmt == GK_CSR && A->plan.kind == 2) ? (A->plan.n_empty ? 3 : 2) : 1;
+                       : (A->fmt == GK_CSR && A->plan.seg) ? (A->plan.n_empty ? 3 : 2) : 1;
     d->solve_format = A->fmt != GK_CSR ? (int32_t)A->fmt
                       : !A->solve_fmt_tuned ? -1
                       : A->solve_fmt ? (int32_t)A->solve_fmt->fmt : (int32_t)GK_CSR;

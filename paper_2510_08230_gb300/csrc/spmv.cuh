@@ -574,7 +574,14 @@ __device__ __forceinline__ void load8(const H* p, H (&v)[8]) {
     for (int k = 0; k < 8; ++k) v[k] = q.e[k];
 }
 
-template <typename V, typename T>
+// L1: gather x through L1 (the plan found that units' columns lie close
+// together, so neighbouring rows share lines), else through L2 only.
+template <bool L1, typename T>
+__device__ __forceinline__ T gather_x(const T* p) {
+    return L1 ? __ldg(p) : __ldcg(p);
+}
+
+template <bool L1, typename V, typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 5 : 6)
 k_csr_seg(int64_t nnz, int64_t nunits, const int32_t* __restrict__ row_end,
           const int32_t* __restrict__ row_id, const int32_t* __restrict__ unit_row,
@@ -612,14 +619,13 @@ k_csr_seg(int64_t nnz, int64_t nunits, const int32_t* __restrict__ row_end,
     __syncwarp();
     for (int q = lane; q < nrow; q += 32)
         mark[(int64_t)__ldg(row_end + i0 + q) - 1 - k0] = (int16_t)q;
-    // x at skewed matrices' columns reuses little in L1: through L2 only
     if (k0 + SEG_UNIT <= nnz) {
 #pragma unroll
-        for (int k = 0; k < E; ++k) xv[k] = __ldcg(x + c[k]);
+        for (int k = 0; k < E; ++k) xv[k] = gather_x<L1>(x + c[k]);
         if constexpr (sizeof(T) != 8) load8(va + kl, v);
     } else {
 #pragma unroll
-        for (int k = 0; k < E; ++k) xv[k] = kl + k < nnz ? __ldcg(x + c[k]) : T(0);
+        for (int k = 0; k < E; ++k) xv[k] = kl + k < nnz ? gather_x<L1>(x + c[k]) : T(0);
     }
     __syncwarp();
     const int4 mq = reinterpret_cast<const int4*>(mark)[lane];
@@ -818,6 +824,40 @@ k_csr_vector(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restric
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, G);
         if (gl == 0 && r < n) epi.row(r, s, acc.v);
+    }
+    epi.finish(acc.v);
+}
+
+// CSR, one row per thread (lanes = 1): small matrices of short rows, where a
+// launch is latency only.  Entries are read straight from global memory, four
+// at a time before their FMAs, in CSR order: the sums of the tile kernels.
+// Blocks of 64 threads spread a few thousand rows over many SMs.
+constexpr int ROW_THREADS = 64;
+
+template <typename V, typename T, class Epi>
+__global__ void __launch_bounds__(ROW_THREADS)
+k_csr_row(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+          const V* __restrict__ va, const T* __restrict__ x, Epi epi) {
+    if (epi.skip()) return;
+    AccArr<Epi> acc{};
+    for (int64_t r = blockIdx.x * (int64_t)ROW_THREADS + threadIdx.x; r < n;
+         r += (int64_t)gridDim.x * ROW_THREADS) {
+        int32_t k = __ldg(rp + r);
+        const int32_t e = __ldg(rp + r + 1);
+        T s = T(0);
+        for (; k < e; k += 4) {
+            T v[4], xv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k + u < e) {
+                    v[u] = ldv(va + k + u);
+                    xv[u] = __ldg(x + __ldg(ci + k + u));
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k + u < e) s = fmadd(v[u], xv[u], s);
+        }
+        epi.row(r, s, acc.v);
     }
     epi.finish(acc.v);
 }
@@ -1124,7 +1164,12 @@ gk_status launch_spmv_rows(gk_matrix A, const T* x, const Epi& epi, cudaStream_t
         const int32_t n = A->n;
         const V* va = (const V*)A->val;
         switch (G) {
-            case 1: k_csr_vector<1, V, T, Epi><<<grid, 256, 0, s>>>(n, A->row_ptr, A->col, va, x, epi); break;
+            case 1:
+                grid = (unsigned)std::max<int64_t>(
+                    1, std::min<int64_t>(((int64_t)n + ROW_THREADS - 1) / ROW_THREADS,
+                                         (int64_t)sms * 8));
+                k_csr_row<V, T, Epi><<<grid, ROW_THREADS, 0, s>>>(n, A->row_ptr, A->col, va, x, epi);
+                break;
             case 2: k_csr_vector<2, V, T, Epi><<<grid, 256, 0, s>>>(n, A->row_ptr, A->col, va, x, epi); break;
             case 4: k_csr_vector<4, V, T, Epi><<<grid, 256, 0, s>>>(n, A->row_ptr, A->col, va, x, epi); break;
             case 8: k_csr_vector<8, V, T, Epi><<<grid, 256, 0, s>>>(n, A->row_ptr, A->col, va, x, epi); break;

@@ -305,3 +305,38 @@ def test_segmented_units(name, dtype):
         hit[rows[m.col_idx == m.col_idx[0]]] = True
         assert np.array_equal(~np.isfinite(_run(A, xb, 1.0, 0.0, None, dtype)), hit)
     A.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16", "f16"])
+@pytest.mark.parametrize("name,kernel", [("rows_of_16", 0), ("rows_of_17", 0), ("one_wave", 0),
+                                         ("past_one_wave", 6), ("skewed_small", 2),
+                                         ("short_and_empty", 0)])
+def test_small_matrix_kernels(name, kernel, dtype):
+    """The automatic choice on both sides of its lines: one row per thread
+    (rows of at most 16 entries, one wave of blocks), vector, segmented; and
+    the same product inside a captured graph on the first call."""
+    import torch
+    wave = 64 * 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(4)
+    lengths = {"rows_of_16": [16] * 501, "rows_of_17": [17] * 501,
+               "one_wave": None, "past_one_wave": None,
+               "skewed_small": [3] * 3000 + [900], "short_and_empty": rng.integers(0, 9, 333)}[name]
+    m = _rows_of(lengths, 4096, 9) if lengths is not None else W.laplacian_1d(
+        wave if name == "one_wave" else wave + 1)
+    A = gk.Matrix.from_csr(m, dtype)
+    assert A.desc["spmv_kernel"] == kernel
+    x = rng.uniform(-1, 1, m.ncols)
+    xt = torch.from_numpy(x).to(torch_dev(), vec_dtype(dtype))
+    yt = torch.full((m.n,), float("nan"), dtype=vec_dtype(dtype), device=xt.device)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        A.apply(xt, yt)
+    graph.replay()
+    torch.cuda.synchronize()
+    ref, scale = oracle_apply(m, x, 1.0, 0.0, None, dtype)
+    assert_rows_close(yt.cpu().numpy(), ref, scale, TOL[dtype], f"{name} {dtype}")
+    y0 = rng.uniform(-1, 1, m.n)
+    y = _run(A, x, -0.5, 2.0, y0, dtype)
+    ref, scale = oracle_apply(m, x, -0.5, 2.0, y0, dtype)
+    assert_rows_close(y, ref, scale, TOL[dtype], f"{name} {dtype} adv")
+    A.close()
