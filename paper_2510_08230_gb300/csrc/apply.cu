@@ -53,9 +53,8 @@ static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double bet
     if (A->fmt == GK_CSR && A->plan.seg) {
         const int64_t units = A->plan.units;
         if (units > 0) {
-            GK_TRY(A->carry.ensure((size_t)units * (sizeof(int32_t) + sizeof(T)) + 16));
-            int32_t* crow = static_cast<int32_t*>(A->carry.ptr);
-            T* cval = reinterpret_cast<T*>(static_cast<char*>(A->carry.ptr) +
+            int32_t* crow = static_cast<int32_t*>(A->plan.carries);
+            T* cval = reinterpret_cast<T*>(static_cast<char*>(A->plan.carries) +
                                            (((size_t)units * sizeof(int32_t) + 15) & ~(size_t)15));
             const int32_t* row_end = A->plan.row_end ? A->plan.row_end : A->row_ptr + 1;
             auto seg = [&](auto kern) {

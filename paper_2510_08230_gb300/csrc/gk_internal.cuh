@@ -176,13 +176,15 @@ struct CsrPlan {
     int4* tile_desc = nullptr;
     int32_t wt_rpl = 2;      // warp-tile: rows per lane (tiles of 32 * wt_rpl rows)
     int32_t units = 0;
-    int32_t* unit_row = nullptr;
+    int32_t* unit_row = nullptr;  // the carries of the units follow it in one allocation
+    void* carries = nullptr;
     int32_t* row_end = nullptr;
     int32_t* row_id = nullptr;
     int32_t* empty_rows = nullptr;
     int32_t n_empty = 0;
     int32_t local_cols = 0;  // the units' columns lie close together
     int32_t* err = nullptr;  // device word set by a kernel whose bounded wait ran out
+                             // (the first of the handle's words)
 };
 
 struct SolverCache;  // solve.cu
@@ -263,6 +265,8 @@ struct gk_matrix_s {
     int32_t* row_ptr = nullptr;
     int32_t* col = nullptr;
     void* val = nullptr;
+    void* slab = nullptr;           // one allocation behind row_ptr, col, val and words
+    int32_t* words = nullptr;       // 64 device words: plan.err, then scratch of the set-up
     // COO view (apply runs the COO kernel; fmt stays GK_CSR for everything else)
     int coo = 0;
     int32_t* coo_row = nullptr;     // row of every entry
@@ -293,7 +297,7 @@ struct gk_matrix_s {
     int solve_fmt_tuned = 0;
     gk::SolverCache* solver = nullptr;
     gk::DevBuf stage_in, stage_out;  // host-pointer apply staging
-    gk::DevBuf carry;                // merge-path block carries
+    gk::DevBuf carry;                // COO unit carries
     cudaStream_t side = nullptr;     // library streams for graph capture (the second
     cudaStream_t side2 = nullptr;    // captures the body of a solve's loop)
     uint64_t wait_ns = 2000000000ull;  // budget of the row-tile kernel's waits (a solve's

@@ -7,7 +7,8 @@
 // scatter (row, col, input position) keys into row buckets in any order,
 // sort each bucket by (col, input position) - a total order, so the result
 // does not depend on the scatter order - then merge equal columns left to
-// right.
+// right.  Sorting goes by classes of row length, merging by entries, so that
+// neither waits for one long row.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -147,9 +148,11 @@ __global__ void k_validate_cols(int64_t nnz, int32_t ncols, const int32_t* __res
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(err, 8u);
 }
 
+// Counts the entries of every row; rank[k] = entry k's place among its row's
+// in arrival order (any order: the rows are sorted).
 __global__ void k_coo_count(int64_t nnz, int32_t n, int32_t ncols, const int32_t* __restrict__ row,
                             const int32_t* __restrict__ col, int32_t* __restrict__ cnt,
-                            unsigned int* err) {
+                            int32_t* __restrict__ rank, unsigned int* err) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nnz;
          k += (int64_t)gridDim.x * blockDim.x) {
         int32_t r = row[k], c = col[k];
@@ -157,39 +160,89 @@ __global__ void k_coo_count(int64_t nnz, int32_t n, int32_t ncols, const int32_t
             atomicOr(err, 8u);
             continue;
         }
-        atomicAdd(cnt + r, 1);
+        rank[k] = atomicAdd(cnt + r, 1);
     }
 }
 
 __global__ void k_coo_scatter(int64_t nnz, const int32_t* __restrict__ row,
-                              const int32_t* __restrict__ col, const int64_t* __restrict__ start,
-                              int32_t* __restrict__ cursor, uint64_t* __restrict__ keys) {
+                              const int32_t* __restrict__ col, const int32_t* __restrict__ start,
+                              const int32_t* __restrict__ rank, uint64_t* __restrict__ keys) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nnz;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        int32_t r = row[k];
-        int64_t pos = start[r] + atomicAdd(cursor + r, 1);
-        keys[pos] = ((uint64_t)(uint32_t)col[k] << 32) | (uint64_t)(uint32_t)k;
-    }
+         k += (int64_t)gridDim.x * blockDim.x)
+        keys[start[row[k]] + rank[k]] = ((uint64_t)(uint32_t)col[k] << 32) | (uint64_t)(uint32_t)k;
 }
 
-// Sort rows of length in (W/2, W] (W <= 32) with W-lane bitonic networks.
+// Rows are sorted by classes of length, each with its own kernel and list of
+// rows (a kernel that visits every row to find its own spends most of its
+// lanes on others'): classes 0 to 8 hold lengths 2, ..4, ..8, up to ..512 (a
+// group of 2 to 32 lanes, then a warp with 2 to 16 keys a lane), 9 lengths to
+// SORT_BLOCK_MAX (a block), 10 longer ones.  Rows of one entry need none.
+constexpr int SORT_CLASSES = 11;
+constexpr int SORT_BLOCK_MAX = 16384;  // keys in shared memory (128 KB)
+
+__device__ __forceinline__ int sort_class(int32_t L) {
+    if (L < 2) return -1;
+    if (L > 512) return L <= SORT_BLOCK_MAX ? 9 : 10;
+    return 31 - __clz(L - 1);  // 2: 0, 3-4: 1, 5-8: 2, ... 257-512: 8
+}
+
+// Sizes of the classes and the longest row ({sizes, longest} in `out`).
+__global__ void k_class_sizes(int32_t n, const int32_t* __restrict__ cnt, int32_t* __restrict__ out) {
+    __shared__ int32_t sz[SORT_CLASSES + 1];
+    if (threadIdx.x <= SORT_CLASSES) sz[threadIdx.x] = 0;
+    __syncthreads();
+    int32_t longest = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t L = cnt[i];
+        const int c = sort_class(L);
+        if (c >= 0) atomicAdd(sz + c, 1);
+        longest = max(longest, L);
+    }
+    atomicMax(sz + SORT_CLASSES, longest);
+    __syncthreads();
+    if (threadIdx.x < SORT_CLASSES && sz[threadIdx.x]) atomicAdd(out + threadIdx.x, sz[threadIdx.x]);
+    if (threadIdx.x == SORT_CLASSES) atomicMax(out + SORT_CLASSES, sz[SORT_CLASSES]);
+}
+
+struct ClassOffsets {
+    int32_t o[SORT_CLASSES];
+};
+
+// Lists the rows of every class (in any order) from off.o[class] on.
+__global__ void k_class_lists(int32_t n, const int32_t* __restrict__ cnt, ClassOffsets off,
+                              int32_t* __restrict__ cursor, int32_t* __restrict__ list) {
+    __shared__ int32_t sz[SORT_CLASSES], base[SORT_CLASSES];
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (threadIdx.x < SORT_CLASSES) sz[threadIdx.x] = 0;
+    __syncthreads();
+    const int c = i < n ? sort_class(cnt[i]) : -1;
+    const int32_t at = c >= 0 ? atomicAdd(sz + c, 1) : 0;
+    __syncthreads();
+    if (threadIdx.x < SORT_CLASSES && sz[threadIdx.x])
+        base[threadIdx.x] = off.o[threadIdx.x] + atomicAdd(cursor + threadIdx.x, sz[threadIdx.x]);
+    __syncthreads();
+    if (c >= 0) list[base[c] + at] = (int32_t)i;
+}
+
+// Rows of length in (W/2, W] (W <= 32): W-lane bitonic networks.
 template <int W>
-__global__ void k_sort_rows_sub(int32_t n, const int64_t* __restrict__ start,
-                                uint64_t* __restrict__ keys) {
+__global__ void k_sort_rows_sub(int32_t m, const int32_t* __restrict__ list,
+                                const int32_t* __restrict__ start, uint64_t* __restrict__ keys) {
     const int lane = threadIdx.x & (W - 1);
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / W;
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / W;
     // the loop trip count is uniform across the warp (groups advance together)
     const int64_t warp_first = g - (threadIdx.x & 31) / W;
-    for (int64_t base = warp_first; base < n; base += ng) {
-        const int64_t r = base + (threadIdx.x & 31) / W;
-        int64_t a = 0, L = 0;
-        if (r < n) {
+    for (int64_t base = warp_first; base < m; base += ng) {
+        const int64_t q = base + (threadIdx.x & 31) / W;
+        int32_t a = 0, L = 0;
+        if (q < m) {
+            const int32_t r = list[q];
             a = start[r];
             L = start[r + 1] - a;
         }
-        const bool mine = (L > W / 2) && (L <= W);
-        uint64_t v = (mine && lane < L) ? keys[a + lane] : ~0ull;
+        uint64_t v = lane < L ? keys[a + lane] : ~0ull;
 #pragma unroll
         for (int k = 2; k <= W; k <<= 1) {
 #pragma unroll
@@ -201,53 +254,141 @@ __global__ void k_sort_rows_sub(int32_t n, const int64_t* __restrict__ start,
                 v = (lower == up) ? mn : mx;
             }
         }
-        if (mine && lane < L) keys[a + lane] = v;
+        if (lane < L) keys[a + lane] = v;
     }
 }
 
-// Sort rows of length in (lo, hi] with one block per row, keys padded to a
-// power of two in shared memory (dynamic smem of cap keys).
-__global__ void k_sort_rows_block(int32_t n, const int64_t* __restrict__ start,
-                                  uint64_t* __restrict__ keys, int64_t lo, int64_t hi, int cap) {
+// Bitonic exchanges of 32 E keys in a warp's registers, key i in register
+// i / 32 of lane i mod 32: those over 32 and more places stay in a lane.
+// One step of distance j of the merge of size k; `down`: the order of keys
+// whose bit k is clear is descending.
+template <int E>
+__device__ __forceinline__ void bitonic_step(uint64_t (&v)[E], int k, int j, bool down) {
+    const int lane = threadIdx.x & 31;
+    if (j >= 32) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int f = e ^ (j >> 5);
+            if (f > e) {
+                const bool up = (((e << 5) & k) == 0) != down;
+                const uint64_t x = v[e], y = v[f];
+                const bool swap = (x > y) == up;
+                v[e] = swap ? y : x;
+                v[f] = swap ? x : y;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const uint64_t o = __shfl_xor_sync(0xffffffffu, v[e], j);
+            const bool up = ((((e << 5) | lane) & k) == 0) != down;
+            const bool lower = (lane & j) == 0;
+            v[e] = (lower == up) == (v[e] < o) ? v[e] : o;
+        }
+    }
+}
+
+// Sorts the 32 E keys, ascending or (last_down) descending.
+template <int E>
+__device__ __forceinline__ void bitonic_sort(uint64_t (&v)[E], bool last_down) {
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) bitonic_step<E>(v, k, j, k == 32 * E && last_down);
+}
+
+// The steps of distance 16 E and less of a merge larger than the keys.
+template <int E>
+__device__ __forceinline__ void bitonic_merge(uint64_t (&v)[E], bool down) {
+#pragma unroll
+    for (int j = 16 * E; j > 0; j >>= 1) bitonic_step<E>(v, 0, j, down);
+}
+
+// Rows of length in (16 E, 32 E]: one warp each.
+template <int E>
+__global__ void __launch_bounds__(128)
+k_sort_rows_warp(int32_t m, const int32_t* __restrict__ list, const int32_t* __restrict__ start,
+                 uint64_t* __restrict__ keys) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < m;
+         q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int32_t r = list[q], a = start[r], L = start[r + 1] - a;
+        uint64_t v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = e * 32 + lane < L ? keys[a + e * 32 + lane] : ~0ull;
+        bitonic_sort<E>(v, false);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (e * 32 + lane < L) keys[a + e * 32 + lane] = v[e];
+    }
+}
+
+// Longer rows: one block per row, keys padded to a power of two P in shared
+// memory.  Each warp sorts chunks of 512 keys in its registers; of the merge
+// steps only the exchanges over 512 and more places go through shared memory
+// with a block barrier each (6 of the 78 steps of 4096 keys), the rest of
+// every merge runs chunk by chunk in registers again.  2,500 rows of 513 to
+// 4096 entries: 215 us, 425 with every step in shared memory.
+constexpr int CHUNK_E = 16, CHUNK = 32 * CHUNK_E;
+
+__global__ void __launch_bounds__(256)
+k_sort_rows_block(int32_t m, const int32_t* __restrict__ list, const int32_t* __restrict__ start,
+                  uint64_t* __restrict__ keys) {
     extern __shared__ uint64_t sk[];
-    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
-        const int64_t a = start[r], L = start[r + 1] - a;
-        if (L <= lo || L > hi) continue;
-        int P = 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int64_t q = blockIdx.x; q < m; q += gridDim.x) {
+        const int32_t r = list[q], a = start[r], L = start[r + 1] - a;
+        int P = CHUNK;
         while (P < L) P <<= 1;
-        for (int i = threadIdx.x; i < P; i += blockDim.x) sk[i] = i < L ? keys[a + i] : ~0ull;
+        for (int base = warp * CHUNK; base < P; base += nw * CHUNK) {
+            uint64_t v[CHUNK_E];
+#pragma unroll
+            for (int e = 0; e < CHUNK_E; ++e) {
+                const int i = base + e * 32 + lane;
+                v[e] = i < L ? keys[a + i] : ~0ull;
+            }
+            bitonic_sort<CHUNK_E>(v, (base & CHUNK) != 0);
+#pragma unroll
+            for (int e = 0; e < CHUNK_E; ++e) sk[base + e * 32 + lane] = v[e];
+        }
         __syncthreads();
-        for (int k = 2; k <= P; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < P; i += blockDim.x) {
-                    int p = i ^ j;
-                    if (p > i) {
-                        bool up = ((i & k) == 0);
-                        uint64_t x = sk[i], y = sk[p];
-                        if ((x > y) == up) {
-                            sk[i] = y;
-                            sk[p] = x;
-                        }
+        for (int k = 2 * CHUNK; k <= P; k <<= 1) {
+            for (int j = k >> 1; j >= CHUNK; j >>= 1) {
+                for (int t = threadIdx.x; t < P / 2; t += blockDim.x) {
+                    const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), p = i | j;
+                    const bool up = (i & k) == 0;
+                    const uint64_t x = sk[i], y = sk[p];
+                    if ((x > y) == up) {
+                        sk[i] = y;
+                        sk[p] = x;
                     }
                 }
                 __syncthreads();
             }
+            for (int base = warp * CHUNK; base < P; base += nw * CHUNK) {
+                uint64_t v[CHUNK_E];
+#pragma unroll
+                for (int e = 0; e < CHUNK_E; ++e) v[e] = sk[base + e * 32 + lane];
+                bitonic_merge<CHUNK_E>(v, (base & k) != 0);
+#pragma unroll
+                for (int e = 0; e < CHUNK_E; ++e) sk[base + e * 32 + lane] = v[e];
+            }
+            __syncthreads();
         }
         for (int i = threadIdx.x; i < L; i += blockDim.x) keys[a + i] = sk[i];
         __syncthreads();
-        (void)cap;
     }
 }
 
 // Rows longer than the shared-memory sorter: bitonic sort in a global
 // scratch area of P keys per block.
-__global__ void k_sort_rows_global(int32_t n, const int64_t* __restrict__ start,
-                                   uint64_t* __restrict__ keys, int64_t lo,
+__global__ void k_sort_rows_global(int32_t m, const int32_t* __restrict__ list,
+                                   const int32_t* __restrict__ start, uint64_t* __restrict__ keys,
                                    uint64_t* __restrict__ scratch, int64_t P) {
     uint64_t* sk = scratch + (int64_t)blockIdx.x * P;
-    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
+    for (int64_t row = blockIdx.x; row < m; row += gridDim.x) {
+        const int32_t r = list[row];
         const int64_t a = start[r], L = start[r + 1] - a;
-        if (L <= lo) continue;
         int64_t Q = 1;
         while (Q < L) Q <<= 1;
         for (int64_t i = threadIdx.x; i < Q; i += blockDim.x) sk[i] = i < L ? keys[a + i] : ~0ull;
@@ -273,53 +414,98 @@ __global__ void k_sort_rows_global(int32_t n, const int64_t* __restrict__ start,
     }
 }
 
-__global__ void k_count_unique(int32_t n, const int64_t* __restrict__ start,
-                               const uint64_t* __restrict__ keys, int64_t* __restrict__ ucnt) {
+// first[p] = 1 where a row begins
+__global__ void k_row_firsts(int32_t n, const int32_t* __restrict__ start,
+                             unsigned char* __restrict__ first) {
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        int64_t a = start[r], b = start[r + 1], c = 0;
-        uint32_t prev = 0;
-        for (int64_t k = a; k < b; ++k) {
-            uint32_t col = (uint32_t)(keys[k] >> 32);
-            if (k == a || col != prev) ++c;
-            prev = col;
-        }
-        ucnt[r] = c;
+         r += (int64_t)gridDim.x * blockDim.x)
+        if (start[r + 1] > start[r]) first[start[r]] = 1;
+}
+
+// Whether sorted entry p is the first of its (row, col): the others are added
+// to it.  The passes below give every entry to a thread, so the time does
+// not depend on how the entries spread over the rows (a thread per row took
+// 1,634 us for 8M entries, 4096 of them in one row).
+__device__ __forceinline__ bool is_head(const uint64_t* __restrict__ keys,
+                                        const unsigned char* __restrict__ first, int64_t p) {
+    return first[p] || (uint32_t)(keys[p] >> 32) != (uint32_t)(keys[p - 1] >> 32);
+}
+
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_head_counts(int64_t nnz, const uint64_t* __restrict__ keys,
+              const unsigned char* __restrict__ first, int64_t* __restrict__ bsum) {
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
+    int32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        const int64_t p = base + i * SCAN_THREADS + threadIdx.x;
+        if (p < nnz) c += is_head(keys, first, p);
+    }
+    __shared__ int32_t sh[32];
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        c = __reduce_add_sync(0xffffffffu, sh[threadIdx.x]);
+        if (threadIdx.x == 0) bsum[blockIdx.x] = c;
     }
 }
 
+// Writes the heads' columns and sums (each with the equal entries that follow
+// it, in input order) at their places, and every entry's number of heads
+// before it.  boff: exclusive scan of k_head_counts.
 template <typename VIn, typename VOut, typename Acc>
-__global__ void k_merge_unique(int32_t n, const int64_t* __restrict__ start,
-                               const uint64_t* __restrict__ keys, const int64_t* __restrict__ uoff,
-                               const VIn* __restrict__ val, int32_t* __restrict__ out_col,
-                               VOut* __restrict__ out_val) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        int64_t a = start[r], b = start[r + 1], o = uoff[r];
-        int64_t k = a;
-        while (k < b) {
-            uint32_t c = (uint32_t)(keys[k] >> 32);
-            Acc s = (Acc)to_acc(val[(uint32_t)keys[k]]);
-            int64_t j = k + 1;
-            while (j < b && (uint32_t)(keys[j] >> 32) == c) {
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_merge_heads(int64_t nnz, const uint64_t* __restrict__ keys,
+              const unsigned char* __restrict__ first, const int64_t* __restrict__ boff,
+              const VIn* __restrict__ val, int32_t* __restrict__ before,
+              int32_t* __restrict__ out_col, VOut* __restrict__ out_val) {
+    __shared__ int32_t wsum[SCAN_ITEMS][32], slice[SCAN_ITEMS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
+    bool head[SCAN_ITEMS];
+    unsigned heads[SCAN_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        const int64_t p = base + i * SCAN_THREADS + threadIdx.x;
+        head[i] = p < nnz && is_head(keys, first, p);
+        heads[i] = __ballot_sync(0xffffffffu, head[i]);
+        if (lane == 0) wsum[i][warp] = __popc(heads[i]);
+    }
+    __syncthreads();
+    if (warp < SCAN_ITEMS) {  // exclusive over the warps of slice `warp`
+        const int32_t w = wsum[warp][lane];
+        const int32_t inc = warp_incl_scan(w);
+        wsum[warp][lane] = inc - w;
+        if (lane == 31) slice[warp] = inc;
+    }
+    __syncthreads();
+    int64_t o = boff[blockIdx.x];
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        const int64_t p = base + i * SCAN_THREADS + threadIdx.x;
+        const int32_t at = (int32_t)o + wsum[i][warp] + __popc(heads[i] & ((1u << lane) - 1u));
+        if (p < nnz) before[p] = at;
+        if (head[i]) {
+            const uint64_t key = keys[p];
+            Acc s = (Acc)to_acc(val[(uint32_t)key]);
+            for (int64_t j = p + 1; j < nnz && !is_head(keys, first, j); ++j)
                 s = s + (Acc)to_acc(val[(uint32_t)keys[j]]);
-                ++j;
-            }
-            out_col[o] = (int32_t)c;
-            out_val[o] = from_acc<VOut>(s);
-            ++o;
-            k = j;
+            out_col[at] = (int32_t)(key >> 32);
+            out_val[at] = from_acc<VOut>(s);
         }
+        o += slice[i];
     }
 }
 
-__global__ void k_i64_to_i32(int64_t m, const int64_t* __restrict__ in, int32_t* __restrict__ out,
-                             unsigned int* err) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t v = in[i];
-        if (v > INT32_MAX) atomicOr(err, 16u);
-        out[i] = (int32_t)v;
+// row_ptr from the entries' counts of heads before them
+__global__ void k_row_ptr(int32_t n, int64_t nnz, const int32_t* __restrict__ start,
+                          const int32_t* __restrict__ before, const int64_t* __restrict__ total,
+                          int32_t* __restrict__ rp) {
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r <= n;
+         r += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t a = start[r];
+        rp[r] = a < nnz ? before[a] : (int32_t)*total;
     }
 }
 
@@ -551,12 +737,6 @@ static gk_status dispatch_dtype(gk_dtype d, F&& f) {
     return GK_ERR_INVALID;
 }
 
-static gk_status read_err(unsigned int* derr, cudaStream_t s, unsigned int* herr) {
-    GK_CUDA(cudaMemcpyAsync(herr, derr, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-    GK_CUDA(cudaStreamSynchronize(s));
-    return GK_OK;
-}
-
 static gk_matrix new_handle() {
     gk_matrix A = new (std::nothrow) gk_matrix_s();
     if (A) cudaGetDevice(&A->device);
@@ -564,15 +744,18 @@ static gk_matrix new_handle() {
 }
 
 static void free_arrays(gk_matrix A) {
-    dfree(A->row_ptr);
-    dfree(A->col);
-    dfree(A->val);
+    if (A->slab) {
+        dfree(A->slab);
+    } else {
+        for (void* q : {(void*)A->row_ptr, (void*)A->col, A->val, (void*)A->words}) dfree(q);
+    }
+    A->slab = nullptr;
+    A->words = nullptr;
     dfree(A->slice_len);
     dfree(A->slice_set);
     dfree(A->plan.tile_desc);
     for (int32_t* q : {A->plan.unit_row, A->plan.row_end, A->plan.row_id, A->plan.empty_rows})
         dfree(q);
-    dfree(A->plan.err);
     dfree(A->dinv);
     dfree(A->binv);
     A->binv = nullptr;
@@ -589,6 +772,28 @@ static void free_arrays(gk_matrix A) {
     A->slice_set = nullptr;
     A->plan = CsrPlan();
     A->dinv = nullptr;
+}
+
+// row_ptr, col, val (each with the 64 bytes of slack of an allocation of its
+// own) and the handle's words in one allocation: a cudaMalloc or cudaFree
+// takes 30 to 90 us of host time, as long as the kernels that fill the arrays.
+static gk_status alloc_csr(gk_matrix A) {
+    auto up = [](size_t b) { return (b + 64 + 255) & ~(size_t)255; };
+    const size_t nz = (size_t)std::max<int64_t>(A->nnz, 1);
+    const size_t col = up(4 * ((size_t)A->n + 1)), val = col + up(4 * nz);
+    const size_t words = val + up(value_bytes(A->dtype) * nz);
+    if (dmalloc(&A->slab, words + 256) != cudaSuccess) return GK_ERR_OOM;
+    char* p = static_cast<char*>(A->slab);
+    A->row_ptr = (int32_t*)p;
+    A->col = (int32_t*)(p + col);
+    A->val = p + val;
+    A->words = (int32_t*)(p + words);
+    return GK_OK;
+}
+
+static gk_status ensure_words(gk_matrix A) {
+    if (!A->words) GK_CUDA(dmalloc_t(&A->words, 64));
+    return GK_OK;
 }
 
 static void destroy_handle(gk_matrix A) {
@@ -657,9 +862,9 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
     CsrPlan& P = A->plan;
     dfree(P.tile_desc);
     for (int32_t* q : {P.unit_row, P.row_end, P.row_id, P.empty_rows}) dfree(q);
-    dfree(P.err);
     P = CsrPlan();
-    GK_CUDA(dmalloc_t(&P.err, 4));
+    GK_TRY(ensure_words(A));
+    P.err = A->words;
     GK_CUDA(cudaMemsetAsync(P.err, 0, 4, s));
     if (A->fmt != GK_CSR || A->n == 0) return GK_OK;
     const double mean = A->mean_row;
@@ -781,19 +986,20 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
         if (P.units > 0) {
             const int32_t step = std::max(1, P.units / 4096);
             const int32_t sampled = (P.units + step - 1) / step;
-            TmpBuf cnt;
-            GK_TRY(cnt.ensure(4));
-            GK_CUDA(cudaMemsetAsync(cnt.ptr, 0, 4, s));
+            int32_t* cnt = A->words + 16;
+            GK_CUDA(cudaMemsetAsync(cnt, 0, 4, s));
             k_unit_span<<<(unsigned)((sampled + 7) / 8), 256, 0, s>>>(
                 A->nnz, P.units, step, (int32_t)(LOCAL_COLS_BYTES / vector_bytes(A->dtype)), A->col,
-                (int32_t*)cnt.ptr);
+                cnt);
             int32_t close = 0;
-            GK_CUDA(cudaMemcpyAsync(&close, cnt.ptr, 4, cudaMemcpyDeviceToHost, s));
+            GK_CUDA(cudaMemcpyAsync(&close, cnt, 4, cudaMemcpyDeviceToHost, s));
             GK_CUDA(cudaStreamSynchronize(s));
             P.local_cols = 2 * close > sampled;
         }
-        GK_TRY(A->carry.ensure((size_t)P.units * (4 + vector_bytes(A->dtype)) + 16));
-        GK_CUDA(dmalloc_t(&P.unit_row, (size_t)P.units + 1));
+        const size_t urow = (4 * ((size_t)P.units + 1) + 255) & ~(size_t)255;
+        GK_CUDA(dmalloc((void**)&P.unit_row,
+                        urow + (size_t)P.units * (4 + vector_bytes(A->dtype)) + 16));
+        P.carries = (char*)P.unit_row + urow;
         k_unit_rows<<<grid_for(P.units + 1), 256, 0, s>>>(
             m, P.row_end ? P.row_end : A->row_ptr + 1, P.units, P.unit_row);
         GK_CUDA(cudaGetLastError());
@@ -802,22 +1008,21 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
 }
 
 // Validates a CSR handle's arrays, computes max/mean row length and plans.
-static gk_status finish_csr(gk_matrix A, cudaStream_t s) {
-    DevBuf flags;
-    GK_TRY(flags.ensure(16));
-    unsigned int* derr = reinterpret_cast<unsigned int*>(flags.ptr);
+// cols_valid: the columns have been checked.
+static gk_status finish_csr(gk_matrix A, cudaStream_t s, bool cols_valid = false) {
+    GK_TRY(ensure_words(A));
+    unsigned int* derr = reinterpret_cast<unsigned int*>(A->words + 8);
     int32_t* dmax = reinterpret_cast<int32_t*>(derr + 1);
-    GK_CUDA(cudaMemsetAsync(flags.ptr, 0, 16, s));
+    GK_CUDA(cudaMemsetAsync(derr, 0, 16, s));
     if (A->n > 0)
         k_validate_rowptr<<<grid_for(A->n), 256, 0, s>>>(A->n, A->nnz, A->row_ptr, derr, dmax,
                                                          dmax + 1);
-    if (A->nnz > 0)
+    if (A->nnz > 0 && !cols_valid)
         k_validate_cols<<<grid_for(A->nnz), 256, 0, s>>>(A->nnz, A->ncols, A->col, derr);
     GK_CUDA(cudaGetLastError());
     unsigned int h[3] = {0, 0, 0};
-    GK_CUDA(cudaMemcpyAsync(h, flags.ptr, 12, cudaMemcpyDeviceToHost, s));
+    GK_CUDA(cudaMemcpyAsync(h, derr, 12, cudaMemcpyDeviceToHost, s));
     GK_CUDA(cudaStreamSynchronize(s));
-    flags.release();
     if (h[0]) return GK_ERR_INVALID;
     A->max_row = (int32_t)h[1];
     A->empty_rows_known = (int32_t)h[2];
@@ -882,10 +1087,7 @@ gk_status gk_matrix_create_csr(int32_t n, int32_t ncols, int64_t nnz, const int3
         destroy_handle(A);
         return e;
     };
-    if (dmalloc_t(&A->row_ptr, (size_t)n + 1) != cudaSuccess ||
-        dmalloc_t(&A->col, (size_t)std::max<int64_t>(nnz, 1)) != cudaSuccess ||
-        dmalloc(&A->val, value_bytes(dtype) * (size_t)std::max<int64_t>(nnz, 1)) != cudaSuccess)
-        return fail(GK_ERR_OOM);
+    if ((st = alloc_csr(A)) != GK_OK) return fail(st);
     if ((st = copy_in(A->row_ptr, row_ptr, sizeof(int32_t) * ((size_t)n + 1), mem, s)) != GK_OK ||
         (st = copy_in(A->col, col_idx, sizeof(int32_t) * (size_t)nnz, mem, s)) != GK_OK ||
         (st = copy_in(A->val, values, value_bytes(dtype) * (size_t)nnz, mem, s)) != GK_OK)
@@ -906,89 +1108,117 @@ gk_status gk_matrix_create_coo(int32_t n, int32_t ncols, int64_t nnz, const int3
     if (nnz > 0 && (!row || !col || !values)) return GK_ERR_INVALID;
     cudaStream_t s = (cudaStream_t)stream;
     const size_t vb = value_bytes(dtype);
-    // device staging of the triplets
-    DevBuf drow, dcol, dval, cnt, start, cursor, keys, ucnt, uoff, tmp, flags, scratch;
-    auto cleanup = [&]() {
-        drow.release(); dcol.release(); dval.release(); cnt.release(); start.release();
-        cursor.release(); keys.release(); ucnt.release(); uoff.release(); tmp.release();
-        flags.release(); scratch.release();
+    const size_t nz1 = (size_t)std::max<int64_t>(nnz, 1), n1 = (size_t)n + 1;
+    const int64_t nblk = std::max<int64_t>(1, (nnz + SCAN_TILE - 1) / SCAN_TILE);
+    // one scratch allocation (an allocation and its free cost more than most
+    // of the kernels); triplets on the device are read in place
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) & ~(size_t)255;
+        return o;
     };
+    const bool host = mem == GK_MEM_HOST;
+    const size_t o_keys = part(8 * nz1), o_rank = part(4 * nz1), o_first = part(nz1);
+    const size_t o_cnt = part(4 * n1), o_start = part(4 * n1), o_list = part(4 * n1);
+    const size_t o_bsum = part(8 * (size_t)std::max(nblk + 1, n / (int64_t)SCAN_TILE + 1)), o_info = part(256);
+    const size_t o_row = part(host ? 4 * nz1 : 0), o_col = part(host ? 4 * nz1 : 0);
+    const size_t o_val = part(host ? vb * nz1 : 0);
+    TmpBuf scratch, longs;
+    if (scratch.ensure(at)) return GK_ERR_OOM;
+    char* base = static_cast<char*>(scratch.ptr);
     gk_matrix A = nullptr;
     auto fail = [&](gk_status e) {
-        cleanup();
         destroy_handle(A);
         return e;
     };
-    const size_t nz1 = (size_t)std::max<int64_t>(nnz, 1);
-    if (drow.ensure(4 * nz1) || dcol.ensure(4 * nz1) || dval.ensure(vb * nz1) ||
-        cnt.ensure(4 * ((size_t)n + 1)) || start.ensure(8 * ((size_t)n + 1)) ||
-        cursor.ensure(4 * ((size_t)n + 1)) || keys.ensure(8 * nz1) ||
-        ucnt.ensure(8 * ((size_t)n + 1)) || uoff.ensure(8 * ((size_t)n + 1)) || flags.ensure(16))
-        return fail(GK_ERR_OOM);
     gk_status st;
-    if ((st = copy_in(drow.ptr, row, 4 * (size_t)nnz, mem, s)) != GK_OK ||
-        (st = copy_in(dcol.ptr, col, 4 * (size_t)nnz, mem, s)) != GK_OK ||
-        (st = copy_in(dval.ptr, values, vb * (size_t)nnz, mem, s)) != GK_OK)
-        return fail(st);
-    unsigned int* derr = reinterpret_cast<unsigned int*>(flags.ptr);
-    int32_t* dcnt = reinterpret_cast<int32_t*>(cnt.ptr);
-    int64_t* dstart = reinterpret_cast<int64_t*>(start.ptr);
-    int32_t* dcur = reinterpret_cast<int32_t*>(cursor.ptr);
-    uint64_t* dkeys = reinterpret_cast<uint64_t*>(keys.ptr);
-    if (cudaMemsetAsync(flags.ptr, 0, 16, s) || cudaMemsetAsync(dcnt, 0, 4 * ((size_t)n + 1), s) ||
-        cudaMemsetAsync(dcur, 0, 4 * ((size_t)n + 1), s))
-        return fail(GK_ERR_CUDA);
-    if (nnz > 0)
-        k_coo_count<<<grid_for(nnz), 256, 0, s>>>(nnz, n, ncols, (const int32_t*)drow.ptr,
-                                                  (const int32_t*)dcol.ptr, dcnt, derr);
-    unsigned int herr = 0;
-    if ((st = read_err(derr, s, &herr)) != GK_OK) return fail(st);
-    if (herr) return fail(GK_ERR_INVALID);
-    if ((st = scan_exclusive<int32_t, int64_t>(dcnt, dstart, n, tmp, s)) != GK_OK) return fail(st);
-    if (nnz > 0)
-        k_coo_scatter<<<grid_for(nnz), 256, 0, s>>>(nnz, (const int32_t*)drow.ptr,
-                                                    (const int32_t*)dcol.ptr, dstart, dcur, dkeys);
-    // longest row, for choosing the sorters
-    std::vector<int32_t> hcnt((size_t)n + 1, 0);
-    if (n > 0 && cudaMemcpyAsync(hcnt.data(), dcnt, 4 * (size_t)n, cudaMemcpyDeviceToHost, s))
-        return fail(GK_ERR_CUDA);
-    if (cudaStreamSynchronize(s)) return fail(GK_ERR_CUDA);
-    int64_t maxL = 0;
-    for (int32_t i = 0; i < n; ++i) maxL = std::max<int64_t>(maxL, hcnt[i]);
-    if (n > 0 && maxL > 1) {
-        const unsigned gs = grid_for((int64_t)n * 8);
-        k_sort_rows_sub<2><<<gs, 256, 0, s>>>(n, dstart, dkeys);
-        if (maxL > 2) k_sort_rows_sub<4><<<gs, 256, 0, s>>>(n, dstart, dkeys);
-        if (maxL > 4) k_sort_rows_sub<8><<<gs, 256, 0, s>>>(n, dstart, dkeys);
-        if (maxL > 8) k_sort_rows_sub<16><<<gs, 256, 0, s>>>(n, dstart, dkeys);
-        if (maxL > 16) k_sort_rows_sub<32><<<gs, 256, 0, s>>>(n, dstart, dkeys);
-        if (maxL > 32) {
-            const int cap = 16384;  // keys in shared memory (128 KB)
-            cudaFuncSetAttribute(k_sort_rows_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 cap * 8);
-            const int64_t hi = std::min<int64_t>(maxL, cap);
-            int P = 1;
-            while (P < hi) P <<= 1;
-            k_sort_rows_block<<<(unsigned)std::min<int64_t>(n, num_sms() * 4), 512, (size_t)P * 8,
-                                s>>>(n, dstart, dkeys, 32, cap, P);
-            if (maxL > cap) {
-                int64_t Q = 1;
-                while (Q < maxL) Q <<= 1;
-                const int nb = 4;
-                if (scratch.ensure((size_t)nb * Q * 8)) return fail(GK_ERR_OOM);
-                k_sort_rows_global<<<nb, 1024, 0, s>>>(n, dstart, dkeys, cap,
-                                                       (uint64_t*)scratch.ptr, Q);
-            }
-        }
+    const int32_t *drow = row, *dcol = col;
+    const void* dval = values;
+    if (host) {
+        if ((st = copy_in(base + o_row, row, 4 * (size_t)nnz, mem, s)) != GK_OK ||
+            (st = copy_in(base + o_col, col, 4 * (size_t)nnz, mem, s)) != GK_OK ||
+            (st = copy_in(base + o_val, values, vb * (size_t)nnz, mem, s)) != GK_OK)
+            return fail(st);
+        drow = (const int32_t*)(base + o_row);
+        dcol = (const int32_t*)(base + o_col);
+        dval = base + o_val;
     }
-    int64_t* ducnt = reinterpret_cast<int64_t*>(ucnt.ptr);
-    int64_t* duoff = reinterpret_cast<int64_t*>(uoff.ptr);
-    if (n > 0) k_count_unique<<<grid_for(n), 256, 0, s>>>(n, dstart, dkeys, ducnt);
-    if ((st = scan_exclusive<int64_t, int64_t>(ducnt, duoff, n, tmp, s)) != GK_OK) return fail(st);
-    int64_t nnz_out = 0;
-    if (cudaMemcpyAsync(&nnz_out, duoff + n, 8, cudaMemcpyDeviceToHost, s) ||
+    uint64_t* dkeys = (uint64_t*)(base + o_keys);
+    int32_t* drank = (int32_t*)(base + o_rank);  // then: heads before every entry
+    unsigned char* dfirst = (unsigned char*)(base + o_first);
+    int32_t* dcnt = (int32_t*)(base + o_cnt);
+    int32_t* dstart = (int32_t*)(base + o_start);
+    int32_t* dlist = (int32_t*)(base + o_list);
+    int64_t* dbsum = (int64_t*)(base + o_bsum);
+    // info words: the class sizes and the longest row, the error flags, the
+    // lists' cursors
+    int32_t* dinfo = (int32_t*)(base + o_info);
+    unsigned int* derr = (unsigned int*)(dinfo + 16);
+    int32_t* dcursor = dinfo + 32;
+    if (cudaMemsetAsync(dinfo, 0, 256, s) || cudaMemsetAsync(dcnt, 0, 4 * n1, s) ||
+        cudaMemsetAsync(dfirst, 0, nz1, s))
+        return fail(GK_ERR_CUDA);
+    if (nnz > 0)
+        k_coo_count<<<grid_for(nnz), 256, 0, s>>>(nnz, n, ncols, drow, dcol, dcnt, drank, derr);
+    if (n > 0) k_class_sizes<<<std::min(grid_for(n), (unsigned)num_sms() * 2), 256, 0, s>>>(n, dcnt, dinfo);
+    if ((st = scan_exclusive_in<int32_t, int32_t>(dcnt, dstart, n, dbsum, s)) != GK_OK) return fail(st);
+    int32_t info[17] = {0};
+    if (cudaMemcpyAsync(info, dinfo, sizeof(info), cudaMemcpyDeviceToHost, s) ||
         cudaStreamSynchronize(s))
         return fail(GK_ERR_CUDA);
+    if (info[16]) return fail(GK_ERR_INVALID);
+    if (nnz > 0)
+        k_coo_scatter<<<grid_for(nnz), 256, 0, s>>>(nnz, drow, dcol, dstart, drank, dkeys);
+    ClassOffsets off;
+    int32_t listed = 0;
+    for (int c = 0; c < SORT_CLASSES; ++c) {
+        off.o[c] = listed;
+        listed += info[c];
+    }
+    if (listed > 0) {
+        k_class_lists<<<(unsigned)(((int64_t)n + 255) / 256), 256, 0, s>>>(n, dcnt, off, dcursor, dlist);
+        auto groups = [&](int c, int lanes) { return grid_for((int64_t)info[c] * lanes); };
+        auto l = [&](int c) { return dlist + off.o[c]; };
+        if (info[0]) k_sort_rows_sub<2><<<groups(0, 2), 256, 0, s>>>(info[0], l(0), dstart, dkeys);
+        if (info[1]) k_sort_rows_sub<4><<<groups(1, 4), 256, 0, s>>>(info[1], l(1), dstart, dkeys);
+        if (info[2]) k_sort_rows_sub<8><<<groups(2, 8), 256, 0, s>>>(info[2], l(2), dstart, dkeys);
+        if (info[3]) k_sort_rows_sub<16><<<groups(3, 16), 256, 0, s>>>(info[3], l(3), dstart, dkeys);
+        if (info[4]) k_sort_rows_sub<32><<<groups(4, 32), 256, 0, s>>>(info[4], l(4), dstart, dkeys);
+        auto warps = [&](int c) { return (unsigned)std::min<int64_t>(((int64_t)info[c] + 3) / 4, (int64_t)num_sms() * 16); };
+        if (info[5]) k_sort_rows_warp<2><<<warps(5), 128, 0, s>>>(info[5], l(5), dstart, dkeys);
+        if (info[6]) k_sort_rows_warp<4><<<warps(6), 128, 0, s>>>(info[6], l(6), dstart, dkeys);
+        if (info[7]) k_sort_rows_warp<8><<<warps(7), 128, 0, s>>>(info[7], l(7), dstart, dkeys);
+        if (info[8]) k_sort_rows_warp<16><<<warps(8), 128, 0, s>>>(info[8], l(8), dstart, dkeys);
+        const int32_t longest = info[SORT_CLASSES];
+        if (info[9]) {
+            cudaFuncSetAttribute(k_sort_rows_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 SORT_BLOCK_MAX * 8);
+            int P = 1024;
+            while (P < std::min(longest, SORT_BLOCK_MAX)) P <<= 1;
+            k_sort_rows_block<<<(unsigned)std::min<int64_t>(info[9], (int64_t)num_sms() * 6), 256,
+                                (size_t)P * 8, s>>>(info[9], l(9), dstart, dkeys);
+        }
+        if (info[10]) {
+            int64_t Q = 1;
+            while (Q < longest) Q <<= 1;
+            const int nb = std::min(info[10], 4);
+            if (longs.ensure((size_t)nb * Q * 8)) return fail(GK_ERR_OOM);
+            k_sort_rows_global<<<nb, 1024, 0, s>>>(info[10], l(10), dstart, dkeys,
+                                                   (uint64_t*)longs.ptr, Q);
+        }
+    }
+    // heads: the first entry of every (row, col)
+    int64_t nnz_out = 0;
+    if (nnz > 0) {
+        k_row_firsts<<<grid_for(n), 256, 0, s>>>(n, dstart, dfirst);
+        k_head_counts<<<(unsigned)nblk, SCAN_THREADS, 0, s>>>(nnz, dkeys, dfirst, dbsum);
+        if (cudaMemsetAsync(dbsum + nblk, 0, 8, s)) return fail(GK_ERR_CUDA);
+        k_scan_blocksums<<<1, SCAN_THREADS, 0, s>>>(dbsum, nblk + 1);
+        if (cudaMemcpyAsync(&nnz_out, dbsum + nblk, 8, cudaMemcpyDeviceToHost, s) ||
+            cudaStreamSynchronize(s))
+            return fail(GK_ERR_CUDA);
+    }
     A = new_handle();
     if (!A) return fail(GK_ERR_OOM);
     A->n = n;
@@ -996,23 +1226,23 @@ gk_status gk_matrix_create_coo(int32_t n, int32_t ncols, int64_t nnz, const int3
     A->nnz = nnz_out;
     A->fmt = GK_CSR;
     A->dtype = dtype;
-    if (dmalloc_t(&A->row_ptr, (size_t)n + 1) || dmalloc_t(&A->col, (size_t)std::max<int64_t>(nnz_out, 1)) ||
-        dmalloc(&A->val, vb * (size_t)std::max<int64_t>(nnz_out, 1)))
-        return fail(GK_ERR_OOM);
-    k_i64_to_i32<<<grid_for((int64_t)n + 1), 256, 0, s>>>((int64_t)n + 1, duoff, A->row_ptr, derr);
-    if (n > 0) {
+    if ((st = alloc_csr(A)) != GK_OK) return fail(st);
+    if (nnz > 0) {
         st = dispatch_dtype(dtype, [&](auto tp) -> gk_status {
             using V = typename decltype(tp)::V;
             using Acc = typename AccOf<V>::type;
-            k_merge_unique<V, V, Acc><<<grid_for(n), 256, 0, s>>>(
-                n, dstart, dkeys, duoff, (const V*)dval.ptr, A->col, (V*)A->val);
+            k_merge_heads<V, V, Acc><<<(unsigned)nblk, SCAN_THREADS, 0, s>>>(
+                nnz, dkeys, dfirst, dbsum, (const V*)dval, drank, A->col, (V*)A->val);
             return GK_OK;
         });
         if (st != GK_OK) return fail(st);
+        k_row_ptr<<<grid_for((int64_t)n + 1), 256, 0, s>>>(n, nnz, dstart, drank, dbsum + nblk,
+                                                           A->row_ptr);
+    } else if (cudaMemsetAsync(A->row_ptr, 0, 4 * n1, s)) {
+        return fail(GK_ERR_CUDA);
     }
     if (cudaGetLastError()) return fail(GK_ERR_CUDA);
-    if ((st = finish_csr(A, s)) != GK_OK) return fail(st);
-    cleanup();
+    if ((st = finish_csr(A, s, true)) != GK_OK) return fail(st);
     *out = A;
     return GK_OK;
 }

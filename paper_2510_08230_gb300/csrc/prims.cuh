@@ -90,21 +90,26 @@ __global__ void k_scan_apply(const In* __restrict__ in, int64_t m,
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[m] = (Out)(off + tot);
 }
 
-// out[0..m] = exclusive prefix sum of in[0..m), out[m] = total.
+// out[0..m] = exclusive prefix sum of in[0..m), out[m] = total; bs: scratch of
+// ceil(m / SCAN_TILE) words.
 template <typename In, typename Out>
-gk_status scan_exclusive(const In* in, Out* out, int64_t m, DevBuf& tmp, cudaStream_t s) {
+gk_status scan_exclusive_in(const In* in, Out* out, int64_t m, int64_t* bs, cudaStream_t s) {
     if (m <= 0) {
         GK_CUDA(cudaMemsetAsync(out, 0, sizeof(Out), s));
         return GK_OK;
     }
     const int64_t nb = (m + SCAN_TILE - 1) / SCAN_TILE;
-    GK_TRY(tmp.ensure(sizeof(int64_t) * (size_t)nb));
-    int64_t* bs = reinterpret_cast<int64_t*>(tmp.ptr);
     k_scan_reduce<In><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, m, bs);
     k_scan_blocksums<<<1, SCAN_THREADS, 0, s>>>(bs, nb);
     k_scan_apply<In, Out><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, m, bs, out);
     GK_CUDA(cudaGetLastError());
     return GK_OK;
+}
+
+template <typename In, typename Out>
+gk_status scan_exclusive(const In* in, Out* out, int64_t m, DevBuf& tmp, cudaStream_t s) {
+    GK_TRY(tmp.ensure(sizeof(int64_t) * (size_t)std::max<int64_t>(1, (m + SCAN_TILE - 1) / SCAN_TILE)));
+    return scan_exclusive_in<In, Out>(in, out, m, reinterpret_cast<int64_t*>(tmp.ptr), s);
 }
 
 // ---------------------------------------------------------------- reductions

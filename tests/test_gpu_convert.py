@@ -332,3 +332,21 @@ def test_ell_to_sellp_and_narrowing_conversions():
     assert np.array_equal(bf16_bits_to_f64(gb["values"]), bf16_round_f64(m.values))
     for H in (B, P2, P1, E, A):
         H.close()
+
+
+@pytest.mark.parametrize("dtype,mem", [("f64", "device"), ("f32", "host")])
+def test_coo_to_csr_sort_classes_and_heads(dtype, mem):
+    """Rows at both edges of every sorter's class of lengths, empty rows
+    between them, runs of equal positions across the merge pass's 4096-entry
+    blocks and their 1024-entry slices, a whole row of one position."""
+    rng = np.random.default_rng(8)
+    lengths = [0, 1, 2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 0, 128, 129, 256, 257, 512, 513,
+               1024, 1025, 4096, 0, 16384, 16385]
+    row = np.repeat(np.arange(len(lengths)), lengths)
+    col = rng.integers(0, 20000, row.size)
+    col[rng.random(row.size) < 0.3] = 7            # long runs of one column
+    row = np.concatenate([row, np.full(9000, len(lengths))])
+    col = np.concatenate([col, np.full(9000, 3)])  # a row of one position
+    order = rng.permutation(row.size)
+    v = rng.standard_normal(row.size) * 10.0 ** rng.integers(-3, 4, row.size)
+    _check_coo(len(lengths) + 2, 20000, row[order], col[order], v, dtype, mem)
