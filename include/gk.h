@@ -241,13 +241,14 @@ typedef struct {
                              2 single-block (CSR, CG/BiCGSTAB, n <= 16384);
                              3 cluster of up to 16 blocks (CSR, CG, n <= 16384).
                              Automatic picks 3 for CSR CG with n <= 16384 when a
-                             cluster can be scheduled; for other CG solves
-                             (none or Jacobi) whose SpMV layout is ELL, and for
-                             such inner solves of refinement, one persistent
-                             kernel over the whole GPU while a block's share of
-                             the vectors fits in shared memory (FP64: up to
-                             about 2.1 million rows); else 1.  Block-Jacobi,
-                             ILU(0) and CGS run on engine 1 only. */
+                             cluster can be scheduled; for other CG solves and
+                             for GMRES with n >= 1024 (none or Jacobi) whose
+                             SpMV layout is ELL, and for such inner solves of
+                             refinement, one persistent kernel over the GPU
+                             while a block's share of the vectors fits in
+                             shared memory (FP64: CG up to about 2.1, GMRES
+                             3.9 million rows); else 1.  Block-Jacobi, ILU(0)
+                             and CGS run on engine 1 only. */
     int32_t block_size;   /* block-Jacobi rows per diagonal block, 1..32 */
     int64_t wait_budget_ns; /* longest a device-side wait of this solve may last
                              (the ILU(0) substitutions' polls on values other
@@ -293,9 +294,10 @@ typedef struct {
  * residual and the residual replacement decided by kernels; the host only
  * reads the outcome (GK_SOLVE_LOOP=host launches one graph per pass from
  * the host instead, two in flight; same results).  The solve works on the
- * handle's own copies of b and x.  The persistent CG kernel of the automatic
- * engine runs the same recurrence and stopping rule (its dot products add in
- * another order); such solves of one process run one after another.
+ * handle's own copies of b and x.  The persistent kernels of the automatic
+ * engine run the same recurrences and stopping rules (their dot products add
+ * in another order).  Such solves of one process share the GPU while their
+ * blocks fit on it together, and queue otherwise.
  * SpMV layout (multi-kernel engine and refinement on a CSR matrix): a matrix
  * of at least 2^24 entries whose apply uses the CSR warp-tile kernel
  * (gk_matrix_desc.spmv_kernel 6) solves on its own arrays; otherwise the

@@ -2,7 +2,10 @@
 // SpMV layout, FP64 iterative refinement around FP32 / BF16-stored inner
 // solves) and the host-side helpers of the multi-kernel engine
 // (solve_engine.cuh).
+#include <condition_variable>
+
 #include "gridcg.cuh"
+#include "gridgm.cuh"
 
 namespace gk {
 
@@ -236,9 +239,37 @@ gk_status read_hdr(SolverCache* C, cudaStream_t s) {
     return GK_OK;
 }
 
-std::mutex& grid_cg_mutex() {
-    static std::mutex mu;
-    return mu;
+namespace {
+struct Seats {
+    std::mutex mu;
+    std::condition_variable freed;
+    uint64_t next_ticket = 0, serving = 0;
+    int used = 0;
+};
+Seats& seats() {
+    static Seats* s = new Seats;  // outlives threads still in a solve at exit
+    return *s;
+}
+}  // namespace
+
+GridSeats::GridSeats(bool half, int blocks) : seats_(half ? blocks : 2 * num_sms()) {
+    Seats& g = seats();
+    std::unique_lock<std::mutex> lk(g.mu);
+    const uint64_t ticket = g.next_ticket++;
+    g.freed.wait(lk, [&] { return g.serving == ticket && g.used + seats_ <= 2 * num_sms(); });
+    g.used += seats_;
+    ++g.serving;
+    lk.unlock();
+    g.freed.notify_all();
+}
+
+GridSeats::~GridSeats() {
+    Seats& g = seats();
+    {
+        std::lock_guard<std::mutex> lk(g.mu);
+        g.used -= seats_;
+    }
+    g.freed.notify_all();
 }
 
 gk_status clear_halt(SolverCache* C, cudaStream_t s) {
@@ -285,6 +316,14 @@ static void reset_wait(gk_matrix A) {
         }
 }
 
+// A solve that grid_admits on its method's persistent kernel.
+template <typename V, typename T>
+static gk_status solve_grid(gk_matrix M, const T* b, T* x, int method, int pkind, double tol,
+                            int32_t max_iters, int m, cudaStream_t s, SolveOut* out, bool inner) {
+    return method == GK_CG ? solve_grid_cg<V, T>(M, b, x, pkind, tol, max_iters, s, out, inner)
+                           : solve_grid_gmres<V, T>(M, b, x, pkind, tol, max_iters, m, s, out, inner);
+}
+
 template <typename V, typename T>
 static gk_status solve_plain(gk_matrix A, const void* b, void* x, const gk_solve_opts* o,
                              cudaStream_t s, SolveOut* out) {
@@ -293,9 +332,9 @@ static gk_status solve_plain(gk_matrix A, const void* b, void* x, const gk_solve
     GK_TRY(solve_matrix(A, s, &M));
     M->wait_ns = A->wait_ns;
     gk_status st = GK_ERR_UNSUPPORTED;
-    if (o->engine == 0 && grid_cg_admits(M, o->method, (int)o->precond))
-        st = solve_grid_cg<V, T>(M, (const T*)b, (T*)x, (int)o->precond, o->tol, o->max_iters, s,
-                                 out, false);
+    if (o->engine == 0 && grid_admits(M, o->method, (int)o->precond))
+        st = solve_grid<V, T>(M, (const T*)b, (T*)x, o->method, (int)o->precond, o->tol,
+                              o->max_iters, m, s, out, false);
     if (st == GK_ERR_UNSUPPORTED)
         st = solve_mk<V, T>(M, (const T*)b, (T*)x, o->method, (int)o->precond, o->block_size,
                             o->tol, o->max_iters, m, s, out, false);
@@ -419,9 +458,9 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         const int32_t left = o->max_iters - total_inner;
         auto inner_solve = [&](auto vt) -> gk_status {
             using V = decltype(vt);
-            if (o->engine == 0 && grid_cg_admits(L, o->method, pk)) {
-                const gk_status g = solve_grid_cg<V, float>(L, r32, d32, pk, inner_tol, left, s,
-                                                            &io, true);
+            if (o->engine == 0 && grid_admits(L, o->method, pk)) {
+                const gk_status g = solve_grid<V, float>(L, r32, d32, o->method, pk, inner_tol,
+                                                         left, m, s, &io, true);
                 if (g != GK_ERR_UNSUPPORTED) return g;
             }
             return solve_mk<V, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left, m, s, &io,

@@ -1,6 +1,7 @@
-"""CG's persistent grid-wide kernel (the automatic engine on matrices that
-solve on an ELL layout) against the multi-kernel engine (engine=1) and the
-oracle: every shared-memory mode, odd sizes, both ends of its range."""
+"""The persistent grid-wide kernels of CG and GMRES (the automatic engine on
+matrices that solve on an ELL layout) against the multi-kernel engine
+(engine=1) and the oracle: every shared-memory mode, odd sizes, both ends of
+their range."""
 import numpy as np
 import pytest
 
@@ -21,7 +22,7 @@ def _solve(A, b, dtype, **kw):
     import torch
     bt = torch.from_numpy(b).to(torch_dev(), torch.float64 if dtype == "f64" else torch.float32)
     x = torch.zeros_like(bt)
-    info = A.solve(bt, x, method="cg", **kw)
+    info = A.solve(bt, x, **dict(dict(method="cg"), **kw))
     return x.cpu().numpy().astype(np.float64), info
 
 
@@ -32,6 +33,8 @@ FIXED = {
     "mode0_large": lambda: W.laplacian_2d(601, 599),
     "mode1_wide": lambda: W.banded_spd(40001, 60, 3),     # 121 entries a row
     "mode1": lambda: W.laplacian_1d(900001),
+    "half_limit": lambda: W.laplacian_2d(608, 512),       # 2,048 rows a block: the last half grid
+    "half_mode1": lambda: W.banded_spd(60001, 12, 4),     # 25 entries a row
     "mode2": lambda: W.laplacian_1d(1200001),             # FP64 only: 7,936 rows a block
 }
 
@@ -60,9 +63,35 @@ def test_fixed_iterations_equal_multi_kernel(name, dtype, precond):
     A.close()
 
 
+@pytest.mark.parametrize("name,m", [("mode0_first", 30), ("mode0_odd", 7), ("mode1_wide", 64),
+                                    ("mode1", 33), ("mode2", 9), ("half_limit", 31),
+                                    ("half_mode1", 12)])
+@pytest.mark.parametrize("dtype,precond", [("f64", "jacobi"), ("f64", None), ("f32", "jacobi")])
+def test_gmres_fixed_steps_equal_multi_kernel(name, m, dtype, precond):
+    """m + 5 Arnoldi steps (a restart among them; up to 64 columns, with and
+    without the matrix in shared memory): orthogonalised twice, so the steps
+    of either engine are within a few n eps of exact ones relative to the
+    cycle's residual; a factor 10^3 as for CG."""
+    mat = FIXED[name]()
+    A = gk.Matrix.from_csr(mat, dtype)
+    b = W.uniform_vector(mat.n, 3)
+    kw = dict(method="gmres", precond=precond, tol=1e-30, max_iters=m + 5, krylov_dim=m)
+    x1, i1 = _solve(A, b, dtype, engine=1, **kw)
+    x0, i0 = _solve(A, b, dtype, **kw)
+    assert i0["return"] == i1["return"] == gk.GK_NOT_CONVERGED
+    assert (i0["iters"], i0["restarts"]) == (i1["iters"], i1["restarts"]) == (m + 5, 1)
+    eps = 2.0 ** -53 if dtype == "f64" else 2.0 ** -24
+    tol = 1e3 * np.sqrt(mat.n) * eps
+    assert np.linalg.norm(x0 - x1) <= tol * np.linalg.norm(x1)
+    for key in ("rel_res_true", "rel_res_recurrence"):
+        assert abs(i0[key] - i1[key]) <= tol * (1 + i1[key])
+    A.close()
+
+
+@pytest.mark.parametrize("method", ["cg", "gmres"])
 @pytest.mark.parametrize("mixed", [0, 1, 2, 3])
 @pytest.mark.parametrize("name", ["lap2d", "diff3d"])
-def test_converges_like_multi_kernel(name, mixed):
+def test_converges_like_multi_kernel(name, mixed, method):
     """To a true 1e-10, plain and refined (the inner solves run on the same
     kernel), from a nonzero start; twice, with the same bits."""
     import torch
@@ -73,20 +102,23 @@ def test_converges_like_multi_kernel(name, mixed):
     out = []
     for engine in (1, 0, 0):
         x = torch.from_numpy(0.1 * W.uniform_vector(m.n, 6)).to(torch_dev())
-        info = A.solve(bt, x, method="cg", precond="jacobi", tol=1e-10, max_iters=20000,
+        info = A.solve(bt, x, method=method, precond="jacobi", tol=1e-10, max_iters=40000,
                        mixed=mixed, engine=engine)
         assert info["return"] == gk.GK_OK, info
         assert oracle.true_rel_residual(m, b, x.cpu().numpy()) <= 1e-10
         out.append((x.cpu().numpy(), info))
     assert np.array_equal(out[1][0], out[2][0])
     if not mixed:
-        assert abs(out[0][1]["iters"] - out[1][1]["iters"]) <= max(3, 0.1 * out[0][1]["iters"])
+        assert abs(out[0][1]["iters"] - out[1][1]["iters"]) <= max(
+            3 if method == "cg" else 30, 0.1 * out[0][1]["iters"])
     A.close()
 
 
-def test_edges():
-    """b = 0, an exact initial guess, a breakdown, NaN, an iteration cap of
-    one, and a zero diagonal: the multi-kernel engine's outcomes."""
+@pytest.mark.parametrize("method", ["cg", "gmres"])
+def test_edges(method):
+    """b = 0, an exact initial guess, a negative definite matrix (a breakdown
+    of CG), NaN, an iteration cap of one, and a zero diagonal: the
+    multi-kernel engine's outcomes."""
     import torch
     dev = torch_dev()
     m = W.laplacian_2d(130)
@@ -103,15 +135,55 @@ def test_edges():
         res = []
         for engine in (1, 0):
             x = x0.clone()
-            info = M.solve(b, x, method="cg", tol=1e-10, engine=engine, **dict(dict(max_iters=99), **kw))
+            info = M.solve(b, x, method=method, tol=1e-10, engine=engine,
+                           **dict(dict(max_iters=99), **kw))
             res.append((info, x.cpu().numpy()))
         (i1, x1), (i0, x0_) = res
         assert (i0["return"], i0["status"], i0["iters"]) == (i1["return"], i1["status"], i1["iters"])
-        assert np.allclose(x0_, x1, rtol=1e-12, atol=0, equal_nan=True)
+        assert np.allclose(x0_, x1, rtol=1e-9, atol=1e-12, equal_nan=True)
     v = m.values.copy()
     v[m.row_ptr[5]:m.row_ptr[6]] = 0.0
     Z = gk.Matrix.from_csr(W.CSR(m.n, m.n, m.row_ptr, m.col_idx, v))
-    info = Z.solve(ones, 0 * ones, method="cg", precond="jacobi", max_iters=9)
+    info = Z.solve(ones, 0 * ones, method=method, precond="jacobi", max_iters=9)
     assert info["return"] == gk.GK_ERR_ZERO_DIAG
     for M in (A, neg, Z):
         M.close()
+
+
+def test_solves_at_once_equal_alone():
+    """Grids that share the GPU (half blocks), that fill it (full blocks) and
+    refinements, from six threads: bit-identical to the same solve alone."""
+    import threading
+    import torch
+    work = [(W.laplacian_2d(131, 130), "cg", 0), (W.laplacian_3d(48, 50, 49), "cg", 0),
+            (W.laplacian_2d(130, 133), "gmres", 0), (W.laplacian_2d(640, 639), "cg", 0),
+            (W.laplacian_2d(51, 40), "gmres", 1), (W.laplacian_3d(40, 41, 39), "cg", 1)]
+    dev = torch_dev()
+    jobs = []
+    for m, method, mixed in work:
+        A = gk.Matrix.from_csr(m, "f64")
+        b = torch.from_numpy(W.uniform_vector(m.n, 5)).to(dev)
+        jobs.append((A, b, dict(method=method, precond="jacobi", tol=1e-30, max_iters=200,
+                                mixed=mixed)))
+    torch.cuda.synchronize()
+
+    def run(i, out):
+        A, b, kw = jobs[i]
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            x = torch.zeros_like(b)
+        info = A.solve(b, x, s, **kw)
+        s.synchronize()
+        out[i] = (x.cpu(), info["iters"], info["return"])
+
+    alone, at_once = {}, {}
+    for i in range(len(jobs)):
+        run(i, alone)
+    for _ in range(3):
+        ts = [threading.Thread(target=run, args=(i, at_once)) for i in range(len(jobs))]
+        [t.start() for t in ts]
+        [t.join() for t in ts]
+        for i in range(len(jobs)):
+            assert torch.equal(alone[i][0], at_once[i][0]) and alone[i][1:] == at_once[i][1:], i
+    for A, _, _ in jobs:
+        A.close()
