@@ -220,8 +220,33 @@ struct TriStore {
     int32_t wdist[2] = {1, 1};
     void* wrec = nullptr;
     void* wperm = nullptr;
+    // slab mode (slab = 1: picked): see SlabDir; buckets are nslab * nlev[.]
+    int32_t slab = 0, nslab = 0;
+    int32_t slev[2] = {0, 0}, scap[2] = {0, 0}, secap[2] = {0, 0}, snb[2] = {0, 0}, sterms[2] = {0, 0};
+    int32_t* srows[2] = {nullptr, nullptr};
+    int32_t* sstart[2] = {nullptr, nullptr};
+    int32_t* srange[2] = {nullptr, nullptr};
+    int32_t* sestart[2] = {nullptr, nullptr};
+    int32_t* sepos[2] = {nullptr, nullptr};
+    void* srec[2] = {nullptr, nullptr};
+    void* sperm = nullptr;          // level-ordered input
+    void* shand = nullptr;          // handed-over values
+    void release_slab() {
+        for (int u = 0; u < 2; ++u) {
+            for (int32_t** p : {&srows[u], &sstart[u], &srange[u], &sestart[u], &sepos[u]}) {
+                dfree(*p);
+                *p = nullptr;
+            }
+            dfree(srec[u]);
+            srec[u] = nullptr;
+        }
+        dfree(sperm);
+        dfree(shand);
+        sperm = shand = nullptr;
+    }
     DevBuf w;                       // scratch of one application
     void release() {
+        release_slab();
         dfree(lrows);
         dfree(lstart);
         dfree(wrec);

@@ -487,6 +487,225 @@ static gk_status build_win(TriStore* S, int32_t n, const IluLevels& lv, cudaStre
     return GK_OK;
 }
 
+// ------------------------------------------------------ slab-mode records
+// out[0], out[1]: most terms of a row, deepest dependency in levels; out[2]:
+// the farthest dependency in rows
+template <bool UP>
+__global__ void k_slab_check(int32_t n, const unsigned* __restrict__ lev,
+                             const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                             const int32_t* __restrict__ dpos, unsigned* out) {
+    unsigned nt = 0, md = 0, sp = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t d = dpos[i];
+        const int32_t k0 = UP ? d + 1 : rp[i], k1 = UP ? rp[i + 1] : d;
+        nt = max(nt, (unsigned)(k1 - k0));
+        for (int32_t k = k0; k < k1; ++k) {
+            md = max(md, lev[i] - lev[ci[k]]);
+            sp = max(sp, (unsigned)(UP ? ci[k] - (int32_t)i : (int32_t)i - ci[k]));
+        }
+    }
+    nt = __reduce_max_sync(0xffffffffu, nt);
+    md = __reduce_max_sync(0xffffffffu, md);
+    sp = __reduce_max_sync(0xffffffffu, sp);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, nt);
+        atomicMax(out + 1, md);
+        atomicMax(out + 2, sp);
+    }
+}
+
+// rows and fetched values of every bucket, the levels of every slab (range
+// starts at {INT32_MAX, -1})
+template <bool UP>
+__global__ void k_slab_count(int32_t n, int32_t R, int32_t nlev, const unsigned* __restrict__ lev,
+                             const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                             const int32_t* __restrict__ dpos, int32_t* cnt, int32_t* ecnt,
+                             int32_t* range) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t sl = (int32_t)i / R, l = (int32_t)lev[i] - 1;
+        const int64_t key = (int64_t)sl * nlev + l;
+        const int32_t d = dpos[i];
+        const int32_t k0 = UP ? d + 1 : rp[i], k1 = UP ? rp[i + 1] : d;
+        int32_t ne = 0;
+        for (int32_t k = k0; k < k1; ++k) ne += ci[k] / R != sl;
+        atomicAdd(cnt + key, 1);
+        if (ne) atomicAdd(ecnt + key, ne);
+        atomicMin(range + 2 * sl, l);
+        atomicMax(range + 2 * sl + 1, l);
+    }
+}
+
+__global__ void k_slab_widest(int64_t nk, const int32_t* __restrict__ cnt,
+                              const int32_t* __restrict__ ecnt, int32_t* out) {
+    int32_t a = 0, b = 0;
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nk;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        a = max(a, cnt[k]);
+        b = max(b, ecnt[k]);
+    }
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, a);
+        atomicMax(out + 1, b);
+    }
+}
+
+// cursor: a copy of the buckets' starts
+__global__ void k_slab_scatter(int32_t n, int32_t R, int32_t nlev, const unsigned* __restrict__ lev,
+                               int32_t* cursor, int32_t* __restrict__ rows, int32_t* __restrict__ pos) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t key = (int64_t)((int32_t)i / R) * nlev + (int32_t)lev[i] - 1;
+        const int32_t at = atomicAdd(cursor + key, 1);
+        rows[at] = (int32_t)i;
+        pos[i] = at;
+    }
+}
+
+// record of row rows[idx], and the fetched values it needs; ecursor: a copy
+// of the buckets' first fetched values
+template <typename T, bool UP>
+__global__ void k_slab_rec(int32_t n, int32_t R, int32_t nlev, int32_t cap, int32_t ecap,
+                           const int32_t* __restrict__ range, const int32_t* __restrict__ rows,
+                           const unsigned* __restrict__ lev, const int32_t* __restrict__ pos,
+                           const int32_t* __restrict__ start, const int32_t* __restrict__ estart,
+                           int32_t* ecursor, const int32_t* __restrict__ rp,
+                           const int32_t* __restrict__ ci, const int32_t* __restrict__ dpos,
+                           const T* __restrict__ lu, const T* __restrict__ rdiag,
+                           WinRec<T>* __restrict__ rec, int32_t* __restrict__ epos) {
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = rows[idx], sl = i / R, d = dpos[i];
+        const int64_t key = (int64_t)sl * nlev + (int32_t)lev[i] - 1;
+        WinRec<T> W;
+        W.rd = rdiag[i];
+        for (int t = 0; t < WIN_MAXT; ++t) {
+            W.co[t] = 0;
+            W.v[t] = T(0);
+        }
+        const int32_t nt = UP ? rp[i + 1] - 1 - d : d - rp[i];
+        for (int32_t t = 0; t < nt && t < WIN_MAXT; ++t) {
+            const int32_t k = UP ? rp[i + 1] - 1 - t : rp[i] + t;
+            const int32_t j = ci[k];
+            uint32_t co;
+            if (j / R == sl) {
+                const int64_t kj = (int64_t)sl * nlev + (int32_t)lev[j] - 1;
+                co = (uint32_t)(slab_ring_at((int32_t)lev[j] - 1 - range[2 * sl], cap, ecap) + pos[j] - start[kj]);
+            } else {
+                const int32_t e = atomicAdd(ecursor + key, 1);
+                epos[e] = pos[j];
+                co = (uint32_t)(slab_ext_at((int32_t)lev[i] - 1 - range[2 * sl], ecap) + e - estart[key]);
+            }
+            W.co[t] = (int16_t)co;
+            W.v[t] = lu[k];
+        }
+        rec[idx] = W;
+    }
+}
+
+// Builds the slab-mode data with about `want` slabs (whole multiples of the
+// farthest dependency, where that is shorter than a slab); *ok = false when
+// the matrix does not qualify: more than WIN_MAXT terms a row or
+// dependencies over WIN_MAXD levels back, too many rows or fetched values in
+// a bucket for shared memory, more than 8 buckets a row.  *rows: the rows of
+// a slab; nothing is built when that is `skip`.
+template <typename T>
+static gk_status build_slab(TriStore* S, int32_t n, const IluLevels& lv, int32_t want, int32_t skip,
+                            cudaStream_t s, int32_t* rows, bool* ok) {
+    *ok = false;
+    *rows = 0;
+    if (n == 0) return GK_OK;
+    const unsigned* lev[2] = {(const unsigned*)lv.l1.ptr, (const unsigned*)lv.u1.ptr};
+    const int32_t nlev[2] = {(int32_t)lv.nl1, (int32_t)lv.nu1};
+    const unsigned g = ew_grid(n);
+    TmpBuf misc;
+    GK_TRY(misc.ensure(64));
+    unsigned* mp = (unsigned*)misc.ptr;
+    GK_CUDA(cudaMemsetAsync(mp, 0, 64, s));
+    k_slab_check<false><<<g, 256, 0, s>>>(n, lev[0], S->rp, S->ci, S->dpos, mp);
+    k_slab_check<true><<<g, 256, 0, s>>>(n, lev[1], S->rp, S->ci, S->dpos, mp + 3);
+    GK_CUDA(cudaGetLastError());
+    unsigned h[6];
+    GK_CUDA(cudaMemcpyAsync(h, mp, sizeof(h), cudaMemcpyDeviceToHost, s));
+    GK_CUDA(cudaStreamSynchronize(s));
+    if (h[0] > WIN_MAXT || h[3] > WIN_MAXT || h[1] > WIN_MAXD || h[4] > WIN_MAXD) return GK_OK;
+    int64_t R = ((int64_t)n + want - 1) / want;
+    const int64_t span = std::max<int64_t>(1, std::max(h[2], h[5]));
+    if (R >= span) R = (R + span - 1) / span * span;
+    const int32_t nslab = (int32_t)(((int64_t)n + R - 1) / R);
+    if ((int64_t)nslab * std::max(nlev[0], nlev[1]) > 8 * (int64_t)n + 1024) return GK_OK;
+    *rows = (int32_t)R;
+    if (*rows == skip) return GK_OK;
+    S->nslab = nslab;
+    TmpBuf pos, cur, ecur, tmp;
+    GK_TRY(pos.ensure(sizeof(int32_t) * (size_t)n));
+    constexpr int AL = (int)(16 / sizeof(T));
+    GK_CUDA(dmalloc(&S->sperm, sizeof(T) * ((size_t)n + AL)));
+    GK_CUDA(dmalloc(&S->shand, sizeof(T) * (size_t)n));
+    std::vector<int32_t> hr(2 * (size_t)nslab);
+    for (int u = 0; u < 2; ++u) {
+        const size_t nk = (size_t)nslab * nlev[u];
+        S->slev[u] = nlev[u];
+        S->sterms[u] = (int32_t)h[3 * u];
+        GK_TRY(cur.ensure(sizeof(int32_t) * (nk + 1)));
+        GK_TRY(ecur.ensure(sizeof(int32_t) * (nk + 1)));
+        int32_t *cp = (int32_t*)cur.ptr, *ep = (int32_t*)ecur.ptr;
+        GK_CUDA(dmalloc_t(&S->srows[u], (size_t)n + 4));  // copied in 16-byte pieces
+        GK_CUDA(dmalloc_t(&S->sstart[u], nk + 1));
+        GK_CUDA(dmalloc_t(&S->sestart[u], nk + 1));
+        GK_CUDA(dmalloc_t(&S->srange[u], 2 * (size_t)nslab));
+        GK_CUDA(cudaMemsetAsync(cp, 0, sizeof(int32_t) * (nk + 1), s));
+        GK_CUDA(cudaMemsetAsync(ep, 0, sizeof(int32_t) * (nk + 1), s));
+        GK_CUDA(cudaMemsetAsync(mp, 0, 64, s));
+        for (int32_t k = 0; k < nslab; ++k) {
+            hr[2 * (size_t)k] = INT32_MAX;
+            hr[2 * (size_t)k + 1] = -1;
+        }
+        GK_CUDA(cudaMemcpyAsync(S->srange[u], hr.data(), sizeof(int32_t) * hr.size(),
+                                cudaMemcpyHostToDevice, s));
+        auto count = [&](auto k) {
+            k<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], lev[u], S->rp, S->ci, S->dpos, cp, ep,
+                                S->srange[u]);
+        };
+        u ? count(k_slab_count<true>) : count(k_slab_count<false>);
+        k_slab_widest<<<ew_grid((int64_t)nk), 256, 0, s>>>((int64_t)nk, cp, ep, (int32_t*)mp);
+        GK_CUDA(cudaGetLastError());
+        GK_TRY((scan_exclusive<int32_t, int32_t>(cp, S->sstart[u], (int64_t)nk, tmp, s)));
+        GK_TRY((scan_exclusive<int32_t, int32_t>(ep, S->sestart[u], (int64_t)nk, tmp, s)));
+        int32_t w[2], total = 0;
+        GK_CUDA(cudaMemcpyAsync(w, mp, sizeof(w), cudaMemcpyDeviceToHost, s));
+        GK_CUDA(cudaMemcpyAsync(&total, S->sestart[u] + nk, sizeof(total), cudaMemcpyDeviceToHost, s));
+        GK_CUDA(cudaStreamSynchronize(s));
+        if (w[0] > SLAB_CAP || w[1] > 65535 / SLAB_E) return GK_OK;
+        S->scap[u] = (w[0] + 31) / 32 * 32;
+        S->secap[u] = std::max(1, w[1]);
+        S->snb[u] = slab_values(S->scap[u], S->secap[u]) <= 65536 ? SLAB_NB : 0;  // 16-bit indices
+        while (S->snb[u] >= 2 && slab_smem<T>(S->scap[u], S->secap[u], S->snb[u]) > (size_t)SLAB_SMEM)
+            S->snb[u] -= SLAB_SW;  // whole rounds of the copying warps
+        if (S->snb[u] < 2) return GK_OK;
+        GK_CUDA(dmalloc_t(&S->sepos[u], (size_t)std::max(1, total)));
+        GK_CUDA(dmalloc(&S->srec[u], sizeof(WinRec<T>) * (size_t)n));
+        GK_CUDA(cudaMemcpyAsync(cp, S->sstart[u], sizeof(int32_t) * nk, cudaMemcpyDeviceToDevice, s));
+        GK_CUDA(cudaMemcpyAsync(ep, S->sestart[u], sizeof(int32_t) * nk, cudaMemcpyDeviceToDevice, s));
+        int32_t* pp = (int32_t*)pos.ptr;
+        k_slab_scatter<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], lev[u], cp, S->srows[u], pp);
+        auto fill = [&](auto k) {
+            k<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], S->scap[u], S->secap[u], S->srange[u],
+                                S->srows[u], lev[u], pp, S->sstart[u],
+                                S->sestart[u], ep, S->rp, S->ci, S->dpos, (const T*)S->lu,
+                                (const T*)S->rdiag, (WinRec<T>*)S->srec[u], S->sepos[u]);
+        };
+        u ? fill(k_slab_rec<T, true>) : fill(k_slab_rec<T, false>);
+        GK_CUDA(cudaGetLastError());
+    }
+    GK_CUDA(cudaStreamSynchronize(s));
+    *ok = true;
+    return GK_OK;
+}
+
 static gk_status build_row_levels(TriStore* S, int32_t n, const IluLevels& lv, cudaStream_t s) {
     if (S->lrows) return GK_OK;
     const size_t nl = lv.nl1, nu = lv.nu1;
@@ -543,6 +762,24 @@ static IluDev<T> tri_view(const TriStore* S, int32_t n) {
     f.wrec[0] = S->wrec;
     f.wrec[1] = S->wrec ? static_cast<const char*>(S->wrec) + sizeof(WinRec<T>) * (size_t)n : nullptr;
     f.wperm = static_cast<T*>(S->wperm);
+    f.slab = S->slab;
+    for (int u = 0; u < 2; ++u) {
+        SlabDir& D = f.sd[u];
+        D.nslab = S->nslab;
+        D.nlev = S->slev[u];
+        D.cap = S->scap[u];
+        D.ecap = S->secap[u];
+        D.nb = S->snb[u];
+        D.terms = S->sterms[u];
+        D.rows = S->srows[u];
+        D.start = S->sstart[u];
+        D.range = S->srange[u];
+        D.estart = S->sestart[u];
+        D.epos = S->sepos[u];
+        D.rec = S->srec[u];
+    }
+    f.sperm = static_cast<T*>(S->sperm);
+    f.shand = static_cast<T*>(S->shand);
     return f;
 }
 
@@ -572,13 +809,14 @@ template IluDev<float> ilu_view<float>(gk_matrix);
 template <typename T>
 static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaStream_t s) {
     int forced = 0;
-    bool forced_lvl = false, forced_win = false;
+    bool forced_lvl = false, forced_win = false, forced_slab = false;
     if (const char* e = getenv("GK_ILU_CHUNK")) {
         const int v = atoi(e);
         if (v == 1 || v == 8 || v == 32) forced = v;
         // the chunk state stays valid under a forced level-synchronous mode
         if (!strcmp(e, "lvl")) forced_lvl = true, forced = 32;
         if (!strcmp(e, "win")) forced_win = true, forced = 32;
+        if (!strcmp(e, "slab")) forced_slab = true, forced = 32;
     }
     int64_t mult = 2;
     if (const char* e = getenv("GK_ILU_WARPS")) mult = std::max(1, atoi(e));
@@ -702,6 +940,7 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
             if (forced_win) st = ws;
         } else if (ok) {
             win = forced_win || ms < best;
+            if (win) best = ms;
         }
         if (!win) {  // not picked: its records go
             dfree(S->wrec);
@@ -709,11 +948,67 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
             S->wrec = S->wperm = nullptr;
         }
     }
+    // the slab mode (the same matrices, see ilu_slab.cuh): two slab sizes,
+    // timed against the rest.  64 slabs are better where levels are narrow
+    // (2D 1024^2), 128 where the FP64 pipe bounds a level (128^3 FP64)
+    bool slab = false;
+    if (st == GK_OK && !lvl && (forced_slab || !forced)) {
+        const int want[2] = {64, 128};
+        int32_t built = 0, tried = 0;  // rows of the slab built last, of any tried
+        float slab_best = 0.f;
+        int32_t pick_want = 0, pick_rows = 0;
+        gk_status ss = GK_OK;
+        for (int k = 0; k < 3 && ss == GK_OK; ++k) {
+            // the last pass rebuilds the faster size, if it is not the one built
+            if (k == 2 && (!pick_want || pick_rows == built)) break;
+            bool ok = false;
+            int32_t rows = 0;
+            S->release_slab();
+            ss = build_slab<T>(S, n, lv, k < 2 ? want[k] : pick_want, k < 2 ? tried : 0, s, &rows, &ok);
+            if (ss != GK_OK || !ok) {
+                built = 0;
+                continue;
+            }
+            built = tried = rows;
+            if (k == 2) break;
+            IluDev<T> f = tri_view<T>(S, n);
+            f.slab = 1;
+            T* w = (T*)tmp.ptr;
+            const IluSrc<T> src{(const T*)S->rdiag};
+            float ms = 0.f;
+            ss = ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s);
+            if (ss == GK_OK && cudaEventRecord(e0, s) != cudaSuccess) ss = GK_ERR_CUDA;
+            if (ss == GK_OK)
+                ss = ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s);
+            if (ss == GK_OK && (cudaEventRecord(e1, s) != cudaSuccess ||
+                                cudaEventSynchronize(e1) != cudaSuccess ||
+                                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+                ss = GK_ERR_CUDA;
+            if (ss == GK_OK && (!pick_want || ms < slab_best)) {
+                slab_best = ms;
+                pick_want = want[k];
+                pick_rows = rows;
+            }
+        }
+        if (ss == GK_OK && built && pick_want) slab = forced_slab || slab_best < best;
+        if (ss != GK_OK) {
+            cudaGetLastError();  // no room for the records: keep the other mode
+            if (forced_slab) st = ss;
+        }
+        if (!slab) S->release_slab();
+        if (slab && win) {
+            dfree(S->wrec);
+            dfree(S->wperm);
+            S->wrec = S->wperm = nullptr;
+            win = false;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != GK_OK) return st;
     S->lvl = lvl ? 1 : 0;
     S->win = win ? 1 : 0;
+    S->slab = slab ? 1 : 0;
     TrsvSync h[2];
     GK_CUDA(cudaMemcpyAsync(h, S->sync, sizeof(h), cudaMemcpyDeviceToHost, s));
     GK_CUDA(cudaStreamSynchronize(s));

@@ -71,6 +71,22 @@ struct TrsvSync {
     unsigned pad;
 };
 
+// One triangle in slab mode (ilu_slab.cuh): rows sorted by slab, then level;
+// bucket (slab, level) at slab * nlev + level (levels from 0)
+struct SlabDir {
+    int32_t nslab = 0, nlev = 0;
+    int32_t cap = 0;   // rows of a bucket at most (rounded up to a multiple of 32)
+    int32_t ecap = 0;  // values from other slabs a bucket needs, at most
+    int32_t nb = 0;    // levels of records in flight
+    int32_t terms = 0; // terms of a row at most
+    const int32_t* rows = nullptr;    // n
+    const int32_t* start = nullptr;   // first row of each bucket, and n
+    const int32_t* range = nullptr;   // first and last level of each slab
+    const int32_t* estart = nullptr;  // first fetched value of each bucket, and their number
+    const int32_t* epos = nullptr;    // their positions in the order of rows
+    const void* rec = nullptr;        // WinRec<T>[n] in that order
+};
+
 // Device view of one ILU(0) factorisation with values of type T.
 template <typename T>
 struct IluDev {
@@ -103,6 +119,12 @@ struct IluDev {
     int32_t wdist[2] = {1, 1};           // deepest dependency, in levels
     const void* wrec[2] = {nullptr, nullptr};  // WinRec<T>[n] each
     T* wperm = nullptr;                  // n
+    // slab mode (slab != 0): both triangles, the level-ordered input and the
+    // values handed from slab to slab
+    int32_t slab = 0;
+    SlabDir sd[2];
+    T* sperm = nullptr;
+    T* shand = nullptr;
 };
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
@@ -881,6 +903,12 @@ static gk_status perm_gather(const IluDev<T>& f, bool up, Src src, Skip sk, cuda
     return GK_OK;
 }
 
+}  // namespace gk
+
+#include "ilu_slab.cuh"
+
+namespace gk {
+
 // One level-synchronous substitution: a single cluster of CLT_BLOCKS blocks.
 template <typename T, bool UP, class Src, class Out, class Skip>
 static gk_status launch_clt(const IluDev<T>& f, Src src, Out out, Skip sk, cudaStream_t s) {
@@ -906,6 +934,10 @@ template <typename T, class Src, class Out, class Skip, class Err>
 static gk_status ilu_apply(const IluDev<T>& f, Src src, T* w, Out out, Skip sk, Err on_err,
                            cudaStream_t s) {
     if (f.n == 0) return GK_OK;
+    if (f.slab) {
+        GK_TRY((launch_slab<T, false>(f, src, IluOutStore<T>{w}, sk, IluNoErr{}, s)));
+        return launch_slab<T, true>(f, IluSrc<T>{w}, out, sk, on_err, s);
+    }
     if (f.win) {
         GK_TRY((perm_gather<T>(f, false, src, sk, s)));
         GK_TRY((launch_win<T, false>(f, IluOutStore<T>{w}, sk, IluNoErr{}, s)));
@@ -933,6 +965,11 @@ static gk_status ilu_apply(const IluDev<T>& f, Src src, T* w, Out out, Skip sk, 
 template <typename T>
 static gk_status tri_apply(const IluDev<T>& f, bool up, const T* src, T* x, cudaStream_t s) {
     if (f.n == 0) return GK_OK;
+    if (f.slab) {
+        const IluOutStore<T> o{x};
+        if (up) return launch_slab<T, true>(f, IluSrc<T>{src}, o, IluSkipNever{}, IluNoErr{}, s);
+        return launch_slab<T, false>(f, IluSrc<T>{src}, o, IluSkipNever{}, IluNoErr{}, s);
+    }
     if (f.win) {
         GK_TRY((perm_gather<T>(f, up, IluSrc<T>{src}, IluSkipNever{}, s)));
         if (up) return launch_win<T, true>(f, IluOutStore<T>{x}, IluSkipNever{}, IluNoErr{}, s);
