@@ -43,14 +43,20 @@ constexpr int GRID_AHEAD = 2;
 // two solves at once can share (one's arithmetic runs in the other's waits).
 // Both at 64 registers a thread.
 constexpr int GRID_FULL = 1024, GRID_HALF = 512;
-// The half size up to these rows and matrix entries a block.  Alone (FP64,
-// us per iteration of Jacobi-CG and step of Jacobi-GMRES(30), full / half):
-// n = 17,030 8.8 / 8.2 and 46.9 / 35.9, 117,453 12.3 / 12.3 and 57.3 / 49.7,
-// 300,763 18.1 / 17.9 and 86 / 76, 512,000 24.9 / 25.5 and 113 / 113, 10^6
-// 38.6 / 43.6 and 183 / 195; with 33 entries a row 300,000 36.7 / 41.1 and
-// 110 / 113, with 121 entries a row 90 / 106 and 171 / 208.  Six CG solves of
-// 70K to 430K rows at once: all full 57 ms, with this line 49 ms.
-constexpr int64_t GRID_HALF_ROWS = 2048, GRID_HALF_ENTRIES = 32768;
+// The half size up to these rows a block, where the vectors fit (CG in FP64
+// to 3,400 rows a block, n = 520,000; FP32 to 1,000,000).  Alone (FP64, us per
+// iteration of Jacobi-CG and step of Jacobi-GMRES(30), full / half): n = 17,030
+// 8.8 / 8.2 and 46.9 / 35.9, 117,453 12.3 / 12.3 and 57.3 / 49.7, 300,763 18.1 /
+// 17.9 and 86 / 76, 512,000 24.9 / 25.5 and 113 / 112; with 33 entries a row
+// 300,000 36.7 / 41.0 and 110 / 113, with 121 entries a row 90 / 106 and 171 /
+// 208 (multi-kernel 154 and 202); FP32 CG 10^6 18.2 / 22.9 (34.7).  What a lone
+// solve loses there, a serving mix (24 matrices of 1e3 to 1e6 rows, six
+// workers) gains: solves per second at saturation, and p50 / p99 in ms at 0.8
+// of it: multi-kernel 100, 103 / 966; half to 2,048 rows and 32,768 entries
+// 96, 111 / 619; to 4,096 rows 104, 114 / 694; to 8,192 111, 65 / 618.  GMRES
+// takes the half size where it is not the slower one alone.
+constexpr int64_t GRID_HALF_ROWS = 8192;
+constexpr int64_t GRID_GM_HALF_ROWS = 4096, GRID_GM_HALF_ENTRIES = 131072;
 // The least rows of a block, in bytes of a vector: fewer blocks leave SMs to
 // other solves and make the hand-offs cheaper.  Six solves of 17K to 25K rows
 // at once, 64 / 256 / 512 rows a block: FP64 CG 17.6 / 12.0 / 12.1 ms with
@@ -394,7 +400,7 @@ inline gk_status grid_plan(gk_matrix M, SolverCache* C, int nc, GridPlan* P) {
     GK_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     // less the kernels' static shared memory, and 1 KB the system keeps of each block
     P->room[0] = (int64_t)optin - 1024;
-    P->room[1] = P->R <= GRID_HALF_ROWS && P->R * M->K <= GRID_HALF_ENTRIES ? ((int64_t)optin + 1024) / 2 - 2048 : 0;
+    P->room[1] = P->R <= GRID_HALF_ROWS ? ((int64_t)optin + 1024) / 2 - 2048 : 0;
     if (!coop || (uint64_t)(M->K + 8) * (uint64_t)M->stride * value_bytes(M->dtype) >= (1ull << 32))
         return GK_ERR_UNSUPPORTED;
     P->slot_bytes = (sizeof(unsigned long long) * GRID_ROUNDS * (GRID_VALUES + 2 * (size_t)nc) *

@@ -9,8 +9,8 @@
 // stencil 22.3 / 12.3 (2.6), 10^6-row 3D stencil 59.9 / 38.6 (22), 128^3
 // diffusion 98 / 71 (47), in FP32 56 / 32; 121 entries a row, n = 30,000:
 // 75.6 / 24.5, n = 500,000: 316 / 155.  Six solves at once, 600 iterations
-// each: 17K to 25K rows 25.5 / 12.1 ms, 70K to 430K rows 47 / 49 ms (alone,
-// in turn: 74 / 30 and 105 / 58).  What is left on small matrices is latency: the block's FP64 tree (~2,300 cycles a
+// each: 17K to 25K rows 25.5 / 12.1 ms, 70K to 430K rows 47 / 48 ms (alone,
+// in turn: 74 / 30 and 105 / 60).  What is left on small matrices is latency: the block's FP64 tree (~2,300 cycles a
 // reduction), the hand-offs (~1,700 to 2,600 each) and FP64 divisions; on
 // large ones the FP64 pipe (128^3: 97,000 of 153,000 cycles).
 //
@@ -254,7 +254,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     GK_TRY(grid_plan(M, C, 0, &P));
     int mode = 0;
     while (mode < 2 && (int64_t)grid_cg_smem<GRID_HALF, V, T>(mode, P.R, M->K) > P.room[1]) ++mode;
-    P.half = mode < 2;  // GRID_HALF_ROWS rows of four vectors always fit
+    P.half = mode < 2;
     if (!P.half) {
         mode = 0;
         while (mode < 3 && (int64_t)grid_cg_smem<GRID_FULL, V, T>(mode, P.R, M->K) > P.room[0]) ++mode;

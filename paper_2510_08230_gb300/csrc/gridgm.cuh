@@ -478,7 +478,8 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     GK_TRY(get_cache(M, &C));
     GridPlan P;
     GK_TRY(grid_plan(M, C, m + 1, &P));
-    P.half = (int64_t)grid_gm_smem<GRID_HALF, V, T>(false, m, P.R, M->K) <= P.room[1];
+    P.half = P.R <= GRID_GM_HALF_ROWS && P.R * M->K <= GRID_GM_HALF_ENTRIES &&
+             (int64_t)grid_gm_smem<GRID_HALF, V, T>(false, m, P.R, M->K) <= P.room[1];
     auto smem_of = [&](bool st) {
         return P.half ? grid_gm_smem<GRID_HALF, V, T>(st, m, P.R, M->K)
                       : grid_gm_smem<GRID_FULL, V, T>(st, m, P.R, M->K);

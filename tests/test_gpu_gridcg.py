@@ -33,8 +33,10 @@ FIXED = {
     "mode0_large": lambda: W.laplacian_2d(601, 599),
     "mode1_wide": lambda: W.banded_spd(40001, 60, 3),     # 121 entries a row
     "mode1": lambda: W.laplacian_1d(900001),
-    "half_limit": lambda: W.laplacian_2d(608, 512),       # 2,048 rows a block: the last half grid
+    "half_limit": lambda: W.laplacian_2d(608, 512),       # 2,048 rows a block
     "half_mode1": lambda: W.banded_spd(60001, 12, 4),     # 25 entries a row
+    "half_last": lambda: W.laplacian_1d(152 * 3392),      # FP64: the last half grid of CG
+    "full_first": lambda: W.laplacian_1d(152 * 3520 + 1),
     "mode2": lambda: W.laplacian_1d(1200001),             # FP64 only: 7,936 rows a block
 }
 
