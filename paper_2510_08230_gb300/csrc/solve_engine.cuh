@@ -1956,7 +1956,7 @@ static __global__ void k_write_info(const KState* st, gk_solve_info* info, const
 
 struct SolverCache {
     DevBuf vecs, partials, ticket, state;
-    DevBuf gvecs, gsync;    // k_grid_cg: its vectors; its hand-off slots and outcome
+    DevBuf gvecs, gsync;    // the grid kernels: their vectors; their hand-off slots and outcome
     KState* hst = nullptr;  // pinned mirror of the state header
     int32_t* hzero = nullptr;
     cudaGraphExec_t exec = nullptr;
