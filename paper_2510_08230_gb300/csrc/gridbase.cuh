@@ -21,6 +21,7 @@
 // are spread over the sub-partitions and scalars are formed by one lane.
 #pragma once
 
+#include "grid_limits.h"
 #include "solve_engine.cuh"
 
 namespace gk {
@@ -387,8 +388,7 @@ struct GridPlan {
 };
 
 // GK_ERR_UNSUPPORTED: no cooperative launches, or the kernels' 32-bit byte
-// offsets do not reach the whole matrix (a chunk of 8 entries past the last is
-// formed, not read).
+// offsets do not reach the whole matrix.
 inline gk_status grid_plan(gk_matrix M, SolverCache* C, int nc, GridPlan* P) {
     const int sms = std::min(num_sms(), GRID_MAX_BLOCKS);
     P->R = std::max<int64_t>(GRID_MIN_ROW_BYTES / (int64_t)vector_bytes(M->dtype),
@@ -401,7 +401,7 @@ inline gk_status grid_plan(gk_matrix M, SolverCache* C, int nc, GridPlan* P) {
     // less the kernels' static shared memory, and 1 KB the system keeps of each block
     P->room[0] = (int64_t)optin - 1024;
     P->room[1] = P->R <= GRID_HALF_ROWS ? ((int64_t)optin + 1024) / 2 - 2048 : 0;
-    if (!coop || (uint64_t)(M->K + 8) * (uint64_t)M->stride * value_bytes(M->dtype) >= (1ull << 32))
+    if (!coop || !grid_offsets_fit(M->K, M->stride, (int64_t)value_bytes(M->dtype)))
         return GK_ERR_UNSUPPORTED;
     P->slot_bytes = (sizeof(unsigned long long) * GRID_ROUNDS * (GRID_VALUES + 2 * (size_t)nc) *
                          GRID_MAX_BLOCKS + 255) & ~(size_t)255;
