@@ -317,7 +317,7 @@ struct gk_matrix_s {
     // first use (ilu.cu)
     gk::TriStore* ilu = nullptr;
     gk::TriStore* tri = nullptr;
-    gk_matrix_s* lowp[3] = {nullptr, nullptr, nullptr};  // same layout, other dtype
+    gk_matrix_s* lowp[4] = {};  // same layout, other dtype (by gk_dtype)
     gk_matrix_s* solve_fmt = nullptr;  // SpMV layout picked for solves (null: not tuned)
     int solve_fmt_tuned = 0;
     gk::SolverCache* solver = nullptr;

@@ -798,7 +798,7 @@ static gk_status ensure_words(gk_matrix A) {
 
 static void destroy_handle(gk_matrix A) {
     if (!A) return;
-    for (int i = 0; i < 3; ++i) destroy_handle(A->lowp[i]);
+    for (gk_matrix L : A->lowp) destroy_handle(L);
     if (A->solve_fmt != A) destroy_handle(A->solve_fmt);
     free_solver_cache(A);
     free_arrays(A);
