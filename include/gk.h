@@ -257,7 +257,11 @@ typedef struct {
                              waits on its staged copies) before it gives up: the solve
                              then returns GK_ERR_TIMEOUT and x holds no valid
                              iterate.  0 = the default of 2 s; negative values
-                             are GK_ERR_INVALID */
+                             are GK_ERR_INVALID.  When a hand-off between the
+                             blocks of a persistent kernel takes longer (it is
+                             microseconds, unless other work keeps a block off
+                             the GPU), engine 1 solves from the initial guess
+                             instead */
 } gk_solve_opts;
 
 typedef struct {

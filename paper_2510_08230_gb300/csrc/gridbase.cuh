@@ -14,7 +14,11 @@
 // counter 2,500, stores 4,300.  Slots come in three rounds (a publication
 // ends a round); a block empties its slots of round k + 1 before it publishes
 // in round k: by then every block has left round k - 2, which used them.
-// Every poll is bounded.
+// Every poll is bounded by the solve's wait budget.  A wait can run out
+// although no block is lost: other work may hold an SM that a block of the
+// grid still needs.  Then every block leaves, the error word tells the host
+// (a block that had finished does not know), the caller's x is untouched and
+// the multi-kernel engine, whose kernels wait for nothing, solves instead.
 //
 // FP64: a warp instruction holds its sub-partition's pipe for 65 cycles
 // whatever its mask (16 cycles of the SM with all four busy), so block sums
@@ -64,6 +68,9 @@ constexpr int64_t GRID_GM_HALF_ROWS = 4096, GRID_GM_HALF_ENTRIES = 131072;
 // 8.5 / 8.2 / 8.6 us per iteration alone; inner FP32 solves 16.8 / 11.2 /
 // 8.5 ms with 8.0 / 7.4 / 7.4 us.
 constexpr int64_t GRID_MIN_ROW_BYTES = 2048;
+
+// Budgets below this have the clock read at every poll.
+constexpr uint64_t GRID_SHORT_BUDGET_NS = 10000000;
 
 // why a solve ends (0: it goes on); PASSED, CYCLE: a recurrence residual
 // passed, a GMRES cycle ended
@@ -129,13 +136,15 @@ struct GridTeam {
     }
 
     // A warp spins until ready() holds in all lanes; false: the budget ran
-    // out, here or elsewhere.
+    // out, here or elsewhere.  The clock is read every 256 polls (one of ~700
+    // cycles), or with a budget that this would overrun at every poll.
     template <class F>
     __device__ __forceinline__ bool wait(F&& ready) const {
+        const unsigned between = wait_ns < GRID_SHORT_BUDGET_NS ? 0u : 255u;
         uint64_t t0 = 0;
         for (unsigned spin = 0;; ++spin) {
             if (__all_sync(0xffffffffu, ready())) return true;
-            if ((spin & 255u) != 255u) continue;
+            if ((spin & between) != between) continue;
             bool stop = false;
             if ((threadIdx.x & 31) == 0) {
                 const uint64_t t = globaltimer_ns();
@@ -433,25 +442,43 @@ gk_status grid_launch(K kern, A& args, const GridPlan& P, size_t smem, cudaStrea
     return GK_OK;
 }
 
-// Runs launch() when the GPU has seats for its grid, and reads the outcome.
-// The stream is drained first and last: seats are held for the solve alone.
+// Runs launch() when the GPU has seats for its grid, reads the outcome and
+// copies the solution from `from` to x (bytes).  The stream is drained first
+// and before the seats are given back: they are held for the solve alone.
+// GK_ERR_UNSUPPORTED: a wait ran out; x is as it was.
 template <class F>
-gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* out, F&& launch) {
-    static_assert(sizeof(GridOut) <= HDR, "the pinned header holds the outcome");
-    GridOut* h = reinterpret_cast<GridOut*>(C->hst);
+gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* out, void* x,
+                   const void* from, size_t bytes, F&& launch) {
+    struct Outcome {
+        int32_t err, pad[15];
+        GridOut o;
+    };
+    static_assert(sizeof(Outcome) <= HDR, "the pinned header holds the outcome");
+    Outcome* h = reinterpret_cast<Outcome*>(C->hst);
     GK_CUDA(cudaStreamSynchronize(s));
     {
         GridSeats seats(P.half, P.nb);
         GK_TRY(launch());
-        GK_CUDA(cudaMemcpyAsync(h, P.out(), sizeof(GridOut), cudaMemcpyDeviceToHost, s));
+        GK_CUDA(cudaMemcpyAsync(h, P.err(), sizeof(Outcome), cudaMemcpyDeviceToHost, s));
         GK_CUDA(cudaStreamSynchronize(s));
     }
-    out->status = (gk_status)h->status;
-    out->iters = h->iters;
-    out->restarts = h->restarts;
-    out->rec = h->rec;
-    out->tru = h->tru;
+    if (h->err != 0 || h->o.status == GK_ERR_TIMEOUT) return GK_ERR_UNSUPPORTED;
+    GK_CUDA(cudaMemcpyAsync(x, from, bytes, cudaMemcpyDeviceToDevice, s));
+    out->status = (gk_status)h->o.status;
+    out->iters = h->o.iters;
+    out->restarts = h->o.restarts;
+    out->rec = h->o.rec;
+    out->tru = h->o.tru;
     return GK_OK;
+}
+
+// The kernels' vectors; GK_ERR_UNSUPPORTED when there is no room for them
+// (the handle may hold the multi-kernel engine's already).
+inline gk_status grid_vectors(SolverCache* C, size_t bytes) {
+    const gk_status st = C->gvecs.ensure(bytes);
+    if (st != GK_ERR_OOM) return st;
+    cudaGetLastError();
+    return GK_ERR_UNSUPPORTED;
 }
 
 }  // namespace gk

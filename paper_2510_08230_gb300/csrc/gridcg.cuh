@@ -34,7 +34,7 @@ struct GridCgArgs {
     const V* val;
     const T* b;
     const T* x0;   // the initial guess
-    T* x;          // the solution; mode 2 works on it (padded to whole blocks)
+    T* x;          // the solution, padded to whole blocks; mode 2 works on it
     const T* dinv; // null: no preconditioner
     T* p;          // gathered vector, padded to whole blocks
     unsigned long long *slots, *arrived;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(NT, GRID_FULL / NT) k_grid_cg(const GridCgArgs
         return team.sum<1>(1, v, [&](const double* t) {
                    S.rho = t[0];
                    return 0;
-               }) >= 0 && team.publish();
+               }) == 0 && team.publish();
     };
     // x into A.p, published
     auto publish_x = [&]() -> bool {
@@ -242,8 +242,9 @@ __global__ void __launch_bounds__(NT, GRID_FULL / NT) k_grid_cg(const GridCgArgs
 
 // ------------------------------------------------------------ host side
 
-// One CG solve on k_grid_cg.  GK_ERR_UNSUPPORTED: the matrix is too large
-// for the blocks' shared memory, or the grid cannot be resident at once.
+// One CG solve on k_grid_cg.  GK_ERR_UNSUPPORTED, with x untouched: the matrix
+// is too large for the blocks' shared memory, there is no room for the
+// vectors, the grid cannot be resident at once, or a wait ran out.
 template <typename V, typename T>
 gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, int32_t max_iters,
                         cudaStream_t s, SolveOut* out, bool inner) {
@@ -263,7 +264,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     const bool prec = pkind == 1;
     if (prec) GK_TRY(ensure_jacobi(M, s));
     const size_t vbytes = ((size_t)P.nb * P.R * sizeof(T) + 255) & ~(size_t)255;
-    GK_TRY(C->gvecs.ensure(vbytes * (mode == 2 ? 2 : 1)));
+    GK_TRY(grid_vectors(C, vbytes * 2));
     GridCgArgs<V, T> a;
     a.n = n;
     a.R = (int32_t)P.R;
@@ -273,7 +274,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     a.val = (const V*)M->val;
     a.b = b;
     a.x0 = x;
-    a.x = mode == 2 ? (T*)(static_cast<char*>(C->gvecs.ptr) + vbytes) : x;
+    a.x = (T*)(static_cast<char*>(C->gvecs.ptr) + vbytes);
     a.dinv = prec ? (const T*)M->dinv : nullptr;
     a.p = (T*)C->gvecs.ptr;
     a.slots = P.slots();
@@ -284,9 +285,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     a.max_iters = max_iters;
     a.inner = inner ? 1 : 0;
     a.stall = inner ? 200 : 0;
-    // the hand-offs between blocks take microseconds; a budget below the
-    // default must not fail a solve that waits for nothing else
-    a.wait_ns = std::max<uint64_t>(M->wait_ns, WAIT_LIMIT_NS);
+    a.wait_ns = M->wait_ns;
     auto go = [&](auto nt, auto md) -> gk_status {
         constexpr int NT = decltype(nt)::value, MD = decltype(md)::value;
         const size_t smem = grid_cg_smem<NT, V, T>(MD, P.R, M->K);
@@ -298,14 +297,11 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     constexpr std::integral_constant<int, 0> m0;
     constexpr std::integral_constant<int, 1> m1;
     constexpr std::integral_constant<int, 2> m2;
-    return grid_run(C, P, s, out, [&]() -> gk_status {
-        GK_TRY(P.half      ? (mode == 0 ? go(half, m0) : go(half, m1))
+    return grid_run(C, P, s, out, x, a.x, sizeof(T) * (size_t)n, [&]() -> gk_status {
+        return P.half      ? (mode == 0 ? go(half, m0) : go(half, m1))
                : mode == 0 ? go(full, m0)
                : mode == 1 ? go(full, m1)
-                           : go(full, m2));
-        if (mode == 2)
-            GK_CUDA(cudaMemcpyAsync(x, a.x, sizeof(T) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        return GK_OK;
+                           : go(full, m2);
     });
 }
 

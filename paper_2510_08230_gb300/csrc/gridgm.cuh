@@ -468,8 +468,9 @@ __global__ void __launch_bounds__(NT, GRID_FULL / NT) k_grid_gmres(const GridGmA
 
 // ------------------------------------------------------------ host side
 
-// One GMRES(m) solve on k_grid_gmres.  GK_ERR_UNSUPPORTED: a block's rows of w
-// do not fit its shared memory, or the grid cannot be resident at once.
+// One GMRES(m) solve on k_grid_gmres.  GK_ERR_UNSUPPORTED, with x untouched: a
+// block's rows of w do not fit its shared memory, there is no room for the
+// basis, the grid cannot be resident at once, or a wait ran out.
 template <typename V, typename T>
 gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol, int32_t max_iters,
                            int m, cudaStream_t s, SolveOut* out, bool inner) {
@@ -491,7 +492,7 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     if ((int64_t)smem > room) return GK_ERR_UNSUPPORTED;
     const bool prec = pkind == 1;
     if (prec) GK_TRY(ensure_jacobi(M, s));
-    GK_TRY(C->gvecs.ensure(vbytes * (size_t)(m + 3)));
+    GK_TRY(grid_vectors(C, vbytes * (size_t)(m + 3)));
     char* v = static_cast<char*>(C->gvecs.ptr);
     GridGmArgs<V, T> a;
     a.n = n;
@@ -515,7 +516,7 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     a.tol = tol;
     a.max_iters = max_iters;
     a.stag = inner ? 0.95 : 0.0;
-    a.wait_ns = std::max<uint64_t>(M->wait_ns, WAIT_LIMIT_NS);  // as solve_grid_cg
+    a.wait_ns = M->wait_ns;
     auto go = [&](auto nt, auto st) -> gk_status {
         constexpr int NT = decltype(nt)::value;
         constexpr bool ST = decltype(st)::value;
@@ -525,11 +526,9 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     auto go_staged = [&](auto nt) -> gk_status {
         return staged ? go(nt, std::true_type{}) : go(nt, std::false_type{});
     };
-    return grid_run(C, P, s, out, [&]() -> gk_status {
-        GK_TRY(P.half ? go_staged(std::integral_constant<int, GRID_HALF>{})
-                      : go_staged(std::integral_constant<int, GRID_FULL>{}));
-        GK_CUDA(cudaMemcpyAsync(x, a.x, sizeof(T) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        return GK_OK;
+    return grid_run(C, P, s, out, x, a.x, sizeof(T) * (size_t)n, [&]() -> gk_status {
+        return P.half ? go_staged(std::integral_constant<int, GRID_HALF>{})
+                      : go_staged(std::integral_constant<int, GRID_FULL>{});
     });
 }
 
