@@ -26,6 +26,7 @@
 #pragma once
 
 #include "grid_limits.h"
+#include "grid_seats.h"
 #include "solve_engine.cuh"
 
 namespace gk {
@@ -359,7 +360,8 @@ struct GridRows {
 // half of one (threads and registers; shared memory at most that), so one
 // full grid, or half grids of together no more blocks than 2 an SM, are
 // resident at once wherever the blocks land: no grid is launched that would
-// have to wait for another's blocks.  First come, first served.
+// have to wait for another's blocks.  First come, first served, on each
+// device by itself (the current one).
 class GridSeats {
 public:
     GridSeats(bool half, int blocks);
@@ -368,6 +370,7 @@ public:
     GridSeats& operator=(const GridSeats&) = delete;
 
 private:
+    SeatPool* pool_;
     int seats_;
 };
 

@@ -2,8 +2,6 @@
 // SpMV layout, FP64 iterative refinement around FP32 / BF16-stored inner
 // solves) and the host-side helpers of the multi-kernel engine
 // (solve_engine.cuh).
-#include <condition_variable>
-
 #include "gridcg.cuh"
 #include "gridgm.cuh"
 
@@ -239,38 +237,18 @@ gk_status read_hdr(SolverCache* C, cudaStream_t s) {
     return GK_OK;
 }
 
-namespace {
-struct Seats {
-    std::mutex mu;
-    std::condition_variable freed;
-    uint64_t next_ticket = 0, serving = 0;
-    int used = 0;
-};
-Seats& seats() {
-    static Seats* s = new Seats;  // outlives threads still in a solve at exit
-    return *s;
-}
-}  // namespace
-
-GridSeats::GridSeats(bool half, int blocks) : seats_(half ? blocks : 2 * num_sms()) {
-    Seats& g = seats();
-    std::unique_lock<std::mutex> lk(g.mu);
-    const uint64_t ticket = g.next_ticket++;
-    g.freed.wait(lk, [&] { return g.serving == ticket && g.used + seats_ <= 2 * num_sms(); });
-    g.used += seats_;
-    ++g.serving;
-    lk.unlock();
-    g.freed.notify_all();
+GridSeats::GridSeats(bool half, int blocks) {
+    static SeatPools* pools = new SeatPools;  // outlives threads still in a solve at exit
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, 1);
+    pool_ = &pools->of(dev);
+    seats_ = half ? std::min(blocks, 2 * sms) : 2 * sms;
+    pool_->take(seats_, 2 * sms);
 }
 
-GridSeats::~GridSeats() {
-    Seats& g = seats();
-    {
-        std::lock_guard<std::mutex> lk(g.mu);
-        g.used -= seats_;
-    }
-    g.freed.notify_all();
-}
+GridSeats::~GridSeats() { pool_->give(seats_); }
 
 gk_status clear_halt(SolverCache* C, cudaStream_t s) {
     KState* st = (KState*)C->state.ptr;

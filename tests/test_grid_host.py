@@ -3,6 +3,8 @@ C++ headers with the host compiler.  CPU only."""
 import ctypes
 import os
 import subprocess
+import threading
+import time
 
 import pytest
 
@@ -46,3 +48,50 @@ def test_offsets_of_values_and_columns_fit_32_bits(limits, value_bytes):
     assert not limits(601, 1 << 21, value_bytes)  # 609 * 2^21 * 2 < 2^32 < 601 * 2^21 * 4
     assert not limits(270, 4 << 20, value_bytes)
     assert limits(7, 1 << 21, value_bytes)
+
+
+@pytest.fixture(scope="module")
+def seats(tmp_path_factory):
+    lib = _compile(tmp_path_factory, "seats", '#include "grid_seats.h"\n'
+                   'static gk::SeatPools pools;\n'
+                   'extern "C" float take(int d, int n, int cap) { return pools.of(d).take(n, cap); }\n'
+                   'extern "C" void give(int d, int n) { pools.of(d).give(n); }\n')
+    lib.take.restype = ctypes.c_float
+    return lib
+
+
+def test_seats_are_a_device_s_own(seats):
+    """A device whose seats are all taken does not keep another one's solves
+    waiting."""
+    assert seats.take(0, 304, 304) == 0.0
+    done = threading.Event()
+    t = threading.Thread(target=lambda: (seats.take(1, 304, 304), seats.take(2, 100, 264),
+                                         done.set()), daemon=True)
+    t.start()
+    assert done.wait(5)
+    for d, n in ((0, 304), (1, 304), (2, 100)):
+        seats.give(d, n)
+
+
+def test_seats_in_order_of_arrival(seats):
+    """On one device a large request is not overtaken by later small ones,
+    and the wait it reports is the time it queued."""
+    assert seats.take(3, 200, 304) == 0.0
+    order, waited = [], {}
+
+    def ask(name, n):
+        waited[name] = seats.take(3, n, 304)
+        order.append(name)
+        seats.give(3, n)
+
+    ts = []
+    for name, n in (("large", 304), ("small", 50)):
+        ts.append(threading.Thread(target=ask, args=(name, n), daemon=True))
+        ts[-1].start()
+        time.sleep(0.2)
+    assert order == []
+    seats.give(3, 200)
+    for t in ts:
+        t.join(5)
+    assert order == ["large", "small"]
+    assert waited["large"] >= 300 and waited["small"] >= 150
