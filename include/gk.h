@@ -271,7 +271,8 @@ typedef struct {
     int32_t outer_iters;      /* refinement steps (0 without refinement) */
     double rel_res_recurrence;/* last recurrence / Givens estimate over ||b|| */
     double rel_res_true;      /* ||b - A x||_2 / ||b||_2 recomputed at exit */
-    float device_ms;          /* device time of the solve (CUDA events) */
+    float device_ms;          /* device time of the solve (CUDA events), less the time it
+                                 queued for other solves' persistent kernels */
     int32_t spmv_format;      /* layout the solve's SpMV ran on (GK_CSR, GK_ELL or
                                  GK_SELLP; refinement: the FP64 residual's) */
     int32_t slice_size;       /* SELL-P slice size of that layout, else 0 */

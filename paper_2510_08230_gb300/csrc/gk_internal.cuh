@@ -273,6 +273,7 @@ struct SolveOut {
     int32_t iters = 0, restarts = 0;
     double rec = 0.0, tru = 0.0;
     int32_t layout = GK_CSR, slice = 0, threads = 0;  // the SpMV layout and block size used
+    float queued_ms = 0.f;  // host time spent waiting for other solves' grids
 };
 
 }  // namespace gk

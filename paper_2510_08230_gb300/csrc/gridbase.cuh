@@ -368,6 +368,7 @@ public:
     ~GridSeats();
     GridSeats(const GridSeats&) = delete;
     GridSeats& operator=(const GridSeats&) = delete;
+    float waited_ms = 0.f;  // host time until the seats were free
 
 private:
     SeatPool* pool_;
@@ -461,6 +462,7 @@ gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* 
     GK_CUDA(cudaStreamSynchronize(s));
     {
         GridSeats seats(P.half, P.nb);
+        out->queued_ms += seats.waited_ms;
         GK_TRY(launch());
         GK_CUDA(cudaMemcpyAsync(h, P.err(), sizeof(Outcome), cudaMemcpyDeviceToHost, s));
         GK_CUDA(cudaStreamSynchronize(s));

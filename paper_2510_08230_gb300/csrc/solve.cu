@@ -245,7 +245,7 @@ GridSeats::GridSeats(bool half, int blocks) {
     sms = std::max(sms, 1);
     pool_ = &pools->of(dev);
     seats_ = half ? std::min(blocks, 2 * sms) : 2 * sms;
-    pool_->take(seats_, 2 * sms);
+    waited_ms = pool_->take(seats_, 2 * sms);
 }
 
 GridSeats::~GridSeats() { pool_->give(seats_); }
@@ -449,6 +449,7 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
                                     : inner_solve(__nv_bfloat16()));
         total_inner += io.iters;
         restarts += io.restarts;
+        out->queued_ms += io.queued_ms;
         last_rec = io.rec;
         if (tn < best_tn) {  // x (not yet corrected) is the best iterate
             GK_CUDA(cudaMemcpyAsync(xb, x, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -478,6 +479,7 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         status = fo.status;
         total_inner += fo.iters;
         restarts += fo.restarts + 1;
+        out->queued_ms += fo.queued_ms;
         last_rec = fo.rec;
         tn = fo.tru * bnorm;
     }
@@ -621,7 +623,7 @@ extern "C" gk_status gk_solve(gk_matrix A, const void* b, void* x, const gk_solv
         info->outer_iters = outer;
         info->rel_res_recurrence = out.rec;
         info->rel_res_true = out.tru;
-        info->device_ms = ms;
+        info->device_ms = std::max(0.f, ms - out.queued_ms);
         info->spmv_format = out.layout;
         info->slice_size = out.slice;
         info->block_threads = out.threads;
