@@ -276,8 +276,10 @@ typedef struct {
     int32_t spmv_format;      /* layout the solve's SpMV ran on (GK_CSR, GK_ELL or
                                  GK_SELLP; refinement: the FP64 residual's) */
     int32_t slice_size;       /* SELL-P slice size of that layout, else 0 */
-    int32_t block_threads;    /* threads per block of the single-block engine and
-                                 of gk_solve_batched (autotuned), else 0 */
+    int32_t block_threads;    /* threads per block of the single-block engine, of
+                                 gk_solve_batched (autotuned) and of the persistent
+                                 kernels (512 or 1024; refinement: of its last inner
+                                 solve), else 0 */
 } gk_solve_info;
 
 /* Solve A x = b for square A (Listing 1: solver.apply(b, x) overwrites

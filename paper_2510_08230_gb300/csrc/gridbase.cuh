@@ -469,6 +469,7 @@ gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* 
     }
     if (h->err != 0 || h->o.status == GK_ERR_TIMEOUT) return GK_ERR_UNSUPPORTED;
     GK_CUDA(cudaMemcpyAsync(x, from, bytes, cudaMemcpyDeviceToDevice, s));
+    out->threads = P.half ? GRID_HALF : GRID_FULL;
     out->status = (gk_status)h->o.status;
     out->iters = h->o.iters;
     out->restarts = h->o.restarts;

@@ -450,6 +450,7 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         total_inner += io.iters;
         restarts += io.restarts;
         out->queued_ms += io.queued_ms;
+        out->threads = io.threads;
         last_rec = io.rec;
         if (tn < best_tn) {  // x (not yet corrected) is the best iterate
             GK_CUDA(cudaMemcpyAsync(xb, x, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -480,6 +481,7 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         total_inner += fo.iters;
         restarts += fo.restarts + 1;
         out->queued_ms += fo.queued_ms;
+        out->threads = fo.threads;
         last_rec = fo.rec;
         tn = fo.tru * bnorm;
     }
