@@ -201,7 +201,10 @@ gk_status gk_matrix_destroy(gk_matrix A);
 /* x = A b  (a matrix LinOp's apply, Section 4.2; the paper's SpMV
  * benchmark computes x = A b, Section 6.1).  b has ncols entries, x has n.
  * Both device pointers (stream-ordered, asynchronous) or both host
- * pointers (staged, blocking).  b and x must not overlap. */
+ * pointers (staged, blocking).  b and x must not overlap.  Products with
+ * device pointers may overlap on several streams, except those of a COO
+ * handle and of a CSR matrix with a row of more than 1024 entries, whose
+ * partial sums pass through a buffer of the handle. */
 gk_status gk_apply(gk_matrix A, const void* b, void* x, void* stream);
 
 /* x = alpha * A b + beta * x  (the advanced apply).  When beta == 0, x is

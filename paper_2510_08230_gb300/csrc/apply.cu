@@ -13,6 +13,24 @@ static bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// The carry buffer of a product of A on stream s: each of the first few streams
+// has one of its own, so that products on several streams do not meet.  -1: none
+// is left, or the call is being captured (its graph may run beside anything);
+// the product then does without.  A matrix of longer rows than k_seg_heads
+// serves has one buffer: its products have to be ordered.
+static int carry_slot(gk_matrix A, cudaStream_t s) {
+    if (A->plan.slots == 1) return 0;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    // the id must not be asked for during a capture: that would end it
+    if (cudaStreamIsCapturing(s, &capture) == cudaSuccess) {
+        if (capture != cudaStreamCaptureStatusNone) return -1;
+        if (cudaStreamGetId(s, &id) == cudaSuccess) return A->carry_slots.of(id);
+    }
+    cudaGetLastError();
+    return -1;
+}
+
 template <typename V, typename T>
 static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double beta, void* x,
                             cudaStream_t s) {
@@ -53,9 +71,13 @@ static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double bet
     if (A->fmt == GK_CSR && A->plan.seg) {
         const int64_t units = A->plan.units;
         if (units > 0) {
-            int32_t* crow = static_cast<int32_t*>(A->plan.carries);
-            T* cval = reinterpret_cast<T*>(static_cast<char*>(A->plan.carries) +
-                                           (((size_t)units * sizeof(int32_t) + 15) & ~(size_t)15));
+            const int slot = carry_slot(A, s);
+            char* carries = slot < 0 ? nullptr
+                                     : static_cast<char*>(A->plan.carries) + slot * A->plan.carry_bytes;
+            int32_t* crow = reinterpret_cast<int32_t*>(carries);
+            T* cval = carries ? reinterpret_cast<T*>(
+                                    carries + (((size_t)units * sizeof(int32_t) + 15) & ~(size_t)15))
+                              : nullptr;
             const int32_t* row_end = A->plan.row_end ? A->plan.row_end : A->row_ptr + 1;
             auto seg = [&](auto kern) {
                 kern<<<(unsigned)((units + 7) / 8), 256, 0, s>>>(
@@ -64,10 +86,21 @@ static gk_status spmv_typed(gk_matrix A, double alpha, const void* b, double bet
             };
             if (A->plan.local_cols) seg(k_csr_seg<true, V, T>);
             else seg(k_csr_seg<false, V, T>);
-            const unsigned fg =
-                (unsigned)std::max<int64_t>(1, std::min<int64_t>((units + 255) / 256, 4096));
-            k_carry_fixup<T><<<fg, 256, 0, s>>>((int32_t)units, crow, cval, static_cast<T*>(x),
-                                                (T)alpha, mode);
+            auto blocks = [&](int64_t threads) {
+                return (unsigned)std::max<int64_t>(1, std::min<int64_t>((threads + 255) / 256, 4096));
+            };
+            auto heads = [&](auto kern, int lanes) {
+                kern<<<blocks(units * lanes), 256, 0, s>>>(
+                    units, row_end, A->plan.row_id, A->plan.unit_row, A->col, (const V*)A->val,
+                    static_cast<const T*>(b), static_cast<T*>(x), (T)alpha, mode);
+            };
+            if (carries)
+                k_carry_fixup<T><<<blocks(units), 256, 0, s>>>((int32_t)units, crow, cval,
+                                                               static_cast<T*>(x), (T)alpha, mode);
+            else if (A->max_row <= 64)
+                heads(k_seg_heads<8, V, T>, 8);
+            else
+                heads(k_seg_heads<32, V, T>, 32);
         }
         if (A->plan.n_empty) {
             const unsigned eg = (unsigned)std::max<int64_t>(

@@ -18,6 +18,7 @@
 #include <string>
 
 #include "gk.h"
+#include "stream_slots.h"
 
 namespace gk {
 
@@ -177,7 +178,9 @@ struct CsrPlan {
     int32_t wt_rpl = 2;      // warp-tile: rows per lane (tiles of 32 * wt_rpl rows)
     int32_t units = 0;
     int32_t* unit_row = nullptr;  // the carries of the units follow it in one allocation
-    void* carries = nullptr;
+    void* carries = nullptr;      // `slots` buffers of carry_bytes, each one stream's
+    size_t carry_bytes = 0;
+    int slots = 0;
     int32_t* row_end = nullptr;
     int32_t* row_id = nullptr;
     int32_t* empty_rows = nullptr;
@@ -324,6 +327,7 @@ struct gk_matrix_s {
     gk::SolverCache* solver = nullptr;
     gk::DevBuf stage_in, stage_out;  // host-pointer apply staging
     gk::DevBuf carry;                // COO unit carries
+    gk::StreamSlots carry_slots;     // whose plan.carries' buffers are
     cudaStream_t side = nullptr;     // library streams for graph capture (the second
     cudaStream_t side2 = nullptr;    // captures the body of a solve's loop)
     uint64_t wait_ns = 2000000000ull;  // budget of the row-tile kernel's waits (a solve's

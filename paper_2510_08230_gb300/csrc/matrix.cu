@@ -997,8 +997,9 @@ gk_status build_csr_plan(gk_matrix A, cudaStream_t s) {
             P.local_cols = 2 * close > sampled;
         }
         const size_t urow = (4 * ((size_t)P.units + 1) + 255) & ~(size_t)255;
-        GK_CUDA(dmalloc((void**)&P.unit_row,
-                        urow + (size_t)P.units * (4 + vector_bytes(A->dtype)) + 16));
+        P.slots = A->max_row > SEG_HEADS_MAX ? 1 : StreamSlots::COUNT;
+        P.carry_bytes = ((size_t)P.units * (4 + vector_bytes(A->dtype)) + 16 + 255) & ~(size_t)255;
+        GK_CUDA(dmalloc((void**)&P.unit_row, urow + (size_t)P.slots * P.carry_bytes));
         P.carries = (char*)P.unit_row + urow;
         k_unit_rows<<<grid_for(P.units + 1), 256, 0, s>>>(
             m, P.row_end ? P.row_end : A->row_ptr + 1, P.units, P.unit_row);

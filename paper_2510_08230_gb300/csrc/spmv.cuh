@@ -527,7 +527,7 @@ k_csr_merge(int32_t n, int64_t nnz, const int32_t* __restrict__ rp,
 // shared memory and leave together, so that y is written (and for beta != 0
 // read) in row order.  A row begun in earlier lanes gets their part from a
 // segmented shuffle scan; the row open at the end of a unit goes to
-// k_carry_fixup.
+// k_carry_fixup, or (carry_row null) is left to k_seg_heads.
 // Rows are the matrix's nonempty ones: row_end[i] is the end of the i-th
 // (row_ptr + 1 when no row is empty), row_id[i] its index (null: i);
 // k_empty_rows writes the others.  unit_row[u]: the first of them that ends
@@ -654,7 +654,7 @@ k_csr_seg(int64_t nnz, int64_t nunits, const int32_t* __restrict__ row_end,
     }
     const T before = __shfl_up_sync(FULL, acc, 1);
     if (head >= 0 && lane > 0) sum[head] = before + sum[head];
-    if (lane == 31) {
+    if (lane == 31 && carry_row) {
         // the unit's last nonzero ends a row (also when the matrix ends here): no carry
         const bool open = k0 + SEG_UNIT < nnz && (mw[3] >> 16) < 0;
         carry_row[u] = open ? (row_id ? __ldg(row_id + i0 + nrow) : i0 + nrow) : -1;
@@ -796,6 +796,58 @@ __global__ void k_carry_fixup(int32_t nblocks, const int32_t* __restrict__ carry
         T v = carry_val[b];
         for (int64_t c = b + 1; c < nblocks && carry_row[c] == r; ++c) v = v + carry_val[c];
         y[r] = mode == 0 ? y[r] + v : fmadd(alpha, v, y[r]);
+    }
+}
+
+// The way to finish rows that reach across units of k_csr_seg without carries:
+// the part of a row that lies before the unit in which it ends is summed again
+// and added to y, G lanes a unit.  Nothing passes from one kernel to the next
+// but y.  It runs where a product may not use a carry buffer (see
+// carry_slot), on matrices without rows longer than SEG_HEADS_MAX.  y = A x in
+// FP64 with carries / so / on row tiles, us (n x mean length): 200,000 x 16
+// 17.5 / 25.4 / 69.5, 2M x 8 71.6 / 103 / 192, 2M Zipf rows 93.5 / 161 / 2358,
+// 200,000 x 100 84 / 137 / 324.  (The units of a block handing their open parts
+// on through shared memory, so that only rows across blocks are summed again:
+// 80 to 86 at 2M x 8 and 133 on the Zipf rows, but every product would pay for
+// its barrier; the buffers cost nothing.)
+constexpr int32_t SEG_HEADS_MAX = 1024;
+
+template <int G, typename V, typename T>
+__global__ void __launch_bounds__(256)
+k_seg_heads(int64_t nunits, const int32_t* __restrict__ row_end, const int32_t* __restrict__ row_id,
+            const int32_t* __restrict__ unit_row, const int32_t* __restrict__ ci,
+            const V* __restrict__ va, const T* __restrict__ x, T* __restrict__ y, T alpha, int mode) {
+    constexpr int U = 4;  // entries of a lane in flight
+    const int gl = threadIdx.x & (G - 1);
+    const unsigned group = (G == 32 ? 0xffffffffu : (1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
+    const int64_t step = (int64_t)gridDim.x * blockDim.x / G;
+    for (int64_t u = 1 + (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G; u < nunits; u += step) {
+        const int32_t i = __ldg(unit_row + u), next = __ldg(unit_row + u + 1);
+        const int64_t end = u * SEG_UNIT;
+        int64_t k = i > 0 ? __ldg(row_end + i - 1) : 0;
+        if (next == i || k >= end) continue;  // it ends later, or begins here
+        T s = T(0);
+        for (k += gl; k < end; k += U * G) {
+            int32_t c[U];
+            T xv[U], v[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {  // past the end: the last entry again, not added
+                const int64_t at = min(k + q * G, end - 1);
+                c[q] = __ldg(ci + at);
+                v[q] = cvt<T>(va[at]);
+            }
+#pragma unroll
+            for (int q = 0; q < U; ++q) xv[q] = __ldg(x + c[q]);
+#pragma unroll
+            for (int q = 0; q < U; ++q)
+                if (k + q * G < end) s = fmadd(v[q], xv[q], s);
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(group, s, o);
+        if (gl == 0) {
+            const int32_t r = row_id ? __ldg(row_id + i) : i;
+            y[r] = mode == 0 ? y[r] + s : fmadd(alpha, s, y[r]);
+        }
     }
 }
 
