@@ -1042,6 +1042,20 @@ static gk_status copy_in(void* dst, const void* src, size_t bytes, gk_memory mem
     return GK_OK;
 }
 
+// Whether kernels of the current device can read an array of the caller's
+// where it lies: its own memory (or managed), on the element's alignment.  A
+// copy takes any other device-accessible address.
+static bool readable_in_place(const void* p, size_t element) {
+    cudaPointerAttributes at;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev)) &&
+           reinterpret_cast<uintptr_t>(p) % element == 0;
+}
+
 }  // namespace gk
 
 using namespace gk;
@@ -1112,19 +1126,23 @@ gk_status gk_matrix_create_coo(int32_t n, int32_t ncols, int64_t nnz, const int3
     const size_t nz1 = (size_t)std::max<int64_t>(nnz, 1), n1 = (size_t)n + 1;
     const int64_t nblk = std::max<int64_t>(1, (nnz + SCAN_TILE - 1) / SCAN_TILE);
     // one scratch allocation (an allocation and its free cost more than most
-    // of the kernels); triplets on the device are read in place
+    // of the kernels); triplets on the device are read in place where they
+    // can be
     size_t at = 0;
     auto part = [&](size_t bytes) {
         const size_t o = at;
         at += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    const bool host = mem == GK_MEM_HOST;
+    auto staged = [&](const void* p, size_t element) {
+        return nnz > 0 && (mem == GK_MEM_HOST || !readable_in_place(p, element));
+    };
+    const bool copy_row = staged(row, 4), copy_col = staged(col, 4), copy_val = staged(values, vb);
     const size_t o_keys = part(8 * nz1), o_rank = part(4 * nz1), o_first = part(nz1);
     const size_t o_cnt = part(4 * n1), o_start = part(4 * n1), o_list = part(4 * n1);
     const size_t o_bsum = part(8 * (size_t)std::max(nblk + 1, n / (int64_t)SCAN_TILE + 1)), o_info = part(256);
-    const size_t o_row = part(host ? 4 * nz1 : 0), o_col = part(host ? 4 * nz1 : 0);
-    const size_t o_val = part(host ? vb * nz1 : 0);
+    const size_t o_row = part(copy_row ? 4 * nz1 : 0), o_col = part(copy_col ? 4 * nz1 : 0);
+    const size_t o_val = part(copy_val ? vb * nz1 : 0);
     TmpBuf scratch, longs;
     if (scratch.ensure(at)) return GK_ERR_OOM;
     char* base = static_cast<char*>(scratch.ptr);
@@ -1136,13 +1154,16 @@ gk_status gk_matrix_create_coo(int32_t n, int32_t ncols, int64_t nnz, const int3
     gk_status st;
     const int32_t *drow = row, *dcol = col;
     const void* dval = values;
-    if (host) {
-        if ((st = copy_in(base + o_row, row, 4 * (size_t)nnz, mem, s)) != GK_OK ||
-            (st = copy_in(base + o_col, col, 4 * (size_t)nnz, mem, s)) != GK_OK ||
-            (st = copy_in(base + o_val, values, vb * (size_t)nnz, mem, s)) != GK_OK)
-            return fail(st);
+    if (copy_row) {
+        if ((st = copy_in(base + o_row, row, 4 * (size_t)nnz, mem, s)) != GK_OK) return fail(st);
         drow = (const int32_t*)(base + o_row);
+    }
+    if (copy_col) {
+        if ((st = copy_in(base + o_col, col, 4 * (size_t)nnz, mem, s)) != GK_OK) return fail(st);
         dcol = (const int32_t*)(base + o_col);
+    }
+    if (copy_val) {
+        if ((st = copy_in(base + o_val, values, vb * (size_t)nnz, mem, s)) != GK_OK) return fail(st);
         dval = base + o_val;
     }
     uint64_t* dkeys = (uint64_t*)(base + o_keys);
