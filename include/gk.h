@@ -255,12 +255,13 @@ typedef struct {
     int32_t block_size;   /* block-Jacobi rows per diagonal block, 1..32 */
     int64_t wait_budget_ns; /* longest a device-side wait of this solve may last
                              (the ILU(0) substitutions' polls on values other
-                             warps produce, or the window mode's waits on its
-                             copies of row records; the CSR row-tile kernel's
-                             waits on its staged copies) before it gives up: the solve
-                             then returns GK_ERR_TIMEOUT and x holds no valid
-                             iterate.  0 = the default of 2 s; negative values
-                             are GK_ERR_INVALID.  When a hand-off between the
+                             warps or slabs produce, or the window and slab
+                             modes' waits on their copies of row records; the
+                             CSR row-tile kernel's waits on its staged copies)
+                             before it gives up: the solve then returns
+                             GK_ERR_TIMEOUT and x holds no valid iterate.  0 =
+                             the default of 2 s; negative values are
+                             GK_ERR_INVALID.  When a hand-off between the
                              blocks of a persistent kernel takes longer (it is
                              microseconds, unless other work keeps a block off
                              the GPU), engine 1 solves from the initial guess
@@ -391,7 +392,11 @@ gk_status gk_solve_batched(int32_t count, const gk_matrix* As,
  * window mode instead, when it is faster: one cluster of 16 blocks solves
  * a triangle level by level through distributed shared memory, and its
  * only waits, for its own copies of the next level's row records, take the
- * same budget.  Every mode gives the same bits. */
+ * same budget; or the slab mode (levels of at most 768 rows a slab): blocks
+ * own slabs of consecutive rows, and besides such copies wait for the values
+ * of the slabs before theirs, the last one until the substitution has come
+ * that far (a few hundred microseconds on 10^6 rows), within the same budget.
+ * Every mode gives the same bits. */
 gk_status gk_precond_apply(gk_matrix A, gk_precond kind, int32_t block_size,
                            const void* r, void* z, int64_t wait_budget_ns, void* stream);
 

@@ -35,11 +35,12 @@
 // to the other modes.
 //
 // No wait can be circular: a slab only waits on slabs of rows before it (U:
-// after it), and blocks claim slabs in that order from a counter.  Waits for
-// the block's own copies take the caller's budget, as in the window mode;
-// waits on other slabs (the last one starts only when the wavefront
-// arrives) at least the default limit.  When one runs out, all later ones
-// give up at once and the launch ends with wrong values and the error word.
+// after it), and blocks claim slabs in that order from a counter.  Every wait
+// takes the caller's budget: for the block's own copies, as in the window
+// mode, and for other slabs' values, as in the chunked kernels (the last slab
+// starts only when the wavefront arrives, so a budget below a triangle's time
+// runs out there).  When one runs out, all later ones give up at once and the
+// launch ends with wrong values and the error word.
 #pragma once
 
 namespace gk {
@@ -131,7 +132,6 @@ k_ilu_trsv_slab(IluDev<T> f, Out out, Skip sk, Err on_err) {
     __syncthreads();
     const int slab = UP ? D.nslab - 1 - s_claim : s_claim;
     const int32_t lo = D.range[2 * slab], hi = D.range[2 * slab + 1];
-    const uint64_t hand_ns = f.wait_ns > WAIT_LIMIT_NS ? f.wait_ns : WAIT_LIMIT_NS;
     T* hand = f.shand;
     const int32_t* start = D.start + (size_t)slab * D.nlev;
     int32_t staged = 0;  // copying threads: one past the last level copied or under way
@@ -140,7 +140,7 @@ k_ilu_trsv_slab(IluDev<T> f, Out out, Skip sk, Err on_err) {
         atomicExch(&sy->err, 1u);
     };
     // a wait on other warps of this block, which give up first: they wait at
-    // most hand_ns for a value
+    // most the budget for a value
     auto wait_block = [&](auto ready) {
         uint64_t t0 = 0;
         while (!s_dead) {
@@ -148,7 +148,7 @@ k_ilu_trsv_slab(IluDev<T> f, Out out, Skip sk, Err on_err) {
                 if (ready()) return;
             const uint64_t t = globaltimer_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > 2 * hand_ns) give_up();
+            if ((t - t0) / 2 > f.wait_ns) give_up();
         }
     };
     // until `want` levels have ended
@@ -361,7 +361,7 @@ k_ilu_trsv_slab(IluDev<T> f, Out out, Skip sk, Err on_err) {
                         const uint64_t t = globaltimer_ns();
                         if (t0 == 0) t0 = t;
                         if (s_dead || ld_relaxed_u32(&sy->err) != 0u) break;
-                        if (t - t0 > hand_ns) {
+                        if (t - t0 > f.wait_ns) {
                             give_up();
                             break;
                         }
