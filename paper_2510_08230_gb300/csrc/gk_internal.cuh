@@ -192,6 +192,29 @@ struct CsrPlan {
 
 struct SolverCache;  // solve.cu
 
+// Data of the ILU(0) substitutions' slab mode for both triangles: see SlabDir.
+// Buckets are nslab * nlev[.].  One allocation holds what the sizes of the
+// matrix decide (rows, start, estart, range, perm, hand), one what the buckets
+// decide (records and epos).
+struct SlabStore {
+    int32_t nslab = 0, rows_each = 0;
+    int32_t nlev[2] = {0, 0}, cap[2] = {0, 0}, ecap[2] = {0, 0}, nb[2] = {0, 0}, terms[2] = {0, 0};
+    int32_t* rows[2] = {nullptr, nullptr};
+    int32_t* start[2] = {nullptr, nullptr};
+    int32_t* estart[2] = {nullptr, nullptr};
+    int32_t* range[2] = {nullptr, nullptr};
+    int32_t* epos[2] = {nullptr, nullptr};
+    void* rec[2] = {nullptr, nullptr};
+    void* perm = nullptr;           // level-ordered input
+    void* hand = nullptr;           // handed-over values
+    void *fixed = nullptr, *sized = nullptr;  // the allocations
+    void release() {
+        dfree(fixed);
+        dfree(sized);
+        *this = SlabStore();
+    }
+};
+
 // Two triangular factors sharing one CSR pattern: the ILU(0) factors, or a
 // matrix's own lower and upper triangles (gk_triangular_solve), with what
 // the substitution kernels need.  Built on first use and owned by the
@@ -223,33 +246,11 @@ struct TriStore {
     int32_t wdist[2] = {1, 1};
     void* wrec = nullptr;
     void* wperm = nullptr;
-    // slab mode (slab = 1: picked): see SlabDir; buckets are nslab * nlev[.]
-    int32_t slab = 0, nslab = 0;
-    int32_t slev[2] = {0, 0}, scap[2] = {0, 0}, secap[2] = {0, 0}, snb[2] = {0, 0}, sterms[2] = {0, 0};
-    int32_t* srows[2] = {nullptr, nullptr};
-    int32_t* sstart[2] = {nullptr, nullptr};
-    int32_t* srange[2] = {nullptr, nullptr};
-    int32_t* sestart[2] = {nullptr, nullptr};
-    int32_t* sepos[2] = {nullptr, nullptr};
-    void* srec[2] = {nullptr, nullptr};
-    void* sperm = nullptr;          // level-ordered input
-    void* shand = nullptr;          // handed-over values
-    void release_slab() {
-        for (int u = 0; u < 2; ++u) {
-            for (int32_t** p : {&srows[u], &sstart[u], &srange[u], &sestart[u], &sepos[u]}) {
-                dfree(*p);
-                *p = nullptr;
-            }
-            dfree(srec[u]);
-            srec[u] = nullptr;
-        }
-        dfree(sperm);
-        dfree(shand);
-        sperm = shand = nullptr;
-    }
+    int32_t slab = 0;               // slab mode picked
+    SlabStore sl;
     DevBuf w;                       // scratch of one application
     void release() {
-        release_slab();
+        sl.release();
         dfree(lrows);
         dfree(lstart);
         dfree(wrec);

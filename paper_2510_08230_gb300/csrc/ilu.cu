@@ -317,7 +317,7 @@ static gk_status level_order(int32_t nch, int32_t pad, const DevBuf& lev, int32_
     return GK_OK;
 }
 
-// Chunk levels of both triangles for the two chunk sizes (32 and 8 rows),
+// Chunk levels of both triangles for the chunk sizes (32, 8 and 1 rows),
 // computed once per matrix and shared by the factorisation order and every
 // substitution candidate.
 struct IluLevels {
@@ -515,6 +515,14 @@ __global__ void k_slab_check(int32_t n, const unsigned* __restrict__ lev,
     }
 }
 
+__global__ void k_slab_ranges(int32_t nslab, int32_t* __restrict__ range) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nslab;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        range[2 * k] = INT32_MAX;
+        range[2 * k + 1] = -1;
+    }
+}
+
 // rows and fetched values of every bucket, the levels of every slab (range
 // starts at {INT32_MAX, -1})
 template <bool UP>
@@ -606,102 +614,149 @@ __global__ void k_slab_rec(int32_t n, int32_t R, int32_t nlev, int32_t cap, int3
     }
 }
 
-// Builds the slab-mode data with about `want` slabs (whole multiples of the
-// farthest dependency, where that is shorter than a slab); *ok = false when
-// the matrix does not qualify: more than WIN_MAXT terms a row or
-// dependencies over WIN_MAXD levels back, too many rows or fetched values in
-// a bucket for shared memory, more than 8 buckets a row.  *rows: the rows of
-// a slab; nothing is built when that is `skip`.
-template <typename T>
-static gk_status build_slab(TriStore* S, int32_t n, const IluLevels& lv, int32_t want, int32_t skip,
-                            cudaStream_t s, int32_t* rows, bool* ok) {
-    *ok = false;
-    *rows = 0;
-    if (n == 0) return GK_OK;
-    const unsigned* lev[2] = {(const unsigned*)lv.l1.ptr, (const unsigned*)lv.u1.ptr};
-    const int32_t nlev[2] = {(int32_t)lv.nl1, (int32_t)lv.nu1};
-    const unsigned g = ew_grid(n);
+// What decides whether a matrix qualifies for the slab mode, both triangles:
+// terms of a row, deepest dependency in levels, farthest one in rows.
+struct SlabShape {
+    unsigned terms[2] = {0, 0}, depth[2] = {0, 0}, span = 1;
+    bool fits = false;  // at most WIN_MAXT terms a row, WIN_MAXD levels back
+};
+
+static gk_status slab_shape(const TriStore* S, int32_t n, const IluLevels& lv, cudaStream_t s,
+                            SlabShape* out) {
     TmpBuf misc;
     GK_TRY(misc.ensure(64));
     unsigned* mp = (unsigned*)misc.ptr;
     GK_CUDA(cudaMemsetAsync(mp, 0, 64, s));
-    k_slab_check<false><<<g, 256, 0, s>>>(n, lev[0], S->rp, S->ci, S->dpos, mp);
-    k_slab_check<true><<<g, 256, 0, s>>>(n, lev[1], S->rp, S->ci, S->dpos, mp + 3);
+    const unsigned g = ew_grid(n);
+    k_slab_check<false><<<g, 256, 0, s>>>(n, (const unsigned*)lv.l1.ptr, S->rp, S->ci, S->dpos, mp);
+    k_slab_check<true><<<g, 256, 0, s>>>(n, (const unsigned*)lv.u1.ptr, S->rp, S->ci, S->dpos, mp + 3);
     GK_CUDA(cudaGetLastError());
     unsigned h[6];
     GK_CUDA(cudaMemcpyAsync(h, mp, sizeof(h), cudaMemcpyDeviceToHost, s));
     GK_CUDA(cudaStreamSynchronize(s));
-    if (h[0] > WIN_MAXT || h[3] > WIN_MAXT || h[1] > WIN_MAXD || h[4] > WIN_MAXD) return GK_OK;
+    for (int u = 0; u < 2; ++u) {
+        out->terms[u] = h[3 * u];
+        out->depth[u] = h[3 * u + 1];
+        out->span = std::max(out->span, h[3 * u + 2]);
+    }
+    out->fits = std::max(h[0], h[3]) <= (unsigned)WIN_MAXT && std::max(h[1], h[4]) <= (unsigned)WIN_MAXD;
+    return GK_OK;
+}
+
+// Rows of a slab for about `want` slabs: whole multiples of the farthest
+// dependency, where that is shorter than a slab.
+static int32_t slab_rows(int32_t n, const SlabShape& h, int32_t want) {
     int64_t R = ((int64_t)n + want - 1) / want;
-    const int64_t span = std::max<int64_t>(1, std::max(h[2], h[5]));
-    if (R >= span) R = (R + span - 1) / span * span;
+    if (R >= (int64_t)h.span) R = (R + h.span - 1) / h.span * h.span;
+    return (int32_t)R;
+}
+
+// Builds the slab-mode data with slabs of R rows into B (empty before; the
+// caller releases it); *ok = false when the matrix does not qualify: too many
+// rows or fetched values in a bucket for shared memory, or more than 8 buckets
+// a row.
+template <typename T>
+static gk_status build_slab(const TriStore* S, int32_t n, const IluLevels& lv, const SlabShape& h,
+                            int32_t R, cudaStream_t s, SlabStore* B, bool* ok) {
+    *ok = false;
+    const unsigned* lev[2] = {(const unsigned*)lv.l1.ptr, (const unsigned*)lv.u1.ptr};
+    const int32_t nlev[2] = {(int32_t)lv.nl1, (int32_t)lv.nu1};
     const int32_t nslab = (int32_t)(((int64_t)n + R - 1) / R);
     if ((int64_t)nslab * std::max(nlev[0], nlev[1]) > 8 * (int64_t)n + 1024) return GK_OK;
-    *rows = (int32_t)R;
-    if (*rows == skip) return GK_OK;
-    S->nslab = nslab;
-    TmpBuf pos, cur, ecur, tmp;
-    GK_TRY(pos.ensure(sizeof(int32_t) * (size_t)n));
+    B->nslab = nslab;
+    B->rows_each = R;
+    const unsigned g = ew_grid(n);
     constexpr int AL = (int)(16 / sizeof(T));
-    GK_CUDA(dmalloc(&S->sperm, sizeof(T) * ((size_t)n + AL)));
-    GK_CUDA(dmalloc(&S->shand, sizeof(T) * (size_t)n));
-    std::vector<int32_t> hr(2 * (size_t)nslab);
+    const size_t nk[2] = {(size_t)nslab * nlev[0], (size_t)nslab * nlev[1]};
+    // the arrays whose sizes are known, and the scratch of the set-up
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    size_t o_rows[2], o_start[2], o_estart[2], o_range[2];
     for (int u = 0; u < 2; ++u) {
-        const size_t nk = (size_t)nslab * nlev[u];
-        S->slev[u] = nlev[u];
-        S->sterms[u] = (int32_t)h[3 * u];
-        GK_TRY(cur.ensure(sizeof(int32_t) * (nk + 1)));
-        GK_TRY(ecur.ensure(sizeof(int32_t) * (nk + 1)));
-        int32_t *cp = (int32_t*)cur.ptr, *ep = (int32_t*)ecur.ptr;
-        GK_CUDA(dmalloc_t(&S->srows[u], (size_t)n + 4));  // copied in 16-byte pieces
-        GK_CUDA(dmalloc_t(&S->sstart[u], nk + 1));
-        GK_CUDA(dmalloc_t(&S->sestart[u], nk + 1));
-        GK_CUDA(dmalloc_t(&S->srange[u], 2 * (size_t)nslab));
-        GK_CUDA(cudaMemsetAsync(cp, 0, sizeof(int32_t) * (nk + 1), s));
-        GK_CUDA(cudaMemsetAsync(ep, 0, sizeof(int32_t) * (nk + 1), s));
-        GK_CUDA(cudaMemsetAsync(mp, 0, 64, s));
-        for (int32_t k = 0; k < nslab; ++k) {
-            hr[2 * (size_t)k] = INT32_MAX;
-            hr[2 * (size_t)k + 1] = -1;
-        }
-        GK_CUDA(cudaMemcpyAsync(S->srange[u], hr.data(), sizeof(int32_t) * hr.size(),
-                                cudaMemcpyHostToDevice, s));
+        o_rows[u] = part(4 * ((size_t)n + 4));  // copied in 16-byte pieces
+        o_start[u] = part(4 * (nk[u] + 1));
+        o_estart[u] = part(4 * (nk[u] + 1));
+        o_range[u] = part(8 * (size_t)nslab);
+    }
+    const size_t o_perm = part(sizeof(T) * ((size_t)n + AL)), o_hand = part(sizeof(T) * (size_t)n);
+    GK_CUDA(dmalloc(&B->fixed, at));
+    char* base = static_cast<char*>(B->fixed);
+    B->perm = base + o_perm;
+    B->hand = base + o_hand;
+    at = 0;
+    const size_t nkm = std::max(nk[0], nk[1]);
+    size_t o_cur[2], o_ecur[2];
+    for (int u = 0; u < 2; ++u) {
+        o_cur[u] = part(4 * (nk[u] + 1));
+        o_ecur[u] = part(4 * (nk[u] + 1));
+    }
+    const size_t zeroed = at;
+    const size_t o_misc = part(64), o_pos = part(4 * (size_t)n);
+    const size_t o_scan = part(8 * (nkm / SCAN_TILE + 1));
+    TmpBuf scratch;
+    GK_TRY(scratch.ensure(at));
+    char* tmp = static_cast<char*>(scratch.ptr);
+    GK_CUDA(cudaMemsetAsync(tmp, 0, zeroed + 64, s));
+    int32_t* misc = (int32_t*)(tmp + o_misc);
+    for (int u = 0; u < 2; ++u) {
+        B->nlev[u] = nlev[u];
+        B->terms[u] = (int32_t)h.terms[u];
+        B->rows[u] = (int32_t*)(base + o_rows[u]);
+        B->start[u] = (int32_t*)(base + o_start[u]);
+        B->estart[u] = (int32_t*)(base + o_estart[u]);
+        B->range[u] = (int32_t*)(base + o_range[u]);
+        int32_t *cp = (int32_t*)(tmp + o_cur[u]), *ep = (int32_t*)(tmp + o_ecur[u]);
+        k_slab_ranges<<<ew_grid(nslab), 256, 0, s>>>(nslab, B->range[u]);
         auto count = [&](auto k) {
-            k<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], lev[u], S->rp, S->ci, S->dpos, cp, ep,
-                                S->srange[u]);
+            k<<<g, 256, 0, s>>>(n, R, nlev[u], lev[u], S->rp, S->ci, S->dpos, cp, ep, B->range[u]);
         };
         u ? count(k_slab_count<true>) : count(k_slab_count<false>);
-        k_slab_widest<<<ew_grid((int64_t)nk), 256, 0, s>>>((int64_t)nk, cp, ep, (int32_t*)mp);
+        k_slab_widest<<<ew_grid((int64_t)nk[u]), 256, 0, s>>>((int64_t)nk[u], cp, ep, misc + 2 * u);
         GK_CUDA(cudaGetLastError());
-        GK_TRY((scan_exclusive<int32_t, int32_t>(cp, S->sstart[u], (int64_t)nk, tmp, s)));
-        GK_TRY((scan_exclusive<int32_t, int32_t>(ep, S->sestart[u], (int64_t)nk, tmp, s)));
-        int32_t w[2], total = 0;
-        GK_CUDA(cudaMemcpyAsync(w, mp, sizeof(w), cudaMemcpyDeviceToHost, s));
-        GK_CUDA(cudaMemcpyAsync(&total, S->sestart[u] + nk, sizeof(total), cudaMemcpyDeviceToHost, s));
-        GK_CUDA(cudaStreamSynchronize(s));
-        if (w[0] > SLAB_CAP || w[1] > 65535 / SLAB_E) return GK_OK;
-        S->scap[u] = (w[0] + 31) / 32 * 32;
-        S->secap[u] = std::max(1, w[1]);
-        S->snb[u] = slab_values(S->scap[u], S->secap[u]) <= 65536 ? SLAB_NB : 0;  // 16-bit indices
-        while (S->snb[u] >= 2 && slab_smem<T>(S->scap[u], S->secap[u], S->snb[u]) > (size_t)SLAB_SMEM)
-            S->snb[u] -= SLAB_SW;  // whole rounds of the copying warps
-        if (S->snb[u] < 2) return GK_OK;
-        GK_CUDA(dmalloc_t(&S->sepos[u], (size_t)std::max(1, total)));
-        GK_CUDA(dmalloc(&S->srec[u], sizeof(WinRec<T>) * (size_t)n));
-        GK_CUDA(cudaMemcpyAsync(cp, S->sstart[u], sizeof(int32_t) * nk, cudaMemcpyDeviceToDevice, s));
-        GK_CUDA(cudaMemcpyAsync(ep, S->sestart[u], sizeof(int32_t) * nk, cudaMemcpyDeviceToDevice, s));
-        int32_t* pp = (int32_t*)pos.ptr;
-        k_slab_scatter<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], lev[u], cp, S->srows[u], pp);
+        int64_t* bs = (int64_t*)(tmp + o_scan);
+        GK_TRY((scan_exclusive_in<int32_t, int32_t>(cp, B->start[u], (int64_t)nk[u], bs, s)));
+        GK_TRY((scan_exclusive_in<int32_t, int32_t>(ep, B->estart[u], (int64_t)nk[u], bs, s)));
+        GK_CUDA(cudaMemcpyAsync(misc + 4 + u, B->estart[u] + nk[u], 4, cudaMemcpyDeviceToDevice, s));
+        GK_CUDA(cudaMemcpyAsync(cp, B->start[u], 4 * nk[u], cudaMemcpyDeviceToDevice, s));
+        GK_CUDA(cudaMemcpyAsync(ep, B->estart[u], 4 * nk[u], cudaMemcpyDeviceToDevice, s));
+    }
+    int32_t w[6];  // {rows, fetched values} of the widest bucket of L, of U; fetched values of L, U
+    GK_CUDA(cudaMemcpyAsync(w, misc, sizeof(w), cudaMemcpyDeviceToHost, s));
+    GK_CUDA(cudaStreamSynchronize(s));
+    at = 0;
+    size_t o_epos[2], o_rec[2];
+    for (int u = 0; u < 2; ++u) {
+        if (w[2 * u] > SLAB_CAP || w[2 * u + 1] > 65535 / SLAB_E) return GK_OK;
+        B->cap[u] = (w[2 * u] + 31) / 32 * 32;
+        B->ecap[u] = std::max(1, w[2 * u + 1]);
+        B->nb[u] = slab_values(B->cap[u], B->ecap[u]) <= 65536 ? SLAB_NB : 0;  // 16-bit indices
+        while (B->nb[u] >= 2 && slab_smem<T>(B->cap[u], B->ecap[u], B->nb[u]) > (size_t)SLAB_SMEM)
+            B->nb[u] -= SLAB_SW;  // whole rounds of the copying warps
+        if (B->nb[u] < 2) return GK_OK;
+        o_epos[u] = part(4 * (size_t)std::max(1, w[4 + u]));
+        o_rec[u] = part(sizeof(WinRec<T>) * (size_t)n);
+    }
+    GK_CUDA(dmalloc(&B->sized, at));
+    for (int u = 0; u < 2; ++u) {
+        B->epos[u] = (int32_t*)(static_cast<char*>(B->sized) + o_epos[u]);
+        B->rec[u] = static_cast<char*>(B->sized) + o_rec[u];
+        int32_t* pos = (int32_t*)(tmp + o_pos);
+        k_slab_scatter<<<g, 256, 0, s>>>(n, R, nlev[u], lev[u], (int32_t*)(tmp + o_cur[u]), B->rows[u],
+                                         pos);
         auto fill = [&](auto k) {
-            k<<<g, 256, 0, s>>>(n, (int32_t)R, nlev[u], S->scap[u], S->secap[u], S->srange[u],
-                                S->srows[u], lev[u], pp, S->sstart[u],
-                                S->sestart[u], ep, S->rp, S->ci, S->dpos, (const T*)S->lu,
-                                (const T*)S->rdiag, (WinRec<T>*)S->srec[u], S->sepos[u]);
+            k<<<g, 256, 0, s>>>(n, R, nlev[u], B->cap[u], B->ecap[u], B->range[u], B->rows[u], lev[u],
+                                pos, B->start[u], B->estart[u], (int32_t*)(tmp + o_ecur[u]), S->rp,
+                                S->ci, S->dpos, (const T*)S->lu, (const T*)S->rdiag,
+                                (WinRec<T>*)B->rec[u], B->epos[u]);
         };
         u ? fill(k_slab_rec<T, true>) : fill(k_slab_rec<T, false>);
         GK_CUDA(cudaGetLastError());
     }
-    GK_CUDA(cudaStreamSynchronize(s));
+    GK_CUDA(cudaStreamSynchronize(s));  // the scratch goes
     *ok = true;
     return GK_OK;
 }
@@ -728,6 +783,30 @@ static gk_status build_row_levels(TriStore* S, int32_t n, const IluLevels& lv, c
 
 // claim-order entries S->ord holds (both directions)
 static size_t ord_capacity(int32_t n) { return 2 * 4 * (size_t)std::max((n + 7) / 8, 1); }
+
+// f in the slab mode on the data of B.
+template <typename T>
+static IluDev<T> slab_view(IluDev<T> f, const SlabStore& B) {
+    f.slab = 1;
+    for (int u = 0; u < 2; ++u) {
+        SlabDir& D = f.sd[u];
+        D.nslab = B.nslab;
+        D.nlev = B.nlev[u];
+        D.cap = B.cap[u];
+        D.ecap = B.ecap[u];
+        D.nb = B.nb[u];
+        D.terms = B.terms[u];
+        D.rows = B.rows[u];
+        D.start = B.start[u];
+        D.range = B.range[u];
+        D.estart = B.estart[u];
+        D.epos = B.epos[u];
+        D.rec = B.rec[u];
+    }
+    f.sperm = static_cast<T*>(B.perm);
+    f.shand = static_cast<T*>(B.hand);
+    return f;
+}
 
 template <typename T>
 static IluDev<T> tri_view(const TriStore* S, int32_t n) {
@@ -762,25 +841,7 @@ static IluDev<T> tri_view(const TriStore* S, int32_t n) {
     f.wrec[0] = S->wrec;
     f.wrec[1] = S->wrec ? static_cast<const char*>(S->wrec) + sizeof(WinRec<T>) * (size_t)n : nullptr;
     f.wperm = static_cast<T*>(S->wperm);
-    f.slab = S->slab;
-    for (int u = 0; u < 2; ++u) {
-        SlabDir& D = f.sd[u];
-        D.nslab = S->nslab;
-        D.nlev = S->slev[u];
-        D.cap = S->scap[u];
-        D.ecap = S->secap[u];
-        D.nb = S->snb[u];
-        D.terms = S->sterms[u];
-        D.rows = S->srows[u];
-        D.start = S->sstart[u];
-        D.range = S->srange[u];
-        D.estart = S->sestart[u];
-        D.epos = S->sepos[u];
-        D.rec = S->srec[u];
-    }
-    f.sperm = static_cast<T*>(S->sperm);
-    f.shand = static_cast<T*>(S->shand);
-    return f;
+    return S->slab ? slab_view<T>(f, S->sl) : f;
 }
 
 template <typename T>
@@ -789,6 +850,60 @@ IluDev<T> ilu_view(gk_matrix A) {
 }
 template IluDev<double> ilu_view<double>(gk_matrix);
 template IluDev<float> ilu_view<float>(gk_matrix);
+
+// Where a matrix qualifies for the slab mode it is the fastest: on 22 stencil
+// matrices of 216 to 2,097,152 rows, in FP64 and FP32, an application took 0.23
+// to 0.96 of the next best mode's time (at 33 rows 86 us against 60, at 64 62
+// against 65: below SLAB_MIN_N rows it is not tried).  So nothing else is built
+// or timed for such a matrix.  The first application to a new one, FP64, ms,
+// with the trials of the other modes / without / before there was a slab mode:
+// 2D 64^2 9.1 / 4.1 / 8.1, 20^3 15.6 / 3.8 / 14.5, 2D 300 x 200 310 / 93 /
+// 306, 128^3 640 / 500 / 640.
+constexpr int32_t SLAB_MIN_N = 128;
+
+// The slab mode's data where the matrix qualifies (*picked), in S->sl: the
+// faster of two slab sizes.  64 slabs are better where levels are narrow (2D
+// 1024^2), 128 where the FP64 pipe bounds a level (128^3 FP64).  w: 2 n values.
+template <typename T>
+static gk_status pick_slab(TriStore* S, int32_t n, const IluLevels& lv, T* w, cudaEvent_t e0,
+                           cudaEvent_t e1, cudaStream_t s, bool* picked) {
+    *picked = false;
+    SlabShape h;
+    GK_TRY(slab_shape(S, n, lv, s, &h));
+    if (!h.fits) return GK_OK;
+    struct Kept {
+        SlabStore b;
+        ~Kept() { b.release(); }
+    } best, cand;
+    float best_ms = 0.f;
+    int32_t tried = 0;
+    for (int32_t want : {64, 128}) {
+        const int32_t R = slab_rows(n, h, want);
+        if (R == tried) continue;
+        tried = R;
+        bool ok = false;
+        cand.b.release();
+        GK_TRY(build_slab<T>(S, n, lv, h, R, s, &cand.b, &ok));
+        if (!ok) continue;
+        IluDev<T> f = slab_view<T>(tri_view<T>(S, n), cand.b);
+        const IluSrc<T> src{(const T*)S->rdiag};
+        float ms = 0.f;
+        GK_TRY(ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s));
+        GK_CUDA(cudaEventRecord(e0, s));
+        GK_TRY(ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s));
+        GK_CUDA(cudaEventRecord(e1, s));
+        GK_CUDA(cudaEventSynchronize(e1));
+        GK_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        if (!best.b.nslab || ms < best_ms) {
+            best_ms = ms;
+            std::swap(best.b, cand.b);
+        }
+    }
+    if (!best.b.nslab) return GK_OK;
+    std::swap(S->sl, best.b);
+    *picked = true;
+    return GK_OK;
+}
 
 // Rows per substitution chunk and chunks per warp, timed per matrix:
 // 32-row chunks need the fewest dependency levels, 8-row chunks the
@@ -807,7 +922,7 @@ template IluDev<float> ilu_view<float>(gk_matrix);
 // cluster kernel) forces a shape.  Results never depend on the choice,
 // only the time does.
 template <typename T>
-static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaStream_t s) {
+static gk_status tune_chunks(TriStore* S, int32_t n, IluLevels& lv, cudaStream_t s) {
     int forced = 0;
     bool forced_lvl = false, forced_win = false, forced_slab = false;
     if (const char* e = getenv("GK_ILU_CHUNK")) {
@@ -823,7 +938,6 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
     const int all_cs[4] = {32, 8, 8, 1}, all_cpw[4] = {1, 1, 4, 32};
     // single-row chunks only when their padded claim orders stay within 2n
     const bool rows_ok = (size_t)n + 31 * (size_t)std::max(lv.nl1, lv.nu1) <= 2 * (size_t)n;
-    const int ncand = forced ? 1 : rows_ok ? 4 : 3;
     DevBuf ordb[4], tmp;
     int32_t warps[4][2] = {}, nord[4][2] = {};
     GK_TRY(tmp.ensure(2 * sizeof(T) * (size_t)n));
@@ -833,8 +947,24 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
     gk_status st = GK_OK;
     float best = 0.f;
     int pick = 0;
+    bool slab = false;
+    if (forced_slab || (!forced && n > SLAB_MIN_N)) {
+        const gk_status ss = pick_slab<T>(S, n, lv, (T*)tmp.ptr, e0, e1, s, &slab);
+        if (ss != GK_OK) {
+            cudaGetLastError();  // no room for the records: the other modes
+            slab = false;
+            if (forced_slab) st = ss;
+        }
+    }
+    // the chunk state is valid whatever mode runs
+    const int ncand = forced || slab ? 1 : rows_ok ? 4 : 3;
     for (int k = 0; k < ncand && st == GK_OK; ++k) {
         const int32_t cs = forced ? forced : all_cs[k];
+        if (cs == 8 && !lv.nl8) {
+            st = chunk_levels(S, n, 8, false, lv.l8, &lv.nl8, s);
+            if (st == GK_OK) st = chunk_levels(S, n, 8, true, lv.u8, &lv.nu8, s);
+            if (st != GK_OK) break;
+        }
         const int32_t cpw = forced ? (forced == 1 ? 32 : 1) : all_cpw[k];
         const int32_t nch = (n + cs - 1) / cs;
         // claim-order entries at most, per direction: every level padded
@@ -913,10 +1043,10 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
             lvl = forced_lvl || ms < best;
         }
     }
-    // the window mode (stencil-like matrices, see k_ilu_trsv_win): timed
-    // against the chunks when the matrix qualifies
+    // the window mode (stencil-like matrices too wide for the slab mode, see
+    // k_ilu_trsv_win): timed against the chunks when the matrix qualifies
     bool win = false;
-    if (st == GK_OK && !lvl && (forced_win || !forced)) {
+    if (st == GK_OK && !lvl && !slab && (forced_win || !forced)) {
         bool ok = false;
         gk_status ws = build_row_levels(S, n, lv, s);
         if (ws == GK_OK) ws = build_win<T>(S, n, lv, s, &ok);
@@ -940,67 +1070,11 @@ static gk_status tune_chunks(TriStore* S, int32_t n, const IluLevels& lv, cudaSt
             if (forced_win) st = ws;
         } else if (ok) {
             win = forced_win || ms < best;
-            if (win) best = ms;
         }
         if (!win) {  // not picked: its records go
             dfree(S->wrec);
             dfree(S->wperm);
             S->wrec = S->wperm = nullptr;
-        }
-    }
-    // the slab mode (the same matrices, see ilu_slab.cuh): two slab sizes,
-    // timed against the rest.  64 slabs are better where levels are narrow
-    // (2D 1024^2), 128 where the FP64 pipe bounds a level (128^3 FP64)
-    bool slab = false;
-    if (st == GK_OK && !lvl && (forced_slab || !forced)) {
-        const int want[2] = {64, 128};
-        int32_t built = 0, tried = 0;  // rows of the slab built last, of any tried
-        float slab_best = 0.f;
-        int32_t pick_want = 0, pick_rows = 0;
-        gk_status ss = GK_OK;
-        for (int k = 0; k < 3 && ss == GK_OK; ++k) {
-            // the last pass rebuilds the faster size, if it is not the one built
-            if (k == 2 && (!pick_want || pick_rows == built)) break;
-            bool ok = false;
-            int32_t rows = 0;
-            S->release_slab();
-            ss = build_slab<T>(S, n, lv, k < 2 ? want[k] : pick_want, k < 2 ? tried : 0, s, &rows, &ok);
-            if (ss != GK_OK || !ok) {
-                built = 0;
-                continue;
-            }
-            built = tried = rows;
-            if (k == 2) break;
-            IluDev<T> f = tri_view<T>(S, n);
-            f.slab = 1;
-            T* w = (T*)tmp.ptr;
-            const IluSrc<T> src{(const T*)S->rdiag};
-            float ms = 0.f;
-            ss = ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s);
-            if (ss == GK_OK && cudaEventRecord(e0, s) != cudaSuccess) ss = GK_ERR_CUDA;
-            if (ss == GK_OK)
-                ss = ilu_apply<T>(f, src, w, IluOutStore<T>{w + n}, IluSkipNever{}, IluNoErr{}, s);
-            if (ss == GK_OK && (cudaEventRecord(e1, s) != cudaSuccess ||
-                                cudaEventSynchronize(e1) != cudaSuccess ||
-                                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-                ss = GK_ERR_CUDA;
-            if (ss == GK_OK && (!pick_want || ms < slab_best)) {
-                slab_best = ms;
-                pick_want = want[k];
-                pick_rows = rows;
-            }
-        }
-        if (ss == GK_OK && built && pick_want) slab = forced_slab || slab_best < best;
-        if (ss != GK_OK) {
-            cudaGetLastError();  // no room for the records: keep the other mode
-            if (forced_slab) st = ss;
-        }
-        if (!slab) S->release_slab();
-        if (slab && win) {
-            dfree(S->wrec);
-            dfree(S->wperm);
-            S->wrec = S->wperm = nullptr;
-            win = false;
         }
     }
     cudaEventDestroy(e0);
@@ -1085,12 +1159,10 @@ static gk_status tri_build(TriStore* S, gk_dtype vdt, gk_matrix C, bool factoriz
         GK_CUDA(cudaStreamSynchronize(s));
         if (h[3] & 1u) return GK_ERR_INVALID;
         if (h[3] & 2u) return factorize ? GK_ERR_ZERO_DIAG : GK_ERR_INVALID;
-        // chunk levels for both sizes and directions, once
+        // chunk levels for both directions, once (of 8 rows when they are needed)
         IluLevels lv;
         GK_TRY(chunk_levels(S, n, 32, false, lv.l32, &lv.nl32, s));
         GK_TRY(chunk_levels(S, n, 32, true, lv.u32, &lv.nu32, s));
-        GK_TRY(chunk_levels(S, n, 8, false, lv.l8, &lv.nl8, s));
-        GK_TRY(chunk_levels(S, n, 8, true, lv.u8, &lv.nu8, s));
         GK_TRY(chunk_levels(S, n, 1, false, lv.l1, &lv.nl1, s));
         GK_TRY(chunk_levels(S, n, 1, true, lv.u1, &lv.nu1, s));
         if (factorize) {
