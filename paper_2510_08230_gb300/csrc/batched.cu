@@ -617,7 +617,7 @@ struct BatchCfg {
 struct BatchBufs {
     DevBuf desc, outs, work, pad;
     SysDesc* hdesc = nullptr;
-    SysOut* hout = nullptr;
+    SysOut* hout = nullptr;      // hcap outcomes, then hcap indices: the order of the systems
     size_t hcap = 0;
     ~BatchBufs() {
         if (hdesc) cudaFreeHost(hdesc);
@@ -727,8 +727,9 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
         if (B.hout) cudaFreeHost(B.hout);
         B.hdesc = nullptr;
         B.hout = nullptr;
+        B.hcap = 0;
         GK_CUDA(cudaMallocHost(&B.hdesc, sizeof(SysDesc) * (size_t)count));
-        GK_CUDA(cudaMallocHost(&B.hout, sizeof(SysOut) * (size_t)count));
+        GK_CUDA(cudaMallocHost(&B.hout, (sizeof(SysOut) + sizeof(int32_t)) * (size_t)count));
         B.hcap = (size_t)count;
     }
     GK_TRY(B.desc.ensure(sizeof(SysDesc) * (size_t)count));
@@ -738,10 +739,10 @@ static gk_status run_batch(int32_t count, const gk_matrix* As, const void* const
     char* w = (char*)B.work.ptr;
     char* pw = (char*)B.pad.ptr;
     bool any_pad = false;
-    std::vector<int32_t> order((size_t)count);  // the largest system first
+    int32_t* order = (int32_t*)(B.hout + B.hcap);  // the largest system first
     for (int32_t i = 0; i < count; ++i) order[i] = i;
     auto work = [&](int32_t i) { return As[i]->nnz + 8 * (int64_t)As[i]->n; };
-    std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
+    std::sort(order, order + count, [&](int32_t a, int32_t b) {
         return work(a) != work(b) ? work(a) > work(b) : a < b;
     });
     for (int32_t k = 0; k < count; ++k) {
