@@ -73,12 +73,16 @@ def matrix_bytes(m, refined):
 
 
 def ilu_bytes(m, refined):
-    """Device bytes an ILU(0) solve adds to a cached matrix: the factors'
-    pattern, values, diagonal data and claim orders (per value type: twice
-    once a refined solve factors the FP32 copy too) and two more solver
-    vectors."""
-    b = 4 * (m.n + 1) + 12 * m.nnz + 20 * m.n
-    return b * (2 if refined else 1) + 2 * 8 * m.n
+    """Device bytes an ILU(0) solve adds to a cached matrix, at most: the
+    factors' pattern, values, diagonal data and claim orders, the
+    substitutions' records (per row and triangle 48 bytes, its place and the
+    fetched values' places), vectors and bucket starts (at most 8 buckets a
+    row), per value type: twice once a refined solve factors the FP32 copy
+    too; and two more solver vectors."""
+    n = m.n
+    b = 4 * (n + 1) + 12 * m.nnz + 20 * n
+    b += 2 * (48 + 4 + 16) * n + 2 * 8 * n + 2 * 2 * 4 * (8 * n + 1024)
+    return b * (2 if refined else 1) + 2 * 8 * n
 
 
 # preconditioners the batched engine runs (others go to gk_solve alone)
