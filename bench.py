@@ -11,7 +11,9 @@ Section 6).  value = algorithmic bytes of the step / device time (GB/s),
 where every matrix counts its CSR algorithmic bytes = nnz*(value+index
 bytes) + 4*(n+1) + x and y once, whichever format ran.  Every format is also
 timed and listed under "sweep" with its own algorithmic bytes (ELL/SELL-P
-unpadded without the row pointer, COO with a row index per entry).
+unpadded without the row pointer, COO with a row index per entry).  The last
+line on stdout is the result; the same with every section in full goes to
+stderr.
 Matrices (0.9-1.7 GB each) are larger than L2, so no flush is needed.
 Extra keys: CG solves/s on the 64x64 Laplacian, time to 1e-10 on the 128^3
 diffusion problem for FP32-refined vs plain FP64 Jacobi-CG / GMRES(30) /
@@ -769,6 +771,23 @@ def run_reference(args):
     return 0
 
 
+# sections that go to stderr alone: the line on stdout has to stay short enough
+# for readers that keep the end of a program's output
+DETAILS = ("step", "sweep", "cg", "ir_128cubed", "per_iteration_1000", "abi_overhead",
+           "preconditioners", "oracle", "batched_2048", "serving")
+
+
+def headline(line):
+    """The result line without its detail sections, with the figures of the
+    metric that they hold: CG solves/s and the serving latencies."""
+    out = {k: v for k, v in line.items() if k not in DETAILS}
+    for section, keys in (("cg", ("solves_per_s",)),
+                          ("serving", ("solves_per_s", "p50_ms", "p99_ms"))):
+        if line.get(section):
+            out[section] = {k: line[section][k] for k in keys if k in line[section]}
+    return out
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -978,7 +997,8 @@ def main():
             "serving": serving, "clocks": clk,
             "gpu_launches": launches}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)  # every section in full
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
