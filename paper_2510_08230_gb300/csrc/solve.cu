@@ -389,6 +389,7 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
     constexpr double GROWTH = 4.0;
     constexpr int STAG_STEPS = 3;
     bool finish64 = false;
+    bool grid = o->engine == 0;
     double best_tn = INFINITY;
     std::vector<double> best_hist;  // best_tn before each outer step
     int k = 0;
@@ -436,10 +437,11 @@ static gk_status solve_ir(gk_matrix A, const double* b, double* x, const gk_solv
         const int32_t left = o->max_iters - total_inner;
         auto inner_solve = [&](auto vt) -> gk_status {
             using V = decltype(vt);
-            if (o->engine == 0 && grid_admits(L, o->method, pk)) {
+            if (grid && grid_admits(L, o->method, pk)) {
                 const gk_status g = solve_grid<V, float>(L, r32, d32, o->method, pk, inner_tol,
                                                          left, m, s, &io, true);
                 if (g != GK_ERR_UNSUPPORTED) return g;
+                grid = false;  // a wait that ran out need not do so in every inner solve
             }
             return solve_mk<V, float>(L, r32, d32, o->method, pk, bsz, inner_tol, left, m, s, &io,
                                       true);
