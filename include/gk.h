@@ -323,7 +323,8 @@ gk_status gk_solve(gk_matrix A, const void* b, void* x,
                    const gk_solve_opts* opts, gk_solve_info* info,
                    void* stream);
 
-/* The same solve as gk_solve, enqueued on `stream` without waiting for it:
+/* gk_solve's solve on the multi-kernel engine (the bits of engine = 1, not
+ * of the kernels that gk_solve may pick), enqueued on `stream` without waiting:
  * the call returns once the work is enqueued and the outcome arrives in
  * `info`, a DEVICE pointer to one gk_solve_info the caller owns, when the
  * solve's work on the stream completes (device_ms is 0; read info after
@@ -352,8 +353,8 @@ gk_status gk_solve_async(gk_matrix A, const void* b, void* x,
  * row in CSR order, so the layout never changes a result.  The layout
  * policy (CSR, ELL, SELL-P with S = 8, 16 or 32) and, when no system has more
  * than 1024 rows, the block size (256 or 512 threads; else 512) are autotuned
- * per batch shape on the first call for that shape (value type, method, preconditioner, log2 of the largest n and
- * of the count): each candidate runs the batch capped at 30 iterations from
+ * per batch shape on the first call for that shape (value type, method,
+ * preconditioner, log2 of the largest n and of the count): each candidate runs the batch capped at 30 iterations from
  * the callers' initial guesses, which are restored afterwards; the choice
  * is cached for the process and reported per system in infos (spmv_format,
  * slice_size, block_threads).  Batches of fewer than 64 systems, or with

@@ -9,10 +9,13 @@
 // stencil 22.3 / 12.3 (2.6), 10^6-row 3D stencil 59.9 / 38.6 (22), 128^3
 // diffusion 98 / 71 (47), in FP32 56 / 32; 121 entries a row, n = 30,000:
 // 75.6 / 24.5, n = 500,000: 316 / 155.  Six solves at once, 600 iterations
-// each: 17K to 25K rows 25.5 / 12.1 ms, 70K to 430K rows 47 / 48 ms (alone,
-// in turn: 74 / 30 and 105 / 60).  What is left on small matrices is latency: the block's FP64 tree (~2,300 cycles a
-// reduction), the hand-offs (~1,700 to 2,600 each) and FP64 divisions; on
-// large ones the FP64 pipe (128^3: 97,000 of 153,000 cycles).
+// each, in ms: 17K to 25K rows 25.5 / 12.1 (alone, in turn: 74 / 30), 70K to
+// 430K rows in FP64 38 / 43 to 52 (97 / 58), in FP32 24.6 / 24 to 31 (79 / 40):
+// there two grids fill the GPU and the others queue, which the multi-kernel
+// engine's kernels do not.  What is left on small matrices is latency: the
+// block's FP64 tree (~2,300 cycles a reduction), the hand-offs (~1,700 to 2,600
+// each) and FP64 divisions; on large ones the FP64 pipe (128^3: 97,000 of
+// 153,000 cycles).
 //
 // Block k owns rows [kR, (k+1)R).  The vectors only their owner reads
 // (r, q, and x and the inverse diagonal when they fit) stay in its shared

@@ -31,7 +31,8 @@
 // slab's own rows need stay in a ring of the last WIN_MAXD + 1 levels.
 // Two threads bulk-copy records and level-ordered inputs up to nb levels
 // ahead, and one warp waits for copies and fetched values on the computing
-// warps' behalf and joins their barrier, so that they test nothing.  Every row's subtractions keep the substitution order: the result is bit-identical
+// warps' behalf and joins their barrier, so that they test nothing.  Every
+// row's subtractions keep the substitution order: the result is bit-identical
 // to the other modes.
 //
 // No wait can be circular: a slab only waits on slabs of rows before it (U:
