@@ -197,7 +197,8 @@ struct SolverCache;  // solve.cu
 // matrix decide (rows, start, estart, range, perm, hand), one what the buckets
 // decide (records and epos).
 struct SlabStore {
-    int32_t nslab = 0, rows_each = 0;
+    int32_t nslab = 0;
+    int64_t crossing = 0;           // terms whose value comes from another slab
     int32_t nlev[2] = {0, 0}, cap[2] = {0, 0}, ecap[2] = {0, 0}, nb[2] = {0, 0}, terms[2] = {0, 0};
     int32_t* rows[2] = {nullptr, nullptr};
     int32_t* start[2] = {nullptr, nullptr};

@@ -664,7 +664,6 @@ static gk_status build_slab(const TriStore* S, int32_t n, const IluLevels& lv, c
     const int32_t nslab = (int32_t)(((int64_t)n + R - 1) / R);
     if ((int64_t)nslab * std::max(nlev[0], nlev[1]) > 8 * (int64_t)n + 1024) return GK_OK;
     B->nslab = nslab;
-    B->rows_each = R;
     const unsigned g = ew_grid(n);
     constexpr int AL = (int)(16 / sizeof(T));
     const size_t nk[2] = {(size_t)nslab * nlev[0], (size_t)nslab * nlev[1]};
@@ -757,6 +756,7 @@ static gk_status build_slab(const TriStore* S, int32_t n, const IluLevels& lv, c
         GK_CUDA(cudaGetLastError());
     }
     GK_CUDA(cudaStreamSynchronize(s));  // the scratch goes
+    B->crossing = (int64_t)w[4] + w[5];
     *ok = true;
     return GK_OK;
 }
@@ -851,23 +851,31 @@ IluDev<T> ilu_view(gk_matrix A) {
 template IluDev<double> ilu_view<double>(gk_matrix);
 template IluDev<float> ilu_view<float>(gk_matrix);
 
-// Where a matrix qualifies for the slab mode it is the fastest: on 22 stencil
-// matrices of 216 to 2,097,152 rows, in FP64 and FP32, an application took 0.23
-// to 0.96 of the next best mode's time (at 33 rows 86 us against 60, at 64 62
-// against 65: below SLAB_MIN_N rows it is not tried).  So nothing else is built
-// or timed for such a matrix.  The first application to a new one, FP64, ms,
-// with the trials of the other modes / without / before there was a slab mode:
-// 2D 64^2 9.1 / 4.1 / 8.1, 20^3 15.6 / 3.8 / 14.5, 2D 300 x 200 310 / 93 /
-// 306, 128^3 640 / 500 / 640.
+// Where a matrix qualifies for the slab mode it is the fastest, unless nearly
+// all its dependencies cross slabs: on 22 stencil matrices of 216 to 2,097,152
+// rows, in FP64 and FP32, an application took 0.23 to 0.96 of the next best
+// mode's time (at 33 rows 86 us against 60, at 64 62 against 65: below
+// SLAB_MIN_N rows it is not tried).  So for such a matrix nothing else is built
+// or timed.  The first application to a new one, FP64, ms, with the trials of
+// the other modes / without / before there was a slab mode: 2D 64^2 9.1 / 4.1 /
+// 8.1, 20^3 15.6 / 3.8 / 14.5, 2D 300 x 200 310 / 93 / 306, 128^3 640 / 520 /
+// 640.  Where more than SLAB_CROSS of the dependencies cross (20^3: 0.4), every
+// level waits for another slab, which costs more than a level of the window
+// mode: 60,000 rows in 5,000 interleaved chains 108 us against 72, red-black
+// orderings the same as the others to 10 %.  There all modes are timed.
 constexpr int32_t SLAB_MIN_N = 128;
+constexpr double SLAB_CROSS = 0.75;
 
-// The slab mode's data where the matrix qualifies (*picked), in S->sl: the
-// faster of two slab sizes.  64 slabs are better where levels are narrow (2D
-// 1024^2), 128 where the FP64 pipe bounds a level (128^3 FP64).  w: 2 n values.
+// The slab mode's data where the matrix qualifies (*ms > 0, an application's
+// time), in S->sl: the faster of two slab sizes.  64 slabs are better where
+// levels are narrow (2D 1024^2), 128 where the FP64 pipe bounds a level (128^3
+// FP64).  *sure: no other mode need be timed.  w: 2 n values.
 template <typename T>
-static gk_status pick_slab(TriStore* S, int32_t n, const IluLevels& lv, T* w, cudaEvent_t e0,
-                           cudaEvent_t e1, cudaStream_t s, bool* picked) {
-    *picked = false;
+static gk_status pick_slab(TriStore* S, int32_t n, int64_t nnz, const IluLevels& lv, T* w,
+                           cudaEvent_t e0, cudaEvent_t e1, cudaStream_t s, float* out_ms,
+                           bool* sure) {
+    *out_ms = 0.f;
+    *sure = false;
     SlabShape h;
     GK_TRY(slab_shape(S, n, lv, s, &h));
     if (!h.fits) return GK_OK;
@@ -901,7 +909,8 @@ static gk_status pick_slab(TriStore* S, int32_t n, const IluLevels& lv, T* w, cu
     }
     if (!best.b.nslab) return GK_OK;
     std::swap(S->sl, best.b);
-    *picked = true;
+    *out_ms = std::max(best_ms, 1e-6f);
+    *sure = (double)S->sl.crossing <= SLAB_CROSS * (double)(nnz - n);
     return GK_OK;
 }
 
@@ -922,7 +931,7 @@ static gk_status pick_slab(TriStore* S, int32_t n, const IluLevels& lv, T* w, cu
 // cluster kernel) forces a shape.  Results never depend on the choice,
 // only the time does.
 template <typename T>
-static gk_status tune_chunks(TriStore* S, int32_t n, IluLevels& lv, cudaStream_t s) {
+static gk_status tune_chunks(TriStore* S, int32_t n, int64_t nnz, IluLevels& lv, cudaStream_t s) {
     int forced = 0;
     bool forced_lvl = false, forced_win = false, forced_slab = false;
     if (const char* e = getenv("GK_ILU_CHUNK")) {
@@ -947,14 +956,18 @@ static gk_status tune_chunks(TriStore* S, int32_t n, IluLevels& lv, cudaStream_t
     gk_status st = GK_OK;
     float best = 0.f;
     int pick = 0;
+    float slab_ms = 0.f;
     bool slab = false;
     if (forced_slab || (!forced && n > SLAB_MIN_N)) {
-        const gk_status ss = pick_slab<T>(S, n, lv, (T*)tmp.ptr, e0, e1, s, &slab);
+        const gk_status ss =
+            pick_slab<T>(S, n, nnz, lv, (T*)tmp.ptr, e0, e1, s, &slab_ms, &slab);
         if (ss != GK_OK) {
             cudaGetLastError();  // no room for the records: the other modes
+            slab_ms = 0.f;
             slab = false;
             if (forced_slab) st = ss;
         }
+        if (forced_slab) slab = slab_ms > 0.f;
     }
     // the chunk state is valid whatever mode runs
     const int ncand = forced || slab ? 1 : rows_ok ? 4 : 3;
@@ -1043,8 +1056,8 @@ static gk_status tune_chunks(TriStore* S, int32_t n, IluLevels& lv, cudaStream_t
             lvl = forced_lvl || ms < best;
         }
     }
-    // the window mode (stencil-like matrices too wide for the slab mode, see
-    // k_ilu_trsv_win): timed against the chunks when the matrix qualifies
+    // the window mode (stencil-like matrices, see k_ilu_trsv_win): timed against
+    // the chunks when the matrix qualifies
     bool win = false;
     if (st == GK_OK && !lvl && !slab && (forced_win || !forced)) {
         bool ok = false;
@@ -1070,12 +1083,22 @@ static gk_status tune_chunks(TriStore* S, int32_t n, IluLevels& lv, cudaStream_t
             if (forced_win) st = ws;
         } else if (ok) {
             win = forced_win || ms < best;
+            if (win) best = ms;
         }
         if (!win) {  // not picked: its records go
             dfree(S->wrec);
             dfree(S->wperm);
             S->wrec = S->wperm = nullptr;
         }
+    }
+    if (!slab && !forced && slab_ms > 0.f) slab = slab_ms < best;
+    if (!slab) {
+        S->sl.release();
+    } else if (win) {
+        win = false;
+        dfree(S->wrec);
+        dfree(S->wperm);
+        S->wrec = S->wperm = nullptr;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1193,7 +1216,8 @@ static gk_status tri_build(TriStore* S, gk_dtype vdt, gk_matrix C, bool factoriz
         GK_CUDA(cudaMemcpyAsync(h, mp, sizeof(h), cudaMemcpyDeviceToHost, s));
         GK_CUDA(cudaStreamSynchronize(s));
         S->zero_diag = h[2] != 0;
-        GK_TRY(vdt == GK_F64 ? tune_chunks<double>(S, n, lv, s) : tune_chunks<float>(S, n, lv, s));
+        GK_TRY(vdt == GK_F64 ? tune_chunks<double>(S, n, nnz, lv, s)
+                              : tune_chunks<float>(S, n, nnz, lv, s));
     }
     GK_CUDA(cudaStreamSynchronize(s));
     return GK_OK;

@@ -48,11 +48,52 @@ def test_first_application_times_slabs_alone(monkeypatch):
     assert min(auto) <= 1.5 * min(forced), (auto, forced)
 
 
-@pytest.mark.parametrize("case", ["lap1d_128", "lap1d_129", "lap2d_8x16", "lap2d_43x3", "banded_130",
+def _chains(n, k):
+    """k interleaved chains: row i depends on row i - k alone."""
+    i = np.arange(n)
+    table = np.stack([i - k, i, i + k], 1)
+    keep = (table >= 0) & (table < n)
+    rp = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int32)
+    vals = np.tile([-1.0, 4.0, -1.0], (n, 1))[keep]
+    return W.CSR(n, n, rp, table[keep].astype(np.int32), vals)
+
+
+def test_dependencies_that_all_cross_slabs(monkeypatch):
+    """Every row's one dependency lies in another slab, so each level waits for
+    one: the window mode is faster, and is what the automatic choice runs."""
+    import torch
+    m = _chains(60000, 5000)
+    r = W.uniform_vector(m.n, 3)
+    rt = torch.from_numpy(r).to(torch_dev())
+    zt = torch.zeros_like(rt)
+    want = oracle.ilu0_apply(m, oracle.ilu0(m), r)
+    took = {}
+    for mode in ("win", "slab", "auto"):
+        if mode == "auto":
+            monkeypatch.delenv("GK_ILU_CHUNK")
+        else:
+            monkeypatch.setenv("GK_ILU_CHUNK", mode)
+        A = gk.Matrix.from_csr(m, "f64")
+        times = []
+        for _ in range(8):
+            A.precond_apply(rt, zt, "ilu")
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for _ in range(20):
+                A.precond_apply(rt, zt, "ilu")
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+        took[mode] = min(times)
+        assert np.array_equal(zt.cpu().numpy(), want), mode
+        A.close()
+    assert took["auto"] <= 1.2 * min(took["win"], took["slab"]), took
+
+
+@pytest.mark.parametrize("case", ["chains", "lap1d_128", "lap1d_129", "lap2d_8x16", "lap2d_43x3", "banded_130",
                                   "wide_levels"])
 def test_automatic_mode_bit_exact(case):
     import torch
-    m = {"lap1d_128": lambda: W.laplacian_1d(128), "lap1d_129": lambda: W.laplacian_1d(129),
+    m = {"chains": lambda: _chains(3001, 400), "lap1d_128": lambda: W.laplacian_1d(128), "lap1d_129": lambda: W.laplacian_1d(129),
          "lap2d_8x16": lambda: W.laplacian_2d(8, 16), "lap2d_43x3": lambda: W.laplacian_2d(43, 3),
          "banded_130": lambda: W.banded_spd(130, 5, 3),
          "wide_levels": lambda: W.laplacian_3d(60, 60, 60)}[case]()
