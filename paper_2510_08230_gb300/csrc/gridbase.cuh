@@ -70,8 +70,8 @@ constexpr int64_t GRID_GM_HALF_ROWS = 4096, GRID_GM_HALF_ENTRIES = 131072;
 // 8.5 ms with 8.0 / 7.4 / 7.4 us.
 constexpr int64_t GRID_MIN_ROW_BYTES = 2048;
 
-// Budgets below this have the clock read at every poll.
-constexpr uint64_t GRID_SHORT_BUDGET_NS = 10000000;
+// GridTeam::between for a budget: below 10 ms the clock is read at every poll.
+inline unsigned grid_polls_between(uint64_t wait_ns) { return wait_ns < 10000000 ? 0u : 255u; }
 
 // why a solve ends (0: it goes on); PASSED, CYCLE: a recurrence residual
 // passed, a GMRES cycle ended
@@ -121,6 +121,7 @@ struct GridTeam {
     unsigned long long* arrived;  // blocks that have published, all rounds
     int32_t* err;
     uint64_t wait_ns;
+    unsigned between;  // polls between looks at the clock, less 1: 255 or 0
     int nb, nc;
     bool upper;     // threads of the upper half hold values
     double* red;    // shared: GRID_RED<NT> bytes
@@ -141,11 +142,13 @@ struct GridTeam {
     // cycles), or with a budget that this would overrun at every poll.
     template <class F>
     __device__ __forceinline__ bool wait(F&& ready) const {
-        const unsigned between = wait_ns < GRID_SHORT_BUDGET_NS ? 0u : 255u;
         uint64_t t0 = 0;
-        for (unsigned spin = 0;; ++spin) {
+        // counts in steps of 1, or 256, so that the test is against a constant
+        // (a mask of the budget's: 117,000-row CG 3.16 ms, so 2.94; 128^3 42.6
+        // and 42.5)
+        for (unsigned spin = 255u - between;; spin += 256u - between) {
             if (__all_sync(0xffffffffu, ready())) return true;
-            if ((spin & between) != between) continue;
+            if ((spin & 255u) != 255u) continue;
             bool stop = false;
             if ((threadIdx.x & 31) == 0) {
                 const uint64_t t = globaltimer_ns();
@@ -446,13 +449,24 @@ gk_status grid_launch(K kern, A& args, const GridPlan& P, size_t smem, cudaStrea
     return GK_OK;
 }
 
-// Runs launch() when the GPU has seats for its grid, reads the outcome and
-// copies the solution from `from` to x (bytes).  The stream is drained first
-// and before the seats are given back: they are held for the solve alone.
+// x = from when the solve ended by itself: a wait that ran out leaves x alone.
+template <typename T>
+static __global__ void __launch_bounds__(256)
+k_grid_take(int32_t n, const int32_t* __restrict__ err, const GridOut* __restrict__ o,
+            const T* __restrict__ from, T* __restrict__ x) {
+    if (*err != 0 || o->status == GK_ERR_TIMEOUT) return;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        x[i] = from[i];
+}
+
+// Runs launch() when the GPU has seats for its grid, copies the solution from
+// `from` to x and reads the outcome.  The stream is drained first and before
+// the seats are given back: they are held for the solve alone.
 // GK_ERR_UNSUPPORTED: a wait ran out; x is as it was.
-template <class F>
-gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* out, void* x,
-                   const void* from, size_t bytes, F&& launch) {
+template <typename T, class F>
+gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* out, int32_t n,
+                   const T* from, T* x, F&& launch) {
     struct Outcome {
         int32_t err, pad[15];
         GridOut o;
@@ -464,11 +478,13 @@ gk_status grid_run(SolverCache* C, const GridPlan& P, cudaStream_t s, SolveOut* 
         GridSeats seats(P.half, P.nb);
         out->queued_ms += seats.waited_ms;
         GK_TRY(launch());
+        k_grid_take<T><<<(unsigned)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)num_sms() * 8),
+                         256, 0, s>>>(n, P.err(), P.out(), from, x);
+        GK_CUDA(cudaGetLastError());
         GK_CUDA(cudaMemcpyAsync(h, P.err(), sizeof(Outcome), cudaMemcpyDeviceToHost, s));
         GK_CUDA(cudaStreamSynchronize(s));
     }
     if (h->err != 0 || h->o.status == GK_ERR_TIMEOUT) return GK_ERR_UNSUPPORTED;
-    GK_CUDA(cudaMemcpyAsync(x, from, bytes, cudaMemcpyDeviceToDevice, s));
     out->threads = P.half ? GRID_HALF : GRID_FULL;
     out->status = (gk_status)h->o.status;
     out->iters = h->o.iters;

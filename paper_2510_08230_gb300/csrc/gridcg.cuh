@@ -46,6 +46,7 @@ struct GridCgArgs {
     double tol;
     int32_t max_iters, inner, stall;
     uint64_t wait_ns;
+    unsigned between;  // see GridTeam
 };
 
 // Shared-memory modes: what a block keeps there beside r and q.
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(NT, GRID_FULL / NT) k_grid_cg(const GridCgArgs
     const int tid = threadIdx.x;
     const int32_t r0 = (int32_t)blockIdx.x * R;
     const int32_t nloc = min(R, A.n - r0);  // >= 1
-    GridTeam<NT> team{A.slots, A.arrived, A.err, A.wait_ns, (int)gridDim.x, 0, nloc > NT / 2,
+    GridTeam<NT> team{A.slots, A.arrived, A.err, A.wait_ns, A.between, (int)gridDim.x, 0, nloc > NT / 2,
                   reinterpret_cast<double*>(smem), part, &s_code, 0u};
     const GridRows<NT, V, T, MODE == 0> rows{R, A.K, r0, nloc, A.stride, A.col, A.val, s_val,
                                              reinterpret_cast<int32_t*>(s_val + (size_t)(MODE == 0 ? R * A.K : 0))};
@@ -289,6 +290,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     a.inner = inner ? 1 : 0;
     a.stall = inner ? 200 : 0;
     a.wait_ns = M->wait_ns;
+    a.between = grid_polls_between(a.wait_ns);
     auto go = [&](auto nt, auto md) -> gk_status {
         constexpr int NT = decltype(nt)::value, MD = decltype(md)::value;
         const size_t smem = grid_cg_smem<NT, V, T>(MD, P.R, M->K);
@@ -300,7 +302,7 @@ gk_status solve_grid_cg(gk_matrix M, const T* b, T* x, int pkind, double tol, in
     constexpr std::integral_constant<int, 0> m0;
     constexpr std::integral_constant<int, 1> m1;
     constexpr std::integral_constant<int, 2> m2;
-    return grid_run(C, P, s, out, x, a.x, sizeof(T) * (size_t)n, [&]() -> gk_status {
+    return grid_run(C, P, s, out, n, a.x, x, [&]() -> gk_status {
         return P.half      ? (mode == 0 ? go(half, m0) : go(half, m1))
                : mode == 0 ? go(full, m0)
                : mode == 1 ? go(full, m1)

@@ -60,6 +60,7 @@ struct GridGmArgs {
     int32_t max_iters;
     double stag;    // > 0: stop when a cycle's residual exceeds stag x the previous
     uint64_t wait_ns;
+    unsigned between;  // see GridTeam
 };
 
 // Shared memory: the scalar sums, each warp's column sums, h1, h2, the triangular
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(NT, GRID_FULL / NT) k_grid_gmres(const GridGmA
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t r0 = (int32_t)blockIdx.x * R;
     const int32_t nloc = min(R, A.n - r0);  // >= 1
-    GridTeam<NT> team{A.slots, A.arrived, A.err, A.wait_ns, (int)gridDim.x, nc, nloc > NT / 2,
+    GridTeam<NT> team{A.slots, A.arrived, A.err, A.wait_ns, A.between, (int)gridDim.x, nc, nloc > NT / 2,
                   reinterpret_cast<double*>(smem), part, &s_code, 0u};
     const GridRows<NT, V, T, STAGED> rows{R, A.K, r0, nloc, A.stride, A.col, A.val, s_val,
                                           reinterpret_cast<int32_t*>(s_val + (size_t)(STAGED ? R * A.K : 0))};
@@ -524,6 +525,7 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     a.max_iters = max_iters;
     a.stag = inner ? 0.95 : 0.0;
     a.wait_ns = M->wait_ns;
+    a.between = grid_polls_between(a.wait_ns);
     auto go = [&](auto nt, auto st) -> gk_status {
         constexpr int NT = decltype(nt)::value;
         constexpr bool ST = decltype(st)::value;
@@ -533,7 +535,7 @@ gk_status solve_grid_gmres(gk_matrix M, const T* b, T* x, int pkind, double tol,
     auto go_staged = [&](auto nt) -> gk_status {
         return staged ? go(nt, std::true_type{}) : go(nt, std::false_type{});
     };
-    return grid_run(C, P, s, out, x, a.x, sizeof(T) * (size_t)n, [&]() -> gk_status {
+    return grid_run(C, P, s, out, n, a.x, x, [&]() -> gk_status {
         return P.half ? go_staged(std::integral_constant<int, GRID_HALF>{})
                       : go_staged(std::integral_constant<int, GRID_FULL>{});
     });
