@@ -5,10 +5,10 @@
 // the grid reduction's tail (fence, ticket, the last block's pass over the
 // partials, the next launch) while the other SMs idle.  Per Jacobi-CG
 // iteration, multi-kernel against this kernel (GB300, us; the FP64 pipe's
-// own floor in brackets): 17,030-row 2D stencil 20.0 / 8.2, 117,453-row 3D
-// stencil 22.3 / 12.3 (2.6), 10^6-row 3D stencil 59.9 / 38.6 (22), 128^3
-// diffusion 98 / 71 (47), in FP32 56 / 32; 121 entries a row, n = 30,000:
-// 75.6 / 24.5, n = 500,000: 316 / 155.  Six solves at once, 600 iterations
+// own floor in brackets): 17,030-row 2D stencil 20.0 / 7.9, 117,453-row 3D
+// stencil 22.3 / 11.4 (2.6), 10^6-row 3D stencil 59.9 / 37.7 (22), 128^3
+// diffusion 98 / 69.5 (47), in FP32 56 / 30; 121 entries a row, n = 30,000:
+// 75.6 / 24.3, n = 500,000: 316 / 175.  Six solves at once, 600 iterations
 // each, in ms: 17K to 25K rows 25.5 / 12.1 (alone, in turn: 74 / 30), 70K to
 // 430K rows in FP64 38 / 43 to 52 (97 / 58), in FP32 24.6 / 24 to 31 (79 / 40):
 // there two grids fill the GPU and the others queue, which the multi-kernel
